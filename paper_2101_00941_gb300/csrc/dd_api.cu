@@ -172,6 +172,8 @@ struct RangeKernel {
   int nstage = 0;
   int row_slot = 0;
   int zcap = 0;
+  int tab_pitch = 0;
+  int flush = 0;
   size_t smem = 0;
   uint8_t* d_tabs = nullptr;  // device copy of the delay-class tables
   int64_t lsu_wavefronts = 0; // shared-memory work of one row of time tiles (TiledPlan)
@@ -309,6 +311,8 @@ int plan_tiled_shape(const int32_t* tab, int ntr, int cpad, int d, int tt, int t
   r.nstage = tp.nstage;
   r.row_slot = tp.row_slot;
   r.zcap = tp.zcap;
+  r.tab_pitch = tp.tab_pitch;
+  r.flush = tp.flush;
   r.smem = tp.smem;
   r.lsu_wavefronts = tp.lsu_wavefronts;
   r.copy_bytes = tp.copy_bytes;
@@ -496,6 +500,8 @@ int plan_autotune(dd_plan_s* p) {
       A.cpad = p->Cp;
       A.row_slot = k.row_slot;
       A.zcap = k.zcap;
+      A.tab_pitch = k.tab_pitch;
+      A.flush = k.flush;
       A.nstage = k.nstage;
       A.tabs = k.d_tabs;
       A.err = reinterpret_cast<int32_t*>(s.d_count + 1);
@@ -918,7 +924,7 @@ int dd_fuse_search(dd_plan_t p, const int32_t* widths, int32_t nwidths, uint32_t
     const int hp = (int)round_up(wd[nw - 1], 32);
     int32_t e_off = 0;
     size_t fsmem = 0;
-    if (!ddk::fused_smem(d > 1, K.row_slot, K.zcap, K.nstage, hp, &e_off, &fsmem)) {
+    if (!ddk::fused_smem(d > 1, K.row_slot, K.zcap, K.tab_pitch, K.nstage, hp, &e_off, &fsmem)) {
       if (replanned[r]) {  // keep the range as it was planned
         cudaFree(K.d_tabs);
         K = p->rk[r];
@@ -1097,6 +1103,8 @@ static int run_impl(dd_plan_t p, const uint8_t* chunk, int64_t nsamp, void* cuda
       A.cpad = p->Cp;
       A.row_slot = K.row_slot;
       A.zcap = K.zcap;
+      A.tab_pitch = K.tab_pitch;
+      A.flush = K.flush;
       A.nstage = K.nstage;
       A.tabs = K.d_tabs;
       A.err = p->err_word ? p->err_word : reinterpret_cast<int32_t*>(s.d_count + 1);

@@ -15,29 +15,37 @@
 //     (exact in 16-bit lanes: two groups' sums stay below 2^16 for d <= 16). The even and odd
 //     pair words are kept in two planes, so a lane that owns outputs 2m and 2m+1 of a trial
 //     reads one word, and consecutive lanes read consecutive words. The classes depend on the
-//     delay table only, so the plan computes them once (tiled_plan, below) as one fixed-size
-//     table per (trial tile, stage), together with a balanced split of the stage's word building
-//     over the warps; the kernel never searches for them.
+//     delay table only, so the plan computes them once (tiled_plan, below) as one table per
+//     (trial tile, stage), together with a balanced split of the stage's word building over the
+//     warps; the kernel never searches for them.
+//   * Class chains. Sorted by their delay sums, a group's classes differ from their neighbours
+//     by about one channel moved by one sample (about 7 classes and 7 such steps per group on
+//     the 4096-channel plan). A warp therefore sums all eight channels for the first class of
+//     its share only and reaches each further class by the steps x[r + 1] - x[r] of the moved
+//     channels, in the same packed 16-bit lanes (exact: the arithmetic is modulo 2^32 and each
+//     class's own sums fit their lanes).
 //   * TMA brings each stage's 16 channel rows (one 3-D tensor copy: every row from the same
 //     128-byte segment on, so each lands contiguous) and its class table into shared memory
 //     NS - 1 stages ahead (NS = 4 staging buffers, or 3 where 4 do not fit shared memory);
 //     completion is tracked by mbarriers with bounded waits.
-//   * The main loop adds, per (trial, output pair), the two groups' pair words with one IADD
-//     and splits the sum over the two outputs with two DP2As: one 32-bit shared-memory load per
-//     sixteen channel-adds, for uint8 and uint16 (decimated) data alike.
+//   * The main loop adds, per (trial, output pair), the two groups' pair words to a packed
+//     accumulator with one three-input add: one 32-bit shared-memory load per sixteen
+//     channel-adds, for uint8 and uint16 (decimated) data alike. Every TiledArgs::flush stages,
+//     before a 16-bit lane can overflow, two DP2As add the packed sums to the 32-bit outputs.
 //
 // Software pipeline, one __syncthreads per stage s:
 //     TMA for stage s+NS-1 | build the words of stage s+1 | accumulate stage s
 // Words are built from 32-bit loads and funnel shifts; the eight-channel sums are formed in SWAR
-// lanes (bytes split into 16-bit lanes for uint8 data). Where each class's channel rows start in
-// a stage buffer (row word and funnel shift) depends on where the stage's copy starts, so the
-// CTA works it out once per stage, one (class, channel) per thread, two stages ahead. Exact
+// lanes (bytes split into 16-bit lanes for uint8 data). Where a class's rows start in a stage
+// buffer is known at plan time up to the copy's phase within its first segment, one value per
+// stage and tile, which the build adds to the plan's offsets. Exact
 // moments (S1, 128-bit S2) of every series are added in the epilogue with integer atomics, so
 // the search needs no second statistics pass.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 
@@ -49,14 +57,17 @@ namespace {
 
 constexpr int kMaxTileTrials = 64;         // trials per tile: 64 or 32
 constexpr int kThreads = 512;               // threads of the 16-warp shapes
-constexpr int kWarps = kThreads / 32;       // work lists of a stage's build (one per warp, or
-                                            // shared by two warps in 32-warp CTAs)
+constexpr int kWarps = kThreads / 32;
+constexpr int kMaxWarps = 32;
 constexpr int kG = 8;                       // channels per group (one delay class)
 constexpr int kNG = 2;                      // groups per stage
 constexpr int kRows = kG * kNG;             // channel rows per stage
 constexpr int kMaxNStage = 4;               // staging buffers (rows + class table), at most
 constexpr int kMaxCls = 16;                 // classes per group
-constexpr int kMaxWork = 8;                 // build ranges per warp and stage
+constexpr int kMaxSteps = 3;                // channel steps between chained classes
+constexpr int kMaxLinks = 2 * kMaxCls;      // chain links (classes and in-between steps) per group
+constexpr int kMaxTasks = 112;              // build tasks per stage
+constexpr int kBlock = 31;                  // build units stored per 32-lane block
 constexpr int kSegBytes = 128;              // inner extent of a staged-row copy (tensor map)
 constexpr size_t kSmemLimit = 220 * 1024;   // dynamic shared memory a CTA may plan for
 constexpr size_t kSmemLimit2 = 110 * 1024;  // ... when two CTAs share an SM
@@ -66,57 +77,56 @@ __host__ __device__ constexpr int tile_ctas(int D, int TT, int NT) {
   return (NT == 1024 || (D == 64 && TT == 512)) ? 1 : 2;
 }
 
-// One delay class: its channels' first staged sample relative to the tile's first trial
-// (rel), and its pair words in the stage's word region.
-struct ClsEntry {
-  int16_t rel[kG];
-  int16_t zoff;  // first word (multiple of 4)
-  int16_t zlen;  // words (multiple of 4)
-  int32_t pad;
-};
-
-// Entry of trial t of a tile in GroupTab::zstart for a CTA of W warps with tpw trials per warp:
+// Entry of trial t of a tile in StageTab::zstart for a CTA of W warps with tpw trials per warp:
 // warp t mod W reads its trials t, t + W, ... as tpw consecutive entries.
 __host__ __device__ constexpr int trial_slot(int t, int W, int tpw) { return (t % W) * tpw + t / W; }
 
-struct GroupTab {
-  int16_t zstart[kMaxTileTrials];  // stage word offset of each trial's sequence (0: no trial),
-                                   // warp-major: entry trial_slot(t) (a warp's trials contiguous)
-  ClsEntry cls[kMaxCls];
-  int32_t ncls, pad0, pad1, pad2;
+// One link of a group's chain: a delay class, or a step between two classes that are several
+// channel steps apart (un = 0: it stores nothing). A group's classes share a frame of pair words:
+// frame word v of a class is the sum that a trial of smallest delay b in the class uses for
+// output v - (b - F), F being the group's smallest delay. A unit is 4 (uint8) or 2 (uint16)
+// consecutive frame words; the class stores units ulo .. ulo + un - 1. Row offsets are 8 x a byte
+// offset within the stage buffer for frame word 0, before the copy's phase is added: the low five
+// bits of 8 x (offset + phase) are the funnel shift, the rest the row word. step: the channel
+// step that leads here from the preceding link, the row offset of x[r] of x[r + 1] - x[r] with
+// the step's sign in the top two bits (01: add, 11: subtract); 0 for the first link of a chain.
+struct ClsLink {
+  uint32_t off[kG];
+  uint32_t step;
+  int32_t ev, od;  // byte offset of frame word 0's place in the even plane, word 1's in the odd
+  uint32_t range;  // ulo | un << 16
+  __host__ __device__ uint32_t ulo() const { return range & 0xFFFFu; }
+  __host__ __device__ uint32_t un() const { return range >> 16; }
 };
+static_assert(sizeof(ClsLink) == 48, "read as three 16-byte words");
+constexpr uint32_t kStepOff = 0x000FFFFFu, kStepAdd = 0x40000000u, kStepSub = 0xC0000000u;
 
-// The stage's pair-word build, cut at plan time into blocks of 32 units (one per lane) and
-// dealt to the warps in near-equal contiguous shares. A share is a few ranges, each within one
-// class: group << 4 | class, first block << 8, blocks << 16.
+// Head of a stage's table, followed by its links (group 0's, then group 1's).
+// A build task is one block of 31 units of a run of chained links of one group:
+// first link | (links - 1) << 6 | block << 10; warp w runs the tasks of wtask[w].
 struct StageTab {
-  GroupTab g[kNG];
-  uint32_t work[kWarps][kMaxWork];
-  uint8_t nwork[kWarps];
+  int16_t zstart[kNG][kMaxTileTrials];  // stage word offset of each trial's sequence (0: no
+                                        // trial), entry trial_slot(t)
+  uint16_t task[kMaxTasks];
+  uint16_t wtask[kMaxWarps];            // first task | tasks << 8
+  uint8_t nlink[kNG];
+  uint8_t pad[6];
   int32_t xmin;  // smallest delay of the stage's rows for the tile's first trial
-  int32_t pad[3];
+  int32_t pad1;
 };
 static_assert(sizeof(StageTab) % 16 == 0, "class tables are copied in 16-byte units");
-
-// Row addressing of every class of one stage: for each of its eight channels, the byte offset
-// of the row word holding the class's first sample within the stage buffer (8 x uint16) and the
-// funnel shift in bits that brings that sample to bit 0 (8 x uint8).
-struct AddrTab {
-  uint4 addr[kNG][kMaxCls];
-  uint2 sh[kNG][kMaxCls];
-};
-constexpr int kAddrEntries = kNG * kMaxCls * kG;  // one per thread of the first half of the CTA
-static_assert(kAddrEntries <= kThreads, "one addressing entry per thread");
+static_assert(kNG * kMaxLinks <= 64, "a task's fields");
+constexpr int kMaxRun = 16, kMaxBlocks = 64;
 
 __host__ __device__ constexpr size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
 
 struct SmemLayout {
-  size_t raw, z, tab, addr, mbar, total;
+  size_t raw, z, tab, mbar, total;
 };
 
 // The mbarriers come first, at the same place for every tile shape and range (a persistent CTA
 // re-initialises them between tiles of different ranges); the staged rows start 128-byte aligned.
-__host__ __device__ inline SmemLayout smem_layout(int es, int zes, int row_slot, int zcap,
+__host__ __device__ inline SmemLayout smem_layout(int es, int row_slot, int zcap, int pitch,
                                                   int nst) {
   SmemLayout L;
   L.mbar = 0;
@@ -124,11 +134,9 @@ __host__ __device__ inline SmemLayout smem_layout(int es, int zes, int row_slot,
   L.raw = off;
   off = align16(off + (size_t)nst * kRows * row_slot * es);
   L.z = off;
-  off = align16(off + (size_t)2 * zcap * zes);
+  off = align16(off + (size_t)2 * zcap * 4);
   L.tab = off;
-  off = align16(off + sizeof(StageTab) * nst);
-  L.addr = off;
-  off = align16(off + sizeof(AddrTab) * 2);
+  off = align16(off + (size_t)pitch * nst);
   L.total = off;
   return L;
 }
@@ -203,7 +211,8 @@ __device__ __forceinline__ int64_t first_seg(const TiledArgs& a, int64_t j0, int
 __device__ __forceinline__ int32_t stage_xmin(const TiledArgs& a, int stage, int nstages,
                                               int tile) {
   if (stage >= nstages) return 0;
-  return __ldg(&reinterpret_cast<const StageTab*>(a.tabs)[(size_t)tile * nstages + stage].xmin);
+  return __ldg(&reinterpret_cast<const StageTab*>(
+                    a.tabs + ((size_t)tile * nstages + stage) * a.tab_pitch)->xmin);
 }
 
 // Issue of one stage by one thread: one tensor copy of the stage's 16 rows (segments
@@ -211,12 +220,12 @@ __device__ __forceinline__ int32_t stage_xmin(const TiledArgs& a, int stage, int
 // bulk copy of its class table, after arming the stage's mbarrier with their bytes.
 template <typename T>
 __device__ __forceinline__ void issue_stage(const TiledArgs& a, int stage, int nstages,
-                                            T* raw_buf, StageTab* tab_buf,
+                                            T* raw_buf, unsigned char* tab_buf,
                                             unsigned long long* bar, int32_t xmin, int64_t j0,
                                             int tile) {
   const uint32_t row_bytes = (uint32_t)a.row_slot * (uint32_t)sizeof(T);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  mbar_arrive_expect_tx(bar, kRows * row_bytes + (uint32_t)sizeof(StageTab));
+  mbar_arrive_expect_tx(bar, kRows * row_bytes + (uint32_t)a.tab_pitch);
   const int32_t seg = (int32_t)first_seg<T>(a, j0, xmin);
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
@@ -224,225 +233,169 @@ __device__ __forceinline__ void issue_stage(const TiledArgs& a, int stage, int n
       "l"(reinterpret_cast<uint64_t>(&a.rows)), "r"(0), "r"(seg), "r"(stage * kRows),
       "r"(smem_addr(bar))
       : "memory");
-  bulk_g2s(tab_buf, a.tabs + ((size_t)tile * nstages + stage) * sizeof(StageTab),
-           (uint32_t)sizeof(StageTab), bar);
+  bulk_g2s(tab_buf, a.tabs + ((size_t)tile * nstages + stage) * a.tab_pitch,
+           (uint32_t)a.tab_pitch, bar);
 }
 
-// One addressing entry of a stage: entry e = (group, class, channel). The row's copy starts at
-// segment first_seg (issue_stage), so the class's first sample sits
-// m0 + j0 + s_first - first_seg * (segment elements) + rel elements into the row. Its inputs come
-// from the class table and the delay table in global memory (the staged copy of the table may
-// still be in flight), loaded one iteration before the entry is formed.
-struct AddrInputs {
-  int32_t ncls;  // classes of the entry's group (0: no such group)
-  int32_t rel;
-  int32_t smin;
-  int32_t xmin;
-};
-
-__device__ __forceinline__ AddrInputs addr_inputs(const TiledArgs& a, int stage, int nstages,
-                                                  int ngroups, int trial0, int e, int tile) {
-  AddrInputs in{0, 0, 0, 0};
-  const int gl = e / (kMaxCls * kG), p = (e / kG) % kMaxCls, k = e % kG;
-  if (stage < nstages && stage * kNG + gl < ngroups) {
-    const StageTab* st =
-        &reinterpret_cast<const StageTab*>(a.tabs)[(size_t)tile * nstages + stage];
-    const GroupTab* gt = &st->g[gl];
-    in.xmin = __ldg(&st->xmin);
-    in.ncls = __ldg(&gt->ncls);
-    in.rel = __ldg(&gt->cls[p].rel[k]);  // the table is zero past the group's classes
-    in.smin = __ldg(a.shifts + (int64_t)trial0 * a.cpad + stage * kRows + gl * kG + k);
-  }
-  return in;
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(addr));
+  return v;
 }
-
-template <typename T>
-__device__ __forceinline__ void addr_entry(const TiledArgs& a, const AddrInputs& in, int64_t j0,
-                                           int e, AddrTab* at) {
-  constexpr int SEG = kSegBytes / (int)sizeof(T);
-  const int gl = e / (kMaxCls * kG), p = (e / kG) % kMaxCls, k = e % kG;
-  if (p >= in.ncls) return;
-  const int row = gl * kG + k;
-  const int ph = (int)(a.m0 + j0 + in.smin - first_seg<T>(a, j0, in.xmin) * SEG);
-  const uint32_t byte = (uint32_t)(row * a.row_slot + in.rel + ph) * (uint32_t)sizeof(T);
-  reinterpret_cast<uint16_t*>(&at->addr[gl][p])[k] = (uint16_t)(byte & ~3u);
-  reinterpret_cast<uint8_t*>(&at->sh[gl][p])[k] = (uint8_t)((byte & 3u) * 8u);
-}
-
-// The eight channel rows of one class, as one lane reads them: shared-memory byte address of
-// the row word holding its first unit, and the funnel shift of each channel.
-struct RowItem {
-  uint32_t addr[kG];
-  uint32_t sh[kG];
-};
 
 template <typename T>
 struct Word;
 
-// Row words of channel k at byte offset OFF: the word holding the class's first sample and the
-// next one.
-template <int OFF>
-__device__ __forceinline__ void row_words(const RowItem& it, int k, uint32_t& w0, uint32_t& w1) {
-  w0 = lds<OFF>(it.addr[k]);
-  w1 = lds<OFF + 4>(it.addr[k]);
+// The two row words holding a lane's samples of one channel: bits 0 .. 19 of w8 are 8 x the byte
+// offset of the lane-0 sample in the stage buffer (below 2^16 bytes plus a phase below 2^7; a
+// step's sign sits above), base is the buffer's address plus one word per unit.
+__device__ __forceinline__ void row_words(uint32_t base, uint32_t w8, uint32_t& w0, uint32_t& w1) {
+  const uint32_t addr = base + ((w8 >> 3) & 0x1FFFCu);
+  w0 = lds<0>(addr);
+  w1 = lds<4>(addr);
 }
 
 // uint8 data. Unit u covers pair words 4u .. 4u + 3, i.e. the eight-channel sums
-// S[4u .. 4u + 4] (one more than its words, which the last pair word needs). Each channel's two
-// row words are funnel-shifted to the class's first sample; bytes are split into even/odd
-// 16-bit lanes so that eight channels add without carries (8 x 255 < 2^16). The fifth sum is
-// the next unit's first one, S[4(u + 1)]: the next lane's, taken with one shuffle. So a block of
-// 32 lanes stores 31 units (lanes 0 .. 30); lane 31 computes the next block's first unit only
-// to hand its first sum to lane 30 (kBlock = 31). The pair words go to the class's even plane
-// (4u, 4u + 2) and odd plane (4u + 1, 4u + 3); lanes take consecutive units, so every load and
-// store is free of bank conflicts. Every lane of the warp runs the unit (the shuffle needs them
-// all); `live` says whether this lane's words are stored.
+// S[4u .. 4u + 4] (one more than its words, which the last pair word needs). A channel's two row
+// words are funnel-shifted to the unit's first sample; bytes are split into even/odd 16-bit lanes
+// so that eight channels add without carries (8 x 255 < 2^16). The fifth sum is the next unit's
+// first one, S[4(u + 1)]: the next lane's, taken with one shuffle. So a block of 32 lanes stores
+// 31 units (lanes 0 .. 30); lane 31 computes the next block's first unit only to hand its first
+// sum to lane 30. The pair words go to the class's even plane (4u, 4u + 2) and odd plane (4u + 1,
+// 4u + 3); lanes take consecutive units, so every load and store is free of bank conflicts.
 template <>
 struct Word<uint8_t> {
-  static constexpr int kUnit = 4;   // pair words per unit
-  static constexpr int kBlock = 31; // units stored per 32-lane block
-  template <int OFF>
-  static __device__ __forceinline__ void unit(const RowItem& it, uint32_t* ev, uint32_t* od,
-                                              bool live) {
-    uint32_t e = 0, o = 0;
-#pragma unroll
-    for (int k = 0; k < kG; ++k) {
-      uint32_t w0, w1;
-      row_words<OFF>(it, k, w0, w1);
-      const uint32_t a = __funnelshift_r(w0, w1, it.sh[k]);  // samples 0..3 in bytes 0..3
-      e += a & 0x00FF00FFu;                                  // samples 0, 2
-      o += __byte_perm(a, 0, 0x4341);                        // samples 1, 3
-    }
+  static constexpr int kUnit = 4;  // pair words per unit
+  uint32_t e = 0, o = 0;           // samples (0, 2) and (1, 3) in 16-bit lanes
+  __device__ __forceinline__ void add(uint32_t base, uint32_t w8) {
+    uint32_t w0, w1;
+    row_words(base, w8, w0, w1);
+    const uint32_t a = __funnelshift_r(w0, w1, w8);  // samples 0..3 in bytes 0..3
+    e += a & 0x00FF00FFu;
+    o += __byte_perm(a, 0, 0x4341);
+  }
+  // one channel's samples r .. r + 3 replaced by r + 1 .. r + 4 (sign 1) or the reverse (-1)
+  __device__ __forceinline__ void step(uint32_t base, uint32_t w8, int sign) {
+    uint32_t w0, w1;
+    row_words(base, w8, w0, w1);
+    const uint32_t a = __funnelshift_r(w0, w1, w8);
+    const uint32_t x4 = __funnelshift_r(w1, w1, w8);               // sample 4 in byte 0
+    const uint32_t a02 = a & 0x00FF00FFu, a13 = __byte_perm(a, 0, 0x4341);
+    const uint32_t a24 = __byte_perm(a, x4, 0x0402) & 0x00FF00FFu;  // samples 2, 4
+    e += (a13 - a02) * (uint32_t)sign;
+    o += (a24 - a13) * (uint32_t)sign;
+  }
+  __device__ __forceinline__ void emit(uint32_t ev, uint32_t od, uint32_t v, uint32_t n) const {
     const uint32_t nx = __shfl_down_sync(0xffffffffu, e, 1);  // low half: S4 (next unit's S0)
-    if (live) {
-      uint2 x, y;
-      x.x = __byte_perm(e, o, 0x5410);   // S0 | S1 << 16
-      x.y = __byte_perm(e, o, 0x7632);   // S2 | S3 << 16
-      y.x = __byte_perm(o, e, 0x7610);   // S1 | S2 << 16
-      y.y = __byte_perm(o, nx, 0x5432);  // S3 | S4 << 16
-      *reinterpret_cast<uint2*>(ev) = x;
-      *reinterpret_cast<uint2*>(od) = y;
-    }
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.lt.u32 p, %6, %7;\n\t"
+        "@p st.shared.v2.u32 [%0], {%2, %3};\n\t"
+        "@p st.shared.v2.u32 [%1], {%4, %5};\n\t}" ::"r"(ev),
+        "r"(od), "r"(__byte_perm(e, o, 0x5410)),   // S0 | S1 << 16
+        "r"(__byte_perm(e, o, 0x7632)),            // S2 | S3 << 16
+        "r"(__byte_perm(o, e, 0x7610)),            // S1 | S2 << 16
+        "r"(__byte_perm(o, nx, 0x5432)),           // S3 | S4 << 16
+        "r"(v), "r"(n)
+        : "memory");
   }
 };
 
-// uint16 data. Unit u covers pair words 2u, 2u + 1 (sums S[2u .. 2u + 2]) from two row words
-// per channel; 16-bit lanes add eight channels without carries (8 x 255 x d < 2^16), and the
-// third sample, halfword (shift / 16) of the second row word, is added by a DP2A on the
-// rotated word.
+// uint16 data. Unit u covers pair words 2u, 2u + 1 (sums S[2u .. 2u + 2], the third the next
+// lane's first) from two row words per channel; 16-bit lanes add eight channels without carries
+// (8 x 255 x d < 2^16).
 template <>
 struct Word<uint16_t> {
   static constexpr int kUnit = 2;
-  static constexpr int kBlock = 32;  // units per 32-lane block
-  template <int OFF>
-  static __device__ __forceinline__ void unit(const RowItem& it, uint32_t* ev, uint32_t* od,
-                                              bool /*live: always, lanes past the class skip*/) {
-    uint32_t e = 0, s2 = 0;
-#pragma unroll
-    for (int k = 0; k < kG; ++k) {
-      uint32_t w0, w1;
-      row_words<OFF>(it, k, w0, w1);
-      e += __funnelshift_r(w0, w1, it.sh[k]);                  // samples 0, 1
-      s2 = __dp2a_lo(__funnelshift_r(w1, w1, it.sh[k]), 1u, s2);  // sample 2
-    }
-    *ev = e;                           // S0 | S1 << 16
-    *od = __byte_perm(e, s2, 0x5432);  // S1 | S2 << 16
+  uint32_t e = 0;  // samples 0, 1
+  __device__ __forceinline__ void add(uint32_t base, uint32_t w8) {
+    uint32_t w0, w1;
+    row_words(base, w8, w0, w1);
+    e += __funnelshift_r(w0, w1, w8);
+  }
+  __device__ __forceinline__ void step(uint32_t base, uint32_t w8, int sign) {
+    uint32_t w0, w1;
+    row_words(base, w8, w0, w1);
+    const uint32_t a = __funnelshift_r(w0, w1, w8);
+    const uint32_t x2 = __funnelshift_r(w1, w1, w8);  // sample 2 in the low half
+    e += (__byte_perm(a, x2, 0x5432) - a) * (uint32_t)sign;
+  }
+  __device__ __forceinline__ void emit(uint32_t ev, uint32_t od, uint32_t v, uint32_t n) const {
+    const uint32_t nx = __shfl_down_sync(0xffffffffu, e, 1);
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.lt.u32 p, %4, %5;\n\t"
+        "@p st.shared.u32 [%0], %2;\n\t"
+        "@p st.shared.u32 [%1], %3;\n\t}" ::"r"(ev),
+        "r"(od), "r"(e),                  // S0 | S1 << 16
+        "r"(__byte_perm(e, nx, 0x5432)),  // S1 | S2 << 16
+        "r"(v), "r"(n)
+        : "memory");
   }
 };
 
-// Add one pair word (S[u] | S[u + 1] << 16, or the sum of two groups' words) to the two
-// outputs it serves.
+// Add one pair word's two packed sums to the two outputs it serves.
 __device__ __forceinline__ void pair_add(uint32_t z, uint32_t& even, uint32_t& odd) {
   even = __dp2a_lo(z, 0x0001u, even);  // + low half
   odd = __dp2a_lo(z, 0x0100u, odd);    // + high half
 }
 
-// Build every pair word of one stage: a warp walks the ranges of work list `list`; lane l builds
-// unit 32 * b + l of every block b of a range. With HALVES = 1 the warp builds every block, two
-// per pass; with HALVES = 2 two warps share the list, warp `half` building blocks b0 + half,
-// b0 + half + 2, ...
-template <typename T, int HALVES>
-__device__ __forceinline__ void build_stage(const StageTab& tb, const AddrTab& at, uint32_t rawb,
-                                            uint32_t* Zs, int list, int lane, int half) {
-  constexpr int U = Word<T>::kUnit;
-  const int nw = tb.nwork[list];
-  for (int w = 0; w < nw; ++w) {
-    const uint32_t wk = tb.work[list][w];
-    const int gi = (int)((wk >> 4) & 1), p = (int)(wk & 15);
-    const int b0 = (int)((wk >> 8) & 255), nb = (int)(wk >> 16);
-    const int zlen = tb.g[gi].cls[p].zlen;
-    constexpr int B = Word<T>::kBlock;  // units per block
-    int u = B * (b0 + (HALVES == 2 ? half : 0)) + lane;
-    const uint4 ad = at.addr[gi][p];
-    const uint2 sv = at.sh[gi][p];
-    const uint32_t base = rawb + 4u * (uint32_t)u;  // one row word per unit
-    RowItem it;
-    it.addr[0] = base + (ad.x & 0xFFFFu);
-    it.addr[1] = base + (ad.x >> 16);
-    it.addr[2] = base + (ad.y & 0xFFFFu);
-    it.addr[3] = base + (ad.y >> 16);
-    it.addr[4] = base + (ad.z & 0xFFFFu);
-    it.addr[5] = base + (ad.z >> 16);
-    it.addr[6] = base + (ad.w & 0xFFFFu);
-    it.addr[7] = base + (ad.w >> 16);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      it.sh[k] = sv.x >> (8 * k);
-      it.sh[k + 4] = sv.y >> (8 * k);
+// Build one warp's share of a stage's pair words: per task (a run of chained links, one block
+// of 31 units; lane l takes unit 31 * block + l) the eight channels of the first class, then per
+// further link the channel step that leads to it. Every lane runs every unit (the shuffle needs
+// them all); lanes 0 .. 30 store the units inside the class's own range. Loads of lanes past the
+// staged rows stay inside the CTA's shared memory (the rows are followed by the word planes).
+// The loop counts come from warp reductions, which the compiler knows to be the same in every
+// lane: the loops then need no divergence bookkeeping.
+template <typename T>
+__device__ __forceinline__ void build_stage(uint32_t tabp, uint32_t rawb, uint32_t zb,
+                                            uint32_t pos, int warp, int lane) {
+  constexpr uint32_t SEG = kSegBytes / sizeof(T);
+  uint32_t wt;
+  asm volatile("ld.shared.u16 %0, [%1];"
+               : "=r"(wt)
+               : "r"(tabp + (uint32_t)offsetof(StageTab, wtask) + 2u * warp));
+  const uint32_t xmin = lds<offsetof(StageTab, xmin)>(tabp);
+  const uint32_t ph8 = ((pos + xmin) & (SEG - 1)) * 8u * (uint32_t)sizeof(T);
+  uint32_t tp = tabp + (uint32_t)offsetof(StageTab, task) + 2u * (wt & 0xFFu);
+  for (uint32_t left = __reduce_max_sync(0xffffffffu, wt >> 8); left > 0; --left, tp += 2) {
+    uint32_t tk;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(tk) : "r"(tp));
+    tk = __reduce_max_sync(0xffffffffu, tk);
+    uint32_t cp = tabp + (uint32_t)sizeof(StageTab) + (tk & 63u) * (uint32_t)sizeof(ClsLink);
+    const uint32_t u = (tk >> 10) * kBlock + lane;
+    const uint32_t us = lane < kBlock ? u : 0x80000000u;  // lane 31 stores nothing
+    const uint32_t base = rawb + 4u * u;
+    const uint32_t zl = zb + (uint32_t)sizeof(uint32_t) * (Word<T>::kUnit / 2) * u;
+    Word<T> w;
+    const uint4 a = lds128(cp), b = lds128(cp + 16);
+    uint4 lk = lds128(cp + 32);
+    w.add(base, a.x + ph8);
+    w.add(base, a.y + ph8);
+    w.add(base, a.z + ph8);
+    w.add(base, a.w + ph8);
+    w.add(base, b.x + ph8);
+    w.add(base, b.y + ph8);
+    w.add(base, b.z + ph8);
+    w.add(base, b.w + ph8);
+    // the next link's record is loaded before this one's stores
+    uint32_t n = (tk >> 6) & 15u;
+#pragma unroll 1
+    for (; n >= 2; n -= 2, cp += 2u * (uint32_t)sizeof(ClsLink)) {
+      const uint4 l1 = lds128(cp + 32 + sizeof(ClsLink));
+      w.emit(zl + lk.y, zl + lk.z, us - (lk.w & 0xFFFFu), lk.w >> 16);
+      w.step(base, l1.x + ph8, (int32_t)l1.x >> 30);
+      lk = lds128(cp + 32 + 2 * sizeof(ClsLink));
+      w.emit(zl + l1.y, zl + l1.z, us - (l1.w & 0xFFFFu), l1.w >> 16);
+      w.step(base, lk.x + ph8, (int32_t)lk.x >> 30);
     }
-    // even plane: pair words 0, 2, 4, ... of the class; odd plane: 1, 3, 5, ...
-    uint32_t* ev = Zs + tb.g[gi].cls[p].zoff + (U / 2) * u;
-    uint32_t* od = ev + zlen / 2;
-    if constexpr (B == 31) {
-      // uint8: every lane runs every unit (shuffles); lanes 0 .. 30 store the block's units.
-      // Lanes past the class compute nothing they store; their loads stay inside the CTA's
-      // shared memory (the staged rows are followed by the word planes).
-      const bool store_lane = lane < 31;
-      if (HALVES == 1) {
-        for (int b = 0; b < nb; b += 2) {
-          Word<T>::template unit<0>(it, ev, od, store_lane && u * U < zlen);
-          if (b + 1 < nb)
-            Word<T>::template unit<4 * B>(it, ev + B * U / 2, od + B * U / 2,
-                                          store_lane && (u + B) * U < zlen);
-#pragma unroll
-          for (int k = 0; k < kG; ++k) it.addr[k] += 8u * B;  // two blocks further
-          u += 2 * B;
-          ev += B * U;
-          od += B * U;
-        }
-      } else {
-        for (int b = half; b < nb; b += 2) {
-          Word<T>::template unit<0>(it, ev, od, store_lane && u * U < zlen);
-#pragma unroll
-          for (int k = 0; k < kG; ++k) it.addr[k] += 8u * B;
-          u += 2 * B;
-          ev += B * U;
-          od += B * U;
-        }
-      }
-    } else {
-      // uint16: lanes past the class skip their units
-      if (HALVES == 1) {
-        for (int b = 0; b < nb; b += 2) {
-          if (u * U < zlen) Word<T>::template unit<0>(it, ev, od, true);
-          if (b + 1 < nb && (u + B) * U < zlen)
-            Word<T>::template unit<4 * B>(it, ev + B * U / 2, od + B * U / 2, true);
-#pragma unroll
-          for (int k = 0; k < kG; ++k) it.addr[k] += 8u * B;  // two blocks further
-          u += 2 * B;
-          ev += B * U;
-          od += B * U;
-        }
-      } else {
-        for (int b = half; b < nb; b += 2) {
-          if (u * U < zlen) Word<T>::template unit<0>(it, ev, od, true);
-#pragma unroll
-          for (int k = 0; k < kG; ++k) it.addr[k] += 8u * B;
-          u += 2 * B;
-          ev += B * U;
-          od += B * U;
-        }
-      }
+    w.emit(zl + lk.y, zl + lk.z, us - (lk.w & 0xFFFFu), lk.w >> 16);
+    if (n) {
+      lk = lds128(cp + 32 + sizeof(ClsLink));
+      w.step(base, lk.x + ph8, (int32_t)lk.x >> 30);
+      w.emit(zl + lk.y, zl + lk.z, us - (lk.w & 0xFFFFu), lk.w >> 16);
     }
   }
 }
@@ -671,6 +624,18 @@ __global__ void __launch_bounds__(512) k_fused_edges(const __grid_constant__ Til
   }
 }
 
+// Word 32k + lane of every trial's sequence in both groups (shared-memory addresses of word 0)
+// added to the packed sums.
+template <int KP, int kTPW>
+__device__ __forceinline__ void add_words(const uint32_t (&zp)[kTPW], const uint32_t (&zq)[kTPW],
+                                          uint32_t (&pk)[kTPW][KP]) {
+#pragma unroll
+  for (int k = 0; k < KP; ++k)
+#pragma unroll
+    for (int q = 0; q < kTPW; ++q)
+      pk[q][k] += lds<0>(zp[q] + 128 * k) + lds<0>(zq[q] + 128 * k);
+}
+
 template <typename T, int TT, int NS, int D, int NT, bool FUSED = false>
 __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
                                           unsigned char* smem, bool reuse,
@@ -679,12 +644,13 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
   constexpr int KP = TT / 64;       // pair words per lane and trial
   constexpr int W = NT / 32;        // warps
   constexpr int kTPW = D / W;       // trials per warp
-  constexpr int HALVES = W / kWarps;  // warps sharing a build work list
-  const SmemLayout SL = smem_layout(sizeof(T), 4, a.row_slot, a.zcap, NS);
+  const SmemLayout SL = smem_layout(sizeof(T), a.row_slot, a.zcap, a.tab_pitch, NS);
   T* raw = reinterpret_cast<T*>(smem + SL.raw);
   uint32_t* Zbuf = reinterpret_cast<uint32_t*>(smem + SL.z);
-  StageTab* tab = reinterpret_cast<StageTab*>(smem + SL.tab);
-  AddrTab* atab = reinterpret_cast<AddrTab*>(smem + SL.addr);
+  unsigned char* tab = smem + SL.tab;
+  uint32_t sraw = smem_addr(raw), sz = smem_addr(Zbuf), stab = smem_addr(tab);
+  asm volatile("" : "+r"(sraw), "+r"(sz), "+r"(stab));  // worked out once, not per use
+  const uint32_t pos = (uint32_t)(a.m0 + (int64_t)by * TT);  // ring column of the tile (mod 2^32)
   unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + SL.mbar);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -704,18 +670,6 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  // row addressing of stages 0 and 1; stage s + 2 is formed during iteration s from inputs
-  // loaded during iteration s - 1 (the prologue for s = 0)
-  AddrInputs ain{0, 0, 0, 0};
-  {
-    const int s0 = tid / kAddrEntries;
-    if (s0 < 2) {
-      const AddrInputs in0 =
-          addr_inputs(a, s0, nstages, ngroups, trial0, tid % kAddrEntries, bx);
-      addr_entry<T>(a, in0, j0, tid % kAddrEntries, &atab[s0]);
-    }
-    if (tid < kAddrEntries) ain = addr_inputs(a, 2, nstages, ngroups, trial0, tid, bx);
-  }
   __syncthreads();
   // stages whose copies have been issued: NS in the prologue, then one per iteration s >= 1
   // (the same count in every thread)
@@ -723,13 +677,12 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
   int32_t xmin_next = 0;  // first delay of the next stage to issue (issuing thread)
   if (tid == NT - 32) {
     for (int s = 0; s < NS && s < nstages; ++s)
-      issue_stage<T>(a, s, nstages, raw + (size_t)s * stage_elems, &tab[s], &mbar[s],
+      issue_stage<T>(a, s, nstages, raw + (size_t)s * stage_elems, tab + s * a.tab_pitch, &mbar[s],
                      stage_xmin(a, s, nstages, bx), j0, bx);
     xmin_next = stage_xmin(a, NS, nstages, bx);
   }
   bool ok0 = mbar_wait_bounded(&mbar[0], 0);
-  if (ok0) build_stage<T, HALVES>(tab[0], atab[0], smem_addr(raw), Zbuf, warp % kWarps, lane,
-                                  warp / kWarps);
+  if (ok0) build_stage<T>(stab, sraw, sz, pos, warp, lane);
   bool aborted = __syncthreads_or(!ok0);
   int s_abort = 0;  // first stage whose copies may still be in flight
 
@@ -738,71 +691,77 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
   for (int q = 0; q < kTPW; ++q)
 #pragma unroll
     for (int k = 0; k < KT; ++k) acc[q][k] = 0;
+  uint32_t pk[kTPW][KP];  // packed sums of the stages since the last flush
+#pragma unroll
+  for (int q = 0; q < kTPW; ++q)
+#pragma unroll
+    for (int k = 0; k < KP; ++k) pk[q][k] = 0;
+  int left = a.flush;  // stages until the packed sums go to the 32-bit outputs
+  const uint32_t raw_step = (uint32_t)(stage_elems * sizeof(T)), tab_step = (uint32_t)a.tab_pitch;
+  int b0 = 0, b1 = 1;     // staging buffers of stages s and s + 1
+  uint32_t par1 = 0;      // barrier parity of stage s + 1
+  uint32_t zcur = sz, znext = sz + a.zcap * 4u;  // word buffers of stages s and s + 1
 
   for (int s = 0; s < nstages && !aborted; ++s) {
     const int ng = min(kNG, ngroups - s * kNG);
     // (1) TMA for stage s + NS - 1 into the buffers stage s - 1 used (its words were built
     //     during stage s - 2 and its table last read by the accumulation of stage s - 1)
     if (s >= 1 && s + NS - 1 < nstages) {
-      const int s2 = s + NS - 1;
-      const int b2 = s2 % NS;
       if (tid == NT - 32) {
-        issue_stage<T>(a, s2, nstages, raw + (size_t)b2 * stage_elems, &tab[b2], &mbar[b2],
-                       xmin_next, j0, bx);
-        xmin_next = stage_xmin(a, s2 + 1, nstages, bx);
+        const int b2 = b0 == 0 ? NS - 1 : b0 - 1;
+        issue_stage<T>(a, s + NS - 1, nstages, raw + (size_t)b2 * stage_elems,
+                       tab + b2 * a.tab_pitch, &mbar[b2], xmin_next, j0, bx);
+        xmin_next = stage_xmin(a, s + NS, nstages, bx);
       }
-      issued = s2 + 1;
-    }
-    // row addressing of stage s + 2, into the buffer stage s used (read during iteration s - 1)
-    if (tid < kAddrEntries) {
-      if (s + 2 < nstages) addr_entry<T>(a, ain, j0, tid, &atab[s & 1]);
-      ain = addr_inputs(a, s + 3, nstages, ngroups, trial0, tid, bx);
+      issued = s + NS;
     }
     // (2) pair words of stage s + 1
     bool ok = true;
     if (s + 1 < nstages) {
-      const int b1 = (s + 1) % NS;
-      ok = mbar_wait_bounded(&mbar[b1], (uint32_t)(((s + 1) / NS) & 1));
+      ok = mbar_try_wait(&mbar[b1], par1) || mbar_wait_bounded(&mbar[b1], par1);
       if (ok)
-        build_stage<T, HALVES>(tab[b1], atab[(s + 1) & 1],
-                               smem_addr(raw + (size_t)b1 * stage_elems),
-                               Zbuf + (size_t)((s + 1) & 1) * a.zcap, warp % kWarps, lane,
-                               warp / kWarps);
+        build_stage<T>(stab + b1 * tab_step, sraw + b1 * raw_step, znext, pos, warp, lane);
     }
     // (3) accumulate stage s: lane l of the warp reads, for each of its trials, pair word
     //     l + 32k of the trial's plane in both groups (outputs 2(l + 32k) and 2(l + 32k) + 1)
     {
-      const StageTab& tc = tab[s % NS];
-      const uint32_t* Zs = Zbuf + (size_t)(s & 1) * a.zcap + lane;
-      const uint32_t* zp[kTPW];
-      const uint32_t* zq[kTPW];
+      const uint32_t tc = stab + b0 * tab_step + (uint32_t)offsetof(StageTab, zstart) +
+                          2u * kTPW * warp;
+      const uint32_t zs = zcur + 4u * lane;
+      uint32_t zp[kTPW], zq[kTPW];
       static_assert(kTPW == 4 || kTPW == 2, "a warp's offsets are one 8- or 4-byte load");
+      const uint32_t e0 = lds<0>(tc), e1 = lds<2 * kMaxTileTrials>(tc);
+      zp[0] = zs + 4u * (e0 & 0xFFFFu); zp[1] = zs + 4u * (e0 >> 16);
+      zq[0] = zs + 4u * (e1 & 0xFFFFu); zq[1] = zs + 4u * (e1 >> 16);
       if constexpr (kTPW == 4) {
-        const uint2 e0 = *reinterpret_cast<const uint2*>(tc.g[0].zstart + warp * 4);
-        const uint2 e1 = *reinterpret_cast<const uint2*>(tc.g[1].zstart + warp * 4);
-        zp[0] = Zs + (e0.x & 0xFFFFu); zp[1] = Zs + (e0.x >> 16);
-        zp[2] = Zs + (e0.y & 0xFFFFu); zp[3] = Zs + (e0.y >> 16);
-        zq[0] = Zs + (e1.x & 0xFFFFu); zq[1] = Zs + (e1.x >> 16);
-        zq[2] = Zs + (e1.y & 0xFFFFu); zq[3] = Zs + (e1.y >> 16);
-      } else {
-        const uint32_t e0 = *reinterpret_cast<const uint32_t*>(tc.g[0].zstart + warp * 2);
-        const uint32_t e1 = *reinterpret_cast<const uint32_t*>(tc.g[1].zstart + warp * 2);
-        zp[0] = Zs + (e0 & 0xFFFFu); zp[1] = Zs + (e0 >> 16);
-        zq[0] = Zs + (e1 & 0xFFFFu); zq[1] = Zs + (e1 >> 16);
+        const uint32_t e2 = lds<4>(tc), e3 = lds<2 * kMaxTileTrials + 4>(tc);
+        zp[2] = zs + 4u * (e2 & 0xFFFFu); zp[3] = zs + 4u * (e2 >> 16);
+        zq[2] = zs + 4u * (e3 & 0xFFFFu); zq[3] = zs + 4u * (e3 >> 16);
       }
       if (ng == kNG) {  // uniform; only the last stage may hold one group
-#pragma unroll
-        for (int k = 0; k < KP; ++k)
-#pragma unroll
-          for (int q = 0; q < kTPW; ++q)
-            pair_add(zp[q][32 * k] + zq[q][32 * k], acc[q][2 * k], acc[q][2 * k + 1]);
+        add_words<KP, kTPW>(zp, zq, pk);
       } else {
 #pragma unroll
         for (int k = 0; k < KP; ++k)
 #pragma unroll
-          for (int q = 0; q < kTPW; ++q) pair_add(zp[q][32 * k], acc[q][2 * k], acc[q][2 * k + 1]);
+          for (int q = 0; q < kTPW; ++q) pk[q][k] += lds<0>(zp[q] + 128 * k);
+      }
+      if (--left == 0 || s + 1 == nstages) {  // uniform
+        left = a.flush;
+#pragma unroll
+        for (int k = 0; k < KP; ++k)
+#pragma unroll
+          for (int q = 0; q < kTPW; ++q) {
+            pair_add(pk[q][k], acc[q][2 * k], acc[q][2 * k + 1]);
+            pk[q][k] = 0;
+          }
       }
     }
+    b0 = b1;
+    if (++b1 == NS) b1 = 0, par1 ^= 1u;
+    const uint32_t zt = zcur;
+    zcur = znext;
+    znext = zt;
     if (__syncthreads_or(!ok)) {
       aborted = true;
       s_abort = s + 1;
@@ -928,7 +887,7 @@ __global__ void __launch_bounds__(512, 1)
 
 template <typename T, int TT, int NS, int D, int NT>
 cudaError_t launch_tiled_t(const TiledArgs& a, cudaStream_t st) {
-  const SmemLayout SL = smem_layout(sizeof(T), 4, a.row_slot, a.zcap, NS);
+  const SmemLayout SL = smem_layout(sizeof(T), a.row_slot, a.zcap, a.tab_pitch, NS);
   dim3 grid((unsigned)((a.n_trials + D - 1) / D), (unsigned)((a.nout + TT - 1) / TT));
   k_dedisp_tiled<T, TT, NS, D, NT><<<grid, NT, SL.total, st>>>(a);
   return cudaGetLastError();
@@ -958,35 +917,84 @@ cudaError_t prepare_t(size_t smem) {
 
 namespace {
 
-// Cut a stage's classes into blocks of B units (U pair words each; B = 31 for uint8 data, 32
-// for uint16: Word<T>::kBlock) and deal them to the warps in contiguous shares of
-// ceil(blocks / warps); false if a share needs more ranges than a warp's list holds or a class
-// more blocks than a range can name.
-bool deal_work(StageTab& st, int U, int B) {
-  int total = 0;
+// Instruction costs of a build task, for dealing tasks to warps: its set-up with the eight
+// channels of its first class, each link's store, each channel step (counted from build_stage).
+struct BuildCost {
+  int base, emit, step;
+};
+constexpr BuildCost kCostU8{100, 16, 18}, kCostU16{80, 13, 14};
+
+// Deal a stage's build work to W warps: per group and block of 31 units, the chain of links,
+// from and to classes that store units in the block, cut where the plan breaks the chain
+// (link without a step) and where a warp has its share. The share is the smallest, found by
+// bisection, with which W warps suffice. False if the task list overflows.
+bool deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
+  const int first[kNG + 1] = {0, st.nlink[0], st.nlink[0] + st.nlink[1]};
+  int nblk[kNG] = {0, 0};
   for (int gl = 0; gl < kNG; ++gl)
-    for (int p = 0; p < st.g[gl].ncls; ++p) total += (st.g[gl].cls[p].zlen / U + B - 1) / B;
-  const int share = (total + kWarps - 1) / kWarps;
-  int w = 0, used = 0;
-  for (int gl = 0; gl < kNG; ++gl)
-    for (int p = 0; p < st.g[gl].ncls; ++p) {
-      const int nb = (st.g[gl].cls[p].zlen / U + B - 1) / B;
-      if (nb > 255) return false;
-      int b = 0;
-      while (b < nb) {
-        const int take = std::min(nb - b, share - used);
-        if (w >= kWarps || st.nwork[w] >= kMaxWork) return false;
-        st.work[w][st.nwork[w]++] =
-            (uint32_t)(gl << 4 | p) | (uint32_t)b << 8 | (uint32_t)take << 16;
-        b += take;
-        used += take;
-        if (used == share) {
-          ++w;
-          used = 0;
+    for (int p = first[gl]; p < first[gl + 1]; ++p)
+      nblk[gl] = std::max(nblk[gl], (int)(cls[p].ulo() + cls[p].un() + kBlock - 1) / kBlock);
+  if (nblk[0] > kMaxBlocks || nblk[1] > kMaxBlocks) return false;
+  auto stores = [&](int p, int b) {
+    return cls[p].un() && (int)cls[p].ulo() < (b + 1) * kBlock &&
+           (int)(cls[p].ulo() + cls[p].un()) > b * kBlock;
+  };
+  // deal with a given share; returns the warps used (-1 if the task list overflows)
+  auto deal = [&](int share, bool out) {
+    int w = 0, load = 0, nt = 0;
+    if (out) std::memset(st.wtask, 0, sizeof st.wtask);
+    for (int gl = 0; gl < kNG; ++gl)
+      for (int b = 0; b < nblk[gl]; ++b) {
+        int p = first[gl];
+        while (p < first[gl + 1]) {
+          if (!stores(p, b)) {
+            ++p;
+            continue;
+          }
+          if (load > 0 && load + C.base + C.emit > share) {
+            ++w;
+            if (out) st.wtask[w] = (uint16_t)nt;
+            load = 0;
+          }
+          // a run from p: extend while the links chain and fit the share
+          load += C.base + C.emit;
+          int last = p, cost = 0;
+          for (int q = p + 1; q < first[gl + 1] && cls[q].step && q < p + kMaxRun; ++q) {
+            cost += C.step + C.emit;
+            if (load + cost > share) break;
+            if (stores(q, b)) {
+              load += cost;
+              cost = 0;
+              last = q;
+            }
+          }
+          if (out) {
+            if (nt == kMaxTasks) return -1;
+            st.task[nt] = (uint16_t)(p | (last - p) << 6 | b << 10);
+            st.wtask[w] += 1 << 8;
+          }
+          ++nt;
+          p = last + 1;
         }
       }
-    }
-  return true;
+    return w + 1;
+  };
+  int lo = C.base + C.emit, hi = lo;
+  while (deal(hi, false) > W) {
+    lo = hi;
+    hi *= 2;
+  }
+  while (hi - lo > 8) {
+    const int mid = (lo + hi) / 2;
+    if (deal(mid, false) > W) lo = mid; else hi = mid;
+  }
+  return deal(hi, true) > 0;
+}
+
+int stage_tasks(const StageTab& st) {
+  int n = 0;
+  for (int w = 0; w < kMaxWarps; ++w) n += st.wtask[w] >> 8;
+  return n;
 }
 
 // Self-test of the bounded wait above: one thread arms a fresh mbarrier that nothing ever
@@ -1014,47 +1022,46 @@ cudaError_t launch_wait_selftest(int32_t* err, cudaStream_t st) {
 //   accumulation : every warp loads, for its kTPW trials and TT / 64 pair-word columns, one word
 //                  per group present (trials past the range's end load too), plus the trials'
 //                  zstart entries;
-//   build        : per block (31 units for uint8 data, 32 for uint16), 2 row words for each of
-//                  the 8 channels and the two plane stores; per work range, its descriptor,
-//                  class entry and addressing words;
-//   addressing   : two stores per (group, class, channel) entry, by the first 8 warps;
+//   build        : per task its descriptor, the first class's eight row offsets and two row words
+//                  per channel; per link its record, its step's two row words and the two plane
+//                  stores;
 //   copies       : the tensor copy of the 16 staged rows and the bulk copy of the stage table.
 static void tiled_smem_work(TiledPlan& P, int ntiles, int nstages, int ngroups, bool u16) {
-  const StageTab* tabs = reinterpret_cast<const StageTab*>(P.tabs.data());
-  const int W = P.threads / 32, halves = W / kWarps;
+  const int W = P.threads / 32;
   const int KP = P.tt / 64, kTPW = P.trials / W;
-  const int sts_per_block = u16 ? 2 : 4;
+  const int sts_per_class = u16 ? 2 : 4;
   int64_t lsu = 0, bytes = 0;
   for (int ti = 0; ti < ntiles; ++ti)
     for (int s = 0; s < nstages; ++s) {
-      const StageTab& st = tabs[(size_t)ti * nstages + s];
+      const uint8_t* tp = P.tabs.data() + ((size_t)ti * nstages + s) * P.tab_pitch;
+      const StageTab& st = *reinterpret_cast<const StageTab*>(tp);
       const int ng = std::min(kNG, ngroups - s * kNG);
       lsu += (int64_t)W * kTPW * KP * ng;             // accumulation words
-      lsu += (int64_t)W * ng;                         // zstart entries (one load per group)
-      lsu += W;                                       // nwork
-      for (int w = 0; w < kWarps; ++w)
-        for (int k = 0; k < st.nwork[w]; ++k) {
-          const uint32_t wk = st.work[w][k];
-          const int nb = (int)(wk >> 16);
-          lsu += 5 * halves;                          // descriptor, zlen, zoff, addr, shift
-          lsu += (int64_t)nb * (2 * kG + sts_per_block);
-        }
-      lsu += (int64_t)(kAddrEntries / 32) * 2;        // addressing stores
-      bytes += (int64_t)kRows * P.row_slot * (u16 ? 2 : 1) + (int64_t)sizeof(StageTab);
+      lsu += (int64_t)W * ng * (kTPW / 2);            // zstart entries (two a load)
+      lsu += 2 * W;                                   // wtask, xmin
+      for (int t = 0; t < stage_tasks(st); ++t) {
+        const int n = (st.task[t] >> 6) & 15;         // links after the first
+        lsu += 3 + 2 * kG;                            // descriptor, row offsets, row words
+        lsu += (int64_t)(n + 1) * (1 + sts_per_class) + 2 * n;
+      }
+      bytes += (int64_t)kRows * P.row_slot * (u16 ? 2 : 1) + P.tab_pitch;
     }
   P.lsu_wavefronts = lsu;
   P.copy_bytes = bytes;
 }
 
 // Host: delay classes of every (trial tile, stage) of one range, as the kernel reads them.
-// Classes are numbered in order of their first trial; a class's zlen pair words start at a
-// multiple of 4 within the stage, groups one after another, the even plane (pair words 0, 2,
-// 4, ...) in the first zlen / 2 words and the odd plane after it. A trial whose sequence starts
-// o words into its class reads plane (o mod 2) from word o / 2 on. Fails (ok = false) where the
-// kernel's limits do not hold: a 16-bit lane holds the sum of two groups' eight channels of
-// values up to 255 x decimation, so decimation must stay at or below 16; delays must be
-// monotone in the trial within a channel; classes, work lists and the staged rows must fit
-// their fixed-size tables and shared memory.
+// Classes of a group are sorted by their relative delays' sum, which makes neighbours differ by
+// few channel steps (on the 4096- and 8192-channel plans within 2% of a nearest-neighbour chain);
+// where two or three steps separate neighbours, links that store nothing go between them, and
+// where more do, the chain breaks. A class's zlen = un x unit
+// pair words start at a multiple of 4 within the stage, groups one after another, the even plane
+// in the first zlen / 2 words and the odd plane after it. A trial whose sequence starts o words
+// into its class reads plane (o mod 2) from word o / 2 on. Fails (ok = false) where the kernel's
+// limits do not hold: a 16-bit lane holds the sum of two groups' eight channels of values up to
+// 255 x decimation, so decimation must stay at or below 16; delays must be monotone in the trial
+// within a channel; classes, tasks and the staged rows must fit their fixed-size tables and
+// shared memory.
 TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int tt, int D,
                      int nt) {
   TiledPlan P;
@@ -1062,55 +1069,93 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
   const bool u16 = decimation > 1;
   if (decimation < 1 || kRows * 255 * decimation > 65535 || cpad % kG) return P;
   if ((D != 64 && D != 32) || (tt != 512 && tt != 256) || (nt != 512 && nt != 1024)) return P;
-  const int NG = kNG, U = u16 ? 2 : 4;
+  const int NG = kNG, U = u16 ? Word<uint16_t>::kUnit : Word<uint8_t>::kUnit;
+  const int es = u16 ? 2 : 1, W = nt / 32;
   const int ngroups = cpad / kG, nstages = (ngroups + NG - 1) / NG;
   const int ntiles = (ntr + D - 1) / D;
-  int64_t spread = 0, zcap = 0, span = 0;
-  std::vector<StageTab> out((size_t)ntiles * nstages);
+  const BuildCost cost = u16 ? kCostU16 : kCostU8;
+  // staged rows: a stage's common copy window runs from the smallest first-trial delay to the
+  // largest last-trial delay of its channels
+  int64_t spread = 0, span = 0;
   for (int ti = 0; ti < ntiles; ++ti) {
     const int t0 = ti * D, n = std::min(D, ntr - t0);
-    for (int c = 0; c < cpad; ++c) {
-      for (int i = 1; i < n; ++i)
-        if (tab[(int64_t)(t0 + i) * cpad + c] < tab[(int64_t)(t0 + i - 1) * cpad + c]) return P;
-      spread = std::max<int64_t>(spread, tab[(int64_t)(t0 + n - 1) * cpad + c] -
-                                             tab[(int64_t)t0 * cpad + c]);
-    }
-    for (int s = 0; s < nstages; ++s) {
-      StageTab& st = out[(size_t)ti * nstages + s];
-      std::memset(&st, 0, sizeof st);
-      // the rows' common copy window: from the smallest first-trial delay to the largest
-      // last-trial delay of the stage's channels
+    const int32_t* a = tab + (int64_t)t0 * cpad;
+    const int32_t* z = tab + (int64_t)(t0 + n - 1) * cpad;
+    for (int i = 1; i < n; ++i)
+      for (int c = 0; c < cpad; ++c)
+        if (a[(int64_t)i * cpad + c] < a[(int64_t)(i - 1) * cpad + c]) return P;
+    for (int c0 = 0; c0 < cpad; c0 += kRows) {
       int32_t xmin = INT32_MAX, xmax = 0;
-      for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c) {
-        xmin = std::min(xmin, tab[(int64_t)t0 * cpad + c]);
-        xmax = std::max(xmax, tab[(int64_t)(t0 + n - 1) * cpad + c]);
+      for (int c = c0; c < std::min(cpad, c0 + kRows); ++c) {
+        xmin = std::min(xmin, a[c]);
+        xmax = std::max(xmax, z[c]);
+        spread = std::max<int64_t>(spread, z[c] - a[c]);
       }
-      st.xmin = xmin;
       span = std::max<int64_t>(span, (int64_t)xmax - xmin);
-      int words = 0;
+    }
+  }
+  if (spread > 65536) return P;
+  const int SEG = kSegBytes / es;
+  P.tt = tt;
+  P.trials = D;
+  P.threads = nt;
+  P.ctas = tile_ctas(D, tt, nt);
+  P.flush = 65535 / (kRows * 255 * decimation);
+  // staged row: the stage's window (span + tt samples) from up to SEG - 1 samples into its
+  // first segment, and 32 samples the word-wise build may read past the last word it uses
+  P.nseg = (int)std::min<int64_t>((span + tt + 32 + 2 * SEG - 2) / SEG, 256);
+  if (P.nseg > 255) return P;
+  P.row_slot = P.nseg * SEG;
+  // row offsets and their phase fit the 16-bit byte offsets the plan counts with
+  if ((size_t)kRows * P.row_slot * es > 65535) return P;
+
+  // tables at the largest pitch first, repacked below
+  struct Full {
+    StageTab st;
+    ClsLink cls[kNG * kMaxLinks];
+  };
+  std::vector<uint8_t> out;
+  std::vector<size_t> at((size_t)ntiles * nstages + 1, 0);
+  out.reserve((size_t)ntiles * nstages * (sizeof(StageTab) + 18 * sizeof(ClsLink)));
+  int64_t zcap = 0;
+  size_t most = 0;
+  Full F;
+  for (int ti = 0; ti < ntiles; ++ti) {
+    const int t0 = ti * D, n = std::min(D, ntr - t0);
+    for (int s = 0; s < nstages; ++s) {
+      std::memset(&F, 0, sizeof F);
+      StageTab& st = F.st;
+      int32_t xmin = INT32_MAX;
+      for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
+        xmin = std::min(xmin, tab[(int64_t)t0 * cpad + c]);
+      st.xmin = xmin;
+      int words = 0, nl = 0;  // words and links of the groups before
       for (int gl = 0; gl < NG && s * NG + gl < ngroups; ++gl) {
         const int g = s * NG + gl;
-        GroupTab& gt = st.g[gl];
-        const int32_t* first = tab + (int64_t)t0 * cpad + kG * g;
         int b[kMaxTileTrials], cls_of[kMaxTileTrials];
         int32_t ckey[kMaxCls][kG];
-        int cmin[kMaxCls], cmax[kMaxCls];
-        int ncls = 0;
+        int cmin[kMaxCls], cmax[kMaxCls], csum[kMaxCls];
+        int ncls = 0, prev = 0, f0 = INT32_MAX;
+        const int nl0 = nl;
         for (int i = 0; i < n; ++i) {
           const int32_t* sv = tab + (int64_t)(t0 + i) * cpad + kG * g;
           b[i] = *std::min_element(sv, sv + kG);
+          f0 = std::min(f0, b[i]);
           int32_t key[kG];
+          int sum = 0;
           for (int q = 0; q < kG; ++q) {
             const int64_t r = (int64_t)sv[q] - b[i];
             if (r > 32767) return P;
             key[q] = (int32_t)r;
+            sum += (int)r;
           }
           int p = 0;
-          while (p < ncls && !std::equal(key, key + kG, ckey[p])) ++p;
+          while (p < ncls && !(csum[p] == sum && std::equal(key, key + kG, ckey[p]))) ++p;
           if (p == ncls) {
             if (ncls == kMaxCls) return P;
             std::copy(key, key + kG, ckey[ncls]);
             cmin[ncls] = cmax[ncls] = b[i];
+            csum[ncls] = sum;
             ++ncls;
           } else {
             cmin[p] = std::min(cmin[p], b[i]);
@@ -1118,55 +1163,73 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
           }
           cls_of[i] = p;
         }
-        int zoff[kMaxCls], zlens[kMaxCls];
-        for (int p = 0; p < ncls; ++p) {
-          const int zlen = (tt + cmax[p] - cmin[p] + 3) & ~3;
+        int order[kMaxCls], zoff[kMaxCls], zlens[kMaxCls], ulos[kMaxCls];
+        for (int p = 0; p < ncls; ++p) order[p] = p;
+        std::stable_sort(order, order + ncls, [&](int x, int y) { return csum[x] < csum[y]; });
+        for (int k = 0; k < ncls; ++k) {
+          const int p = order[k];
+          const int ulo = (cmin[p] - f0) / U;
+          if (ulo > 32767 || cmax[p] - f0 + tt > 65535) return P;
+          int un = (cmax[p] - f0 + tt + U - 1) / U - ulo;
+          if (u16) un += un & 1;  // 16-byte aligned classes
           zoff[p] = words;
-          ClsEntry& e = gt.cls[p];
-          for (int q = 0; q < kG; ++q) {
-            const int64_t rel = (int64_t)cmin[p] + ckey[p][q] - first[q];
-            if (rel < 0 || rel > 32767) return P;
-            e.rel[q] = (int16_t)rel;
+          zlens[p] = un * U;
+          ulos[p] = ulo;
+          int32_t key[kG];  // walks from the preceding class to this one
+          std::copy(ckey[k > 0 ? prev : p], ckey[k > 0 ? prev : p] + kG, key);
+          auto at_row = [&](int q, int r) {
+            return 8u * es * (uint32_t)((gl * kG + q) * P.row_slot + f0 + r - xmin);
+          };
+          int dist = 0;
+          for (int q = 0; q < kG; ++q) dist += std::abs(ckey[p][q] - key[q]);
+          if (k == 0 || dist > kMaxSteps || nl - nl0 + dist + ncls - k - 1 > kMaxLinks) {
+            std::copy(ckey[p], ckey[p] + kG, key);  // a chain starts here
+            for (int q = 0; q < kG; ++q) F.cls[nl].off[q] = at_row(q, key[q]);
+            ++nl;
           }
-          e.zoff = (int16_t)words;
-          e.zlen = (int16_t)zlen;
-          zlens[p] = zlen;
-          words += zlen;
+          for (int q = 0; q < kG; ++q)
+            while (key[q] != ckey[p][q]) {
+              const bool up = ckey[p][q] > key[q];
+              F.cls[nl].step = (up ? kStepAdd : kStepSub) | at_row(q, up ? key[q] : key[q] - 1);
+              key[q] += up ? 1 : -1;
+              for (int c = 0; c < kG; ++c) F.cls[nl].off[c] = at_row(c, key[c]);
+              ++nl;
+            }
+          ClsLink& e = F.cls[nl - 1];
+          e.ev = 4 * (words - ulo * U / 2);
+          e.od = e.ev + 2 * zlens[p];
+          e.range = (uint32_t)ulo | (uint32_t)un << 16;
+          prev = p;
+          words += zlens[p];
           if (words > 32767) return P;
         }
         for (int i = 0; i < n; ++i) {
-          const int p = cls_of[i], o = b[i] - cmin[p];
-          gt.zstart[trial_slot(i, nt / 32, D / (nt / 32))] =
+          const int p = cls_of[i], o = b[i] - f0 - ulos[p] * U;
+          st.zstart[gl][trial_slot(i, W, D / W)] =
               (int16_t)(zoff[p] + (o % 2) * (zlens[p] / 2) + o / 2);
         }
-        gt.ncls = ncls;
+        st.nlink[gl] = (uint8_t)(nl - nl0);
       }
-      if (!deal_work(st, U, u16 ? 32 : 31)) return P;
+      if (!deal_work(st, F.cls, W, cost)) return P;
       zcap = std::max<int64_t>(zcap, words);
+      const size_t bytes = sizeof(StageTab) + nl * sizeof(ClsLink);
+      most = std::max(most, bytes);
+      const size_t i = (size_t)ti * nstages + s;
+      at[i + 1] = at[i] + bytes;
+      out.insert(out.end(), (uint8_t*)&F, (uint8_t*)&F + bytes);
     }
   }
-  if (spread > 65536) return P;
-  const int SEG = kSegBytes / (u16 ? 2 : 1);
-  P.tt = tt;
-  P.trials = D;
-  P.threads = nt;
-  P.ctas = tile_ctas(D, tt, nt);
-  // staged row: the stage's window (span + tt samples) from up to SEG - 1 samples into its
-  // first segment, and 32 samples the word-wise build may read past the last word it uses
-  P.nseg = (int)((span + tt + 32 + 2 * SEG - 2) / SEG);
-  if (P.nseg > 255) return P;
-  P.row_slot = P.nseg * SEG;
   P.zcap = (int)((std::max<int64_t>(zcap, 4) + 3) / 4 * 4);
-  P.tab_bytes = out.size() * sizeof(StageTab);
+  P.tab_pitch = (int)most;
+  P.tab_bytes = most * ntiles * nstages;
   P.tabs.resize(P.tab_bytes);
-  std::memcpy(P.tabs.data(), out.data(), P.tab_bytes);
-  // addressing entries hold byte offsets within a stage buffer as uint16
-  if ((size_t)kRows * P.row_slot * (u16 ? 2 : 1) > 65535) return P;
+  for (size_t i = 0; i + 1 < at.size(); ++i)
+    std::memcpy(P.tabs.data() + i * most, out.data() + at[i], at[i + 1] - at[i]);
   // as many staging buffers as fit (4, else 3: a copy is then issued two stages ahead)
   const size_t limit = P.ctas == 2 ? kSmemLimit2 : kSmemLimit;
   for (int nst = kMaxNStage; nst >= 3 && !P.ok; --nst) {
     P.nstage = nst;
-    P.smem = smem_layout(u16 ? 2 : 1, 4, P.row_slot, P.zcap, nst).total;
+    P.smem = smem_layout(es, P.row_slot, P.zcap, P.tab_pitch, nst).total;
     P.ok = P.smem <= limit;
   }
   if (P.ok) tiled_smem_work(P, ntiles, nstages, ngroups, u16);
@@ -1187,30 +1250,36 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
   X(uint16_t, 1, 512, 4, 64, 512) X(uint16_t, 1, 512, 3, 64, 512)
 
 // Host: plan one range and verify the tables against the delay table they were built from,
-// independently of how they were built. Returns the number of violations of:
-//   - every trial's tt / 2 pair words lie inside one plane of its class, and the class word
-//     they stand for (o = 2 x plane position + plane) adds, in every channel of the group, the
-//     sample at the trial's own delay (rel + o);
-//   - class word ranges start and end on 16-byte boundaries;
+// independently of how they were built, by running the build's address arithmetic. Returns the
+// number of violations of:
 //   - the stage's copy start is the smallest first-trial delay of its rows, and every read of
 //     every trial stays inside the staged row;
-//   - the build work lists cover every block (31 units for uint8 data, 32 for uint16) of every
-//     class exactly once.
+//   - the tasks, run as the kernel runs them (a first link's row offsets, then the steps),
+//     visit links at exactly their own row offsets, and store every unit of every class
+//     exactly once; class word ranges are 16-byte aligned and do not overlap;
+//   - every trial's tt / 2 pair words lie inside one plane of a class of its group, and the frame
+//     word they stand for adds, in every channel of the group, the sample at the trial's delay;
+//   - a task's loads, phase included, end inside the CTA's shared memory.
 int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, int tt, int D,
                          int* ok) {
   const TiledPlan P = tiled_plan(tab, ntr, cpad, decimation, tt, D, kThreads);
   *ok = P.ok ? 1 : 0;
   if (!P.ok) return 0;
   const bool u16 = decimation > 1;
-  const int U = u16 ? 2 : 4, SEG = kSegBytes / (u16 ? 2 : 1), B = u16 ? 32 : 31;
+  const int U = u16 ? 2 : 4, es = u16 ? 2 : 1, SEG = kSegBytes / es;
   const int ngroups = cpad / kG, nstages = (ngroups + kNG - 1) / kNG;
   const int ntiles = (ntr + D - 1) / D;
-  const StageTab* tabs = reinterpret_cast<const StageTab*>(P.tabs.data());
-  int64_t bad = 0;
+  const SmemLayout L = smem_layout(es, P.row_slot, P.zcap, P.tab_pitch, P.nstage);
+  int64_t bad = (P.tab_pitch % 16) != 0;
+  bad += (int64_t)P.flush * kRows * 255 * decimation > 65535 || P.flush < 1;
   for (int ti = 0; ti < ntiles; ++ti) {
     const int t0 = ti * D, n = std::min(D, ntr - t0);
     for (int s = 0; s < nstages; ++s) {
-      const StageTab& st = tabs[(size_t)ti * nstages + s];
+      const uint8_t* tp = P.tabs.data() + ((size_t)ti * nstages + s) * P.tab_pitch;
+      const StageTab& st = *reinterpret_cast<const StageTab*>(tp);
+      const ClsLink* cls = reinterpret_cast<const ClsLink*>(tp + sizeof(StageTab));
+      const int ncls = st.nlink[0] + st.nlink[1];
+      bad += sizeof(StageTab) + ncls * sizeof(ClsLink) > (size_t)P.tab_pitch;
       int32_t xmin = INT32_MAX;
       for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
         xmin = std::min(xmin, tab[(int64_t)t0 * cpad + c]);
@@ -1218,65 +1287,93 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
       for (int t = t0; t < t0 + n; ++t)
         for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
           bad += (int64_t)tab[(int64_t)t * cpad + c] - xmin + tt + 32 + SEG - 1 > P.row_slot;
-      std::vector<int> covered;  // blocks of every (group, class), in order
-      std::vector<int> first_block(kNG * kMaxCls + 1, 0);
-      for (int gl = 0; gl < kNG; ++gl)
-        for (int p = 0; p < kMaxCls; ++p) {
-          const int nb = p < st.g[gl].ncls ? (st.g[gl].cls[p].zlen / U + B - 1) / B : 0;
-          first_block[gl * kMaxCls + p + 1] = first_block[gl * kMaxCls + p] + nb;
+      std::vector<std::vector<int>> stored(ncls);  // units of each class, times stored
+      std::vector<int> words(P.zcap, 0);           // classes holding each word
+      for (int p = 0; p < ncls; ++p) {
+        stored[p].assign(cls[p].un(), 0);
+        const int z0 = cls[p].ev / 4 + (int)cls[p].ulo() * U / 2, zlen = (int)cls[p].un() * U;
+        if (zlen == 0) continue;  // a step between classes
+        bad += z0 % 4 != 0 || zlen % 4 != 0 || cls[p].od != cls[p].ev + 2 * zlen;
+        if (z0 < 0 || z0 + zlen > P.zcap) {
+          ++bad;
+          continue;
         }
-      covered.assign(first_block.back(), 0);
-      for (int w = 0; w < kWarps; ++w)
-        for (int k = 0; k < st.nwork[w]; ++k) {
-          const uint32_t wk = st.work[w][k];
-          const int gl = (int)((wk >> 4) & 1), p = (int)(wk & 15);
-          const int b0 = (int)((wk >> 8) & 255), nb = (int)(wk >> 16);
-          for (int b = b0; b < b0 + nb; ++b) {
-            const int idx = first_block[gl * kMaxCls + p] + b;
-            if (p >= st.g[gl].ncls || idx >= first_block[gl * kMaxCls + p + 1]) {
-              ++bad;
-            } else {
-              ++covered[idx];
-            }
+        for (int v = z0; v < z0 + zlen; ++v) bad += words[v]++ != 0;
+      }
+      for (int w = 0, t = 0; w < kWarps; ++w) {  // the warps' tasks follow one another
+        bad += (st.wtask[w] >> 8) && (st.wtask[w] & 255) != t;
+        t += st.wtask[w] >> 8;
+      }
+      for (int w = kWarps; w < kMaxWarps; ++w) bad += st.wtask[w] != 0;
+      bad += stage_tasks(st) > kMaxTasks;
+      for (int t = 0; t < std::min(stage_tasks(st), kMaxTasks); ++t) {
+        const int p0 = st.task[t] & 63, np = ((st.task[t] >> 6) & 15) + 1, b = st.task[t] >> 10;
+        const int gl = p0 >= st.nlink[0];
+        if (p0 + np > (gl ? ncls : (int)st.nlink[0])) {
+          ++bad;
+          continue;
+        }
+        uint32_t off[kG];
+        std::copy(cls[p0].off, cls[p0].off + kG, off);
+        for (int p = p0; p < p0 + np; ++p) {
+          if (p > p0) {
+            const uint32_t sw = cls[p].step, at = sw & kStepOff;
+            const bool up = (sw & ~kStepOff) == kStepAdd;
+            bad += !up && (sw & ~kStepOff) != kStepSub;
+            int hit = 0;
+            for (int q = 0; q < kG && !hit; ++q)
+              if (off[q] == (up ? at : at + 8u * es)) {
+                off[q] = up ? at + 8u * es : at;
+                ++hit;
+              }
+            bad += hit != 1;
           }
+          bad += !std::equal(off, off + kG, cls[p].off);
+          for (int l = 0; l < kBlock; ++l) {
+            const int v = b * kBlock + l - (int)cls[p].ulo();
+            if (v >= 0 && v < (int)cls[p].un()) bad += stored[p][v]++ != 0;
+          }
+          // lane 31's second row word at the largest phase
+          for (int q = 0; q < kG; ++q)
+            bad += L.raw + (size_t)(P.nstage - 1) * kRows * P.row_slot * es +
+                       4u * (uint32_t)(b * kBlock + 31) + cls[p].off[q] / 8 + (SEG - 1) * es + 8 >
+                   L.total;
         }
-      for (int v : covered) bad += v != 1;
+      }
+      for (const auto& v : stored)
+        for (int k : v) bad += k != 1;
+      int p1 = 0;
       for (int gl = 0; gl < kNG && s * kNG + gl < ngroups; ++gl) {
-        const GroupTab& gt = st.g[gl];
-        const int c0 = (s * kNG + gl) * kG;
-        for (int p = 0; p < gt.ncls; ++p) bad += (gt.cls[p].zoff % 4) + (gt.cls[p].zlen % 4) != 0;
+        const int c0 = (s * kNG + gl) * kG, g0 = p1;
+        p1 += st.nlink[gl];
         for (int i = 0; i < n; ++i) {
-          const int z = gt.zstart[trial_slot(i, kWarps, D / kWarps)];
-          int p = 0, o = -1;
-          for (; p < gt.ncls; ++p) {
-            const int zo = gt.cls[p].zoff, half = gt.cls[p].zlen / 2;
+          const int z = st.zstart[gl][trial_slot(i, kWarps, D / kWarps)];
+          int p = g0, v = -1;
+          for (; p < p1; ++p) {
+            const int zo = cls[p].ev / 4 + (int)cls[p].ulo() * U / 2;
+            const int half = (int)cls[p].un() * U / 2;
             if (zo <= z && z + tt / 2 <= zo + half) {
-              o = 2 * (z - zo);  // even plane
+              v = (int)cls[p].ulo() * U + 2 * (z - zo);  // even plane
               break;
             }
             if (zo + half <= z && z + tt / 2 <= zo + 2 * half) {
-              o = 2 * (z - zo - half) + 1;  // odd plane
+              v = (int)cls[p].ulo() * U + 2 * (z - zo - half) + 1;  // odd plane
               break;
             }
           }
-          if (p == gt.ncls) {
+          if (p == p1) {
             ++bad;
             continue;
           }
-          for (int q = 0; q < kG; ++q) {
-            const int64_t want = (int64_t)tab[(int64_t)(t0 + i) * cpad + c0 + q] -
-                                 tab[(int64_t)t0 * cpad + c0 + q];
-            bad += (int64_t)gt.cls[p].rel[q] + o != want;
-          }
+          for (int q = 0; q < kG; ++q)
+            bad += (int64_t)cls[p].off[q] / (8 * es) + v !=
+                   (int64_t)(gl * kG + q) * P.row_slot +
+                       tab[(int64_t)(t0 + i) * cpad + c0 + q] - xmin;
         }
       }
     }
   }
   return bad;
-}
-
-size_t tiled_smem_bytes(int is_u16, int row_slot, int zcap, int nstage) {
-  return smem_layout(is_u16 ? 2 : 1, 4, row_slot, zcap, nstage).total;
 }
 
 cudaError_t launch_tiled_persistent(const PersistArgs& p, int is_u16, int tt, int nstage, int D,
@@ -1344,9 +1441,9 @@ cudaError_t make_ring_map(CUtensorMap* map, const void* ring, int is_u16, int64_
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-bool fused_smem(int is_u16, int row_slot, int zcap, int nstage, int hp, int32_t* e_off,
-                size_t* smem) {
-  const SmemLayout L = smem_layout(is_u16 ? 2 : 1, 4, row_slot, zcap, nstage);
+bool fused_smem(int is_u16, int row_slot, int zcap, int pitch, int nstage, int hp,
+                int32_t* e_off, size_t* smem) {
+  const SmemLayout L = smem_layout(is_u16 ? 2 : 1, row_slot, zcap, pitch, nstage);
   const size_t rows = (size_t)kWarps * (hp + 512) * sizeof(uint32_t);
   size_t total = L.total, off = L.raw;
   if (L.tab - L.raw < rows) {  // the staging area is too small: the rows go after it

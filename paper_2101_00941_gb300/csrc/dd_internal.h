@@ -98,6 +98,8 @@ struct TiledArgs {
   int32_t row_slot;        // elements per staged channel row
   int32_t zcap;            // pair words per stage buffer
   int32_t nstage;          // staging buffers (3 or 4)
+  int32_t tab_pitch;       // bytes of one class table (a multiple of 16)
+  int32_t flush;           // stages whose sums fit the packed 16-bit lanes: 65535 / (16 * 255 * d)
   const uint8_t* tabs;     // delay-class tables of the range, one per (trial tile, stage)
   int32_t* err;            // bit 0: a bounded wait ran out
   CUtensorMap rows;        // the ring as [Cp][xd_stride / seg][seg] (make_ring_map)
@@ -170,13 +172,15 @@ struct TiledPlan {
   int nstage = 0;          // staging buffers
   int row_slot = 0;
   int zcap = 0;
+  int tab_pitch = 0;
+  int flush = 0;
   size_t smem = 0;
   size_t tab_bytes = 0;
   std::vector<uint8_t> tabs;
   // Shared-memory work of one row of time tiles (every trial tile of the range, TT outputs),
   // counted from the tables as the kernel issues it: warp-wide shared-memory instructions
   // (wavefronts of the LSU data pipe: accumulation loads, pair-word build loads and stores,
-  // table reads, addressing stores) and the bytes the tensor and bulk copies write.
+  // table reads) and the bytes the tensor and bulk copies write.
   int64_t lsu_wavefronts = 0;
   int64_t copy_bytes = 0;
 };
@@ -196,12 +200,11 @@ cudaError_t launch_tiled(const TiledArgs& a, int is_u16, int tt, int trials, int
 cudaError_t launch_tiled_persistent(const PersistArgs& p, int is_u16, int tt, int nstage,
                                     int trials, int threads, size_t smem, int ctas,
                                     cudaStream_t st);
-size_t tiled_smem_bytes(int is_u16, int row_slot, int zcap, int nstage);
 // Fused search (64 x 512 x 512 instances): where the per-warp prefix-sum rows go in shared
 // memory (inside the staging area when it is large enough, else after it) and the launch's
 // dynamic shared memory; false if that exceeds what a CTA may plan for.
-bool fused_smem(int is_u16, int row_slot, int zcap, int nstage, int hp, int32_t* e_off,
-                size_t* smem);
+bool fused_smem(int is_u16, int row_slot, int zcap, int pitch, int nstage, int hp,
+                int32_t* e_off, size_t* smem);
 cudaError_t prepare_fused(int is_u16, int nstage, size_t smem);
 // Time segments of a fused launch: minimises (waves of one CTA per SM) x (tiles per segment)
 // for ntx trial tiles and ntt time tiles, at most smax segments.
