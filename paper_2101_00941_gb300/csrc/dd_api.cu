@@ -1289,6 +1289,7 @@ int sps_run_ex(dd_plan_t p, const int32_t* widths, int32_t nwidths, float thresh
       c.hist = a.hist;
       c.iters = how->clip_iters;
       c.kappa = how->clip_kappa;
+      c.vmax = (uint32_t)p->C * 255u * (uint32_t)d;
       c.out = s.wst + (int64_t)p->row0[r] * ddk::kMaxWidths;
       DD_CK(ddk::launch_clip_stats(c, st));
       p->launches += 1;

@@ -38,6 +38,7 @@ struct ClipArgs {
   int32_t hist;            // largest decimated width - 1, rounded up to 256
   int32_t iters;           // clipping steps
   double kappa;            // clipping bound in deviations
+  uint32_t vmax;           // the largest series value possible (nchans * 255 * d)
   WidthStats* out;         // [n_trials][nw]
 };
 

@@ -75,11 +75,16 @@ cudaError_t launch_shift_table(const double* freqs, int32_t nchans, int32_t cpad
 
 // ------------------------------------------------------------------ corner turn
 
-// 64 samples x 64 channels per CTA. 16-byte loads of spectra into shared memory, a 4x4 byte
-// transpose in registers (PRMT), 4-byte stores of channel rows.
-__global__ void __launch_bounds__(256) k_corner_turn16(const uint8_t* __restrict__ in, int64_t n,
-                                                       int32_t nchans, uint8_t* __restrict__ ring,
-                                                       int64_t stride, int64_t col0) {
+// 64 samples x 64 channels per CTA: 16 channels of one spectrum per thread into shared memory, a
+// 4x4 byte transpose in registers (PRMT), 4-byte stores of channel rows. ALIGNED: every spectrum
+// starts 16-byte aligned (nchans a multiple of 16), one 16-byte load per thread. Otherwise five
+// aligned words and funnel shifts, or single bytes where a word would leave the chunk. Bound by
+// memory; one byte per thread, which any layout took before, wrote single bytes a row apart
+// (1001 channels x 49984 samples, with the other small launches: 3.7 -> 3.0 ms a chunk).
+template <bool ALIGNED>
+__global__ void __launch_bounds__(256) k_corner_turn(const uint8_t* __restrict__ in, int64_t n,
+                                                     int32_t nchans, uint8_t* __restrict__ ring,
+                                                     int64_t stride, int64_t col0) {
   __shared__ uint32_t S[64][17];
   const int tid = threadIdx.x;
   const int64_t t0 = (int64_t)blockIdx.x * 64;
@@ -89,7 +94,30 @@ __global__ void __launch_bounds__(256) k_corner_turn16(const uint8_t* __restrict
     const int64_t t = t0 + r;
     const int32_t c = c0 + 16 * q;
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (t < n && c < nchans) v = __ldg(reinterpret_cast<const uint4*>(in + t * nchans + c));
+    if (t < n && c < nchans) {
+      if (ALIGNED) {
+        v = __ldg(reinterpret_cast<const uint4*>(in + t * nchans + c));
+      } else {
+        const uint8_t* p = in + t * nchans + c;
+        const uint32_t ph = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3);
+        const uint8_t* w = p - ph;
+        if (w >= in && w + 20 <= in + n * nchans) {
+          const uint32_t* x = reinterpret_cast<const uint32_t*>(w);
+          const uint32_t x0 = __ldg(x), x1 = __ldg(x + 1), x2 = __ldg(x + 2), x3 = __ldg(x + 3),
+                         x4 = __ldg(x + 4);
+          v.x = __funnelshift_r(x0, x1, 8 * ph);
+          v.y = __funnelshift_r(x1, x2, 8 * ph);
+          v.z = __funnelshift_r(x2, x3, 8 * ph);
+          v.w = __funnelshift_r(x3, x4, 8 * ph);
+        } else {
+          uint32_t o[4] = {0, 0, 0, 0};
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            if (c + k < nchans) o[k / 4] |= (uint32_t)p[k] << (8 * (k % 4));
+          v = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+      }
+    }
     S[r][4 * q + 0] = v.x;
     S[r][4 * q + 1] = v.y;
     S[r][4 * q + 2] = v.z;
@@ -116,31 +144,17 @@ __global__ void __launch_bounds__(256) k_corner_turn16(const uint8_t* __restrict
   }
 }
 
-// Any channel count / alignment: one byte per thread.
-__global__ void k_corner_turn1(const uint8_t* __restrict__ in, int64_t n, int32_t nchans,
-                               uint8_t* __restrict__ ring, int64_t stride, int64_t col0) {
-  const int64_t total = n * nchans;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = e / nchans;
-    const int32_t c = (int32_t)(e - t * nchans);
-    ring[(int64_t)c * stride + col0 + t] = in[e];
-  }
-}
-
+// The ring's rows and the column of the first sample are 4-byte aligned (both 256-byte aligned
+// in every plan); the last word of a chunk may write up to 3 zeros past it, into row slack.
 cudaError_t launch_corner_turn(const uint8_t* in, int64_t n, int32_t nchans, uint8_t* ring,
                                int64_t ring_stride, int64_t col0, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const bool fast = (nchans % 16 == 0) && (((uintptr_t)in & 15) == 0) && (ring_stride % 4 == 0) &&
-                    (col0 % 4 == 0) && (((uintptr_t)ring & 3) == 0);
-  if (fast) {
-    dim3 grid((unsigned)((n + 63) / 64), (unsigned)((nchans + 63) / 64));
-    k_corner_turn16<<<grid, 256, 0, st>>>(in, n, nchans, ring, ring_stride, col0);
-  } else {
-    int64_t blocks = (n * nchans + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
-    k_corner_turn1<<<(unsigned)blocks, 256, 0, st>>>(in, n, nchans, ring, ring_stride, col0);
-  }
+  if (ring_stride % 4 || col0 % 4 || ((uintptr_t)ring & 3)) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)((n + 63) / 64), (unsigned)((nchans + 63) / 64));
+  if (nchans % 16 == 0 && ((uintptr_t)in & 15) == 0)
+    k_corner_turn<true><<<grid, 256, 0, st>>>(in, n, nchans, ring, ring_stride, col0);
+  else
+    k_corner_turn<false><<<grid, 256, 0, st>>>(in, n, nchans, ring, ring_stride, col0);
   return cudaGetLastError();
 }
 
@@ -344,17 +358,36 @@ __device__ __forceinline__ U128 add128(U128 a, U128 b) {
   return r;
 }
 
+// One CTA per trial; 16-byte loads, four in flight per thread (one int a load when the row is not
+// 16-byte aligned). The squares of two int32 values sum below 2^64 before the 128-bit add.
 __global__ void __launch_bounds__(256) k_moments(const int32_t* __restrict__ y, int64_t n,
                                                  int64_t stride, Moments* __restrict__ mom) {
   const int32_t i = blockIdx.x;
   const int32_t* yi = y + (int64_t)i * stride;
   unsigned long long s1 = 0;
   U128 s2 = {0, 0};
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-    const int64_t v = yi[j];
-    s1 += (unsigned long long)v;
-    s2 = add128(s2, U128{(unsigned long long)(v * v), 0});
+  auto add2 = [&](int32_t p, int32_t q) {
+    s1 += (unsigned long long)((int64_t)p + q);
+    s2 = add128(s2, U128{(unsigned long long)((int64_t)p * p) + (unsigned long long)((int64_t)q * q), 0});
+  };
+  int64_t j = 0;  // the first sample left to the one-int loop
+  if ((reinterpret_cast<uintptr_t>(yi) & 15) == 0) {
+    const int4* v = reinterpret_cast<const int4*>(yi);
+    const int64_t n4 = n / 4;
+    int64_t k = threadIdx.x;
+    for (; k + 768 < n4; k += 1024) {
+      const int4 a = __ldg(v + k), b = __ldg(v + k + 256), c = __ldg(v + k + 512),
+                 d = __ldg(v + k + 768);
+      add2(a.x, a.y), add2(a.z, a.w), add2(b.x, b.y), add2(b.z, b.w);
+      add2(c.x, c.y), add2(c.z, c.w), add2(d.x, d.y), add2(d.z, d.w);
+    }
+    for (; k < n4; k += 256) {
+      const int4 a = __ldg(v + k);
+      add2(a.x, a.y), add2(a.z, a.w);
+    }
+    j = 4 * n4;
   }
+  for (j += threadIdx.x; j < n; j += blockDim.x) add2(__ldg(yi + j), 0);
   __shared__ unsigned long long sh[3][8];
   for (int off = 16; off > 0; off >>= 1) {
     s1 += __shfl_xor_sync(0xffffffffu, s1, off);
@@ -435,20 +468,25 @@ __device__ __forceinline__ uint32_t window_bound(int w, long long s1, double thr
 }
 
 constexpr int kSpsThreads = 256;
-constexpr int kSpsSeg = kSpsThreads * 16;         // window samples per pass (16 per thread)
+constexpr int kSpsWarps = kSpsThreads / 32;
+constexpr int kSpsPass = 512;                     // window samples per warp and pass
 constexpr int kSpsPad = 3;                        // aligns P[1 + hist + 4k] to 16 bytes
 
-// Exact argmax over the block: largest v among valid lanes, ties to the lowest lane. Returns
-// -1 when the block has no valid lane; `off` = lane offset within the block.
-__device__ __forceinline__ int block_argmax(uint32_t v, bool valid, int B, int lane, int& off) {
-  unsigned long long key =
-      valid ? (((unsigned long long)v << 32) | (0xFFFFFFFFu - (uint32_t)(lane & (B - 1)))) : 0ull;
-  for (int o = B >> 1; o > 0; o >>= 1) {
-    const unsigned long long t = __shfl_xor_sync(0xffffffffu, key, o);
-    key = t > key ? t : key;
+// Exact argmax over the block of B lanes: the largest v among its valid lanes and its lowest lane
+// (`off`, within the block); false when the block has no valid lane.
+__device__ __forceinline__ bool block_argmax(uint32_t v, bool valid, int B, int lane,
+                                             uint32_t& best, int& off) {
+  uint32_t mx = valid ? v : 0u;
+  if (B == 32) {
+    mx = __reduce_max_sync(0xffffffffu, mx);
+  } else {
+    for (int o = B >> 1; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
-  off = key ? (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFu)) : 0;
-  return key ? (int)(key >> 32) : -1;
+  const uint32_t bm = B == 32 ? 0xffffffffu : ((1u << B) - 1u);
+  const uint32_t at = (__ballot_sync(0xffffffffu, valid && v == mx) >> (lane & ~(B - 1))) & bm;
+  best = mx;
+  off = __ffs(at) - 1;
+  return at != 0;
 }
 
 // Prefix sums through window samples q - w .. q + 3 - w of the pass, i.e. entries
@@ -466,80 +504,132 @@ __device__ __forceinline__ uint4 prefix4(const uint32_t* P, int idx, int w) {
   return make_uint4(a.w, b.x, b.y, b.z);
 }
 
-// One pass of the search kernels over window samples seg0 .. seg0 + kSpsSeg - 1 of series yi
-// (zero past n): this lane's four 4-sample chunks (samples seg0 + q0 + 128 g + e) are loaded and
-// turned into uint32 prefix sums continuing from P[H] (the sum through the sample before the
-// pass), returned in v and stored to P[1 + H + q]. Two CTA barriers; P[0 .. H] must be in place.
-__device__ __forceinline__ void sps_pass_prefix(const int32_t* __restrict__ yi, bool vec,
-                                                long long n, long long seg0, int q0, int lane,
-                                                int wid, int H, uint32_t* P, uint32_t* warp_tot,
-                                                uint32_t (&v)[4][4]) {
-#pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    const long long j = seg0 + q0 + 128 * g;
-    if (vec && j + 4 <= n) {
-      const int4 t = __ldg(reinterpret_cast<const int4*>(yi + j));
-      v[g][0] = (uint32_t)t.x;
-      v[g][1] = (uint32_t)t.y;
-      v[g][2] = (uint32_t)t.z;
-      v[g][3] = (uint32_t)t.w;
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) v[g][e] = (j + e < n) ? (uint32_t)__ldg(yi + j + e) : 0u;
+// A warp's view of one series. The search kernels give each warp a segment of consecutive
+// samples of one trial, taken in passes of kSpsPass samples: lane l owns the 4-sample chunks
+// 4l + 128 g (g = 0..3) of the pass. The warp's own shared-memory row P holds uint32 prefix sums
+// of the pass and of the H samples before it (entry 1 + H + q = sum through sample q of the pass;
+// the sums wrap, but every boxcar sum is < 2^31, so the difference of two prefixes is exact). The
+// history is built once per segment from the H samples before it and then carried from pass to
+// pass, so warps never wait for one another: against one CTA per trial with four barriers per
+// 4096-sample pass, a warp's loads of the next pass overlap this pass's boxcars, and a trial's
+// window spreads over as many warps as the chip has room for.
+struct SpsRow {
+  const int32_t* y;
+  uint32_t* P;
+  long long n;
+  int H, lane;
+  bool vec;
+
+  // chunk at sample j: zero outside the window
+  __device__ __forceinline__ uint4 load(long long j) const {
+    if (vec && j >= 0 && j + 4 <= n) {
+      const int4 t = __ldg(reinterpret_cast<const int4*>(y + j));
+      return make_uint4((uint32_t)t.x, (uint32_t)t.y, (uint32_t)t.z, (uint32_t)t.w);
     }
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (j >= 0 && j < n) v.x = (uint32_t)__ldg(y + j);
+    if (j + 1 >= 0 && j + 1 < n) v.y = (uint32_t)__ldg(y + j + 1);
+    if (j + 2 >= 0 && j + 2 < n) v.z = (uint32_t)__ldg(y + j + 2);
+    if (j + 3 >= 0 && j + 3 < n) v.w = (uint32_t)__ldg(y + j + 3);
+    return v;
   }
-  uint32_t run = 0;  // sum of this warp's chunks before the current one (lanes, then g)
+  // inclusive prefix sums of G x 128 samples in place, continuing from `run`; returns the sum
+  // through their last sample
+  template <int G>
+  __device__ __forceinline__ uint32_t scan(uint4 (&v)[G], uint32_t run) const {
+    uint32_t incl[G];
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    v[g][1] += v[g][0];
-    v[g][2] += v[g][1];
-    v[g][3] += v[g][2];
-    uint32_t incl = v[g][3];
+    for (int g = 0; g < G; ++g) {
+      v[g].y += v[g].x;
+      v[g].z += v[g].y;
+      v[g].w += v[g].z;
+      incl[g] = v[g].w;
+    }
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += o;
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, incl[g], off);
+        if (lane >= off) incl[g] += o;
+      }
     }
-    const uint32_t pre = run + incl - v[g][3];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) v[g][e] += pre;
-    run += __shfl_sync(0xffffffffu, incl, 31);
+    for (int g = 0; g < G; ++g) {
+      const uint32_t pre = run + incl[g] - v[g].w;
+      run += __shfl_sync(0xffffffffu, incl[g], 31);
+      v[g].x += pre;
+      v[g].y += pre;
+      v[g].z += pre;
+      v[g].w += pre;
+    }
+    return run;
   }
-  if (lane == 0) warp_tot[wid] = run;
-  __syncthreads();  // warp totals; the history entries P[0 .. H] of this pass
-  uint32_t base = P[H];  // sum through the sample before the pass
-  for (int k = 0; k < wid; ++k) base += warp_tot[k];
-#pragma unroll
-  for (int g = 0; g < 4; ++g) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) v[g][e] += base;  // now prefix sums through each sample
-    *reinterpret_cast<uint4*>(P + 1 + H + q0 + 128 * g) =
-        make_uint4(v[g][0], v[g][1], v[g][2], v[g][3]);
+  // P[0 .. H] for a segment starting at sample s0; returns P[H]
+  __device__ __forceinline__ uint32_t history(long long s0) const {
+    if (lane == 0) P[0] = 0;
+    uint32_t run = 0;
+    for (int q = 0; q < H; q += 256) {
+      uint4 v[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+      if (s0 > 0) {  // before the window every sample is zero
+        v[0] = load(s0 - H + q + 4 * lane);
+        v[1] = load(s0 - H + q + 128 + 4 * lane);
+        run = scan(v, run);
+      }
+      *reinterpret_cast<uint4*>(P + 1 + q + 4 * lane) = v[0];
+      *reinterpret_cast<uint4*>(P + 1 + q + 128 + 4 * lane) = v[1];
+    }
+    return run;
   }
-  __syncthreads();  // the pass's prefix sums
+  __device__ __forceinline__ void load_pass(long long j0, uint4 (&v)[4]) const {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) v[g] = load(j0 + 4 * lane + 128 * g);
+  }
+  __device__ __forceinline__ void store_pass(const uint4 (&v)[4]) const {
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+      *reinterpret_cast<uint4*>(P + 1 + H + 4 * lane + 128 * g) = v[g];
+  }
+  // the last H + 1 entries become the next pass's history
+  __device__ __forceinline__ void carry() const {
+    if (lane == 0) P[0] = P[kSpsPass];
+    for (int q = 0; q < H; q += 128) {
+      const uint4 t = *reinterpret_cast<const uint4*>(P + 1 + kSpsPass + q + 4 * lane);
+      *reinterpret_cast<uint4*>(P + 1 + q + 4 * lane) = t;
+      __syncwarp();  // at H > 512 a later read lies where an earlier write went
+    }
+    __syncwarp();
+  }
+};
+
+__host__ __device__ constexpr int sps_row_words(int hist) { return kSpsPad + 1 + hist + kSpsPass; }
+
+// Samples of a warp's segment: 8 passes (their history re-read is 6% at H = 256), 16 with wide
+// boxcars (H >= 512), fewer while the launch has less than 24 warps per SM and a segment stays
+// at least four times its history.
+inline int64_t sps_segment(int n_trials, int64_t n, int hist) {
+  int64_t seg = kSpsPass * (hist >= 512 ? 16 : 8);
+  while (seg > 2 * kSpsPass && seg / 2 >= 4 * hist &&
+         n_trials * ((n + seg - 1) / seg) < 152 * 24)
+    seg /= 2;
+  while ((n + seg * kSpsWarps - 1) / (seg * kSpsWarps) > 65535) seg *= 2;  // grid rows
+  return seg;
 }
 
-// One CTA per trial; passes of kSpsSeg window samples. Warp v owns pass samples
-// 512v .. 512v + 511, lane l the 4-sample chunks 512v + 128g + 4l (g = 0..3). P holds uint32
-// prefix sums of the pass and of the H samples before it (entry 1 + H + q = sum through window
-// sample seg0 + q; the sums wrap, but every boxcar sum is < 2^31, so the difference of two
-// prefixes is exact). The history part is carried over from the previous pass in shared memory.
-// Every boxcar sum is compared with an integer bound per width below which the SNR cannot reach
-// the threshold; a 32-sample group where one passes is searched exactly by its warp (lane =
-// sample): per width the group's largest boxcar sum (earliest sample) per peak block, then the
-// FP64 SNRs in the oracle's evaluation order.
-__global__ void __launch_bounds__(kSpsThreads) k_sps(const SpsArgs a) {
+// CTA (trial, 8 segments): warp v takes segment 8 * blockIdx.y + v. Every boxcar sum is compared
+// with an integer bound per width below which the SNR cannot reach the threshold; a 32-sample
+// group where one passes is searched exactly by its warp (lane = sample): per width the group's
+// largest boxcar sum (earliest sample) per peak block, then the FP64 SNRs in the oracle's
+// evaluation order. Bound by instruction issue in the filter (one aligned 16-byte prefix load,
+// four subtractions, a three-way maximum and a compare per four boxcar sums).
+__global__ void __launch_bounds__(kSpsThreads, 3) k_sps(const SpsArgs a, const long long seg) {
   extern __shared__ __align__(16) uint32_t Ps[];
-  uint32_t* P = Ps + kSpsPad;  // [1 + hist + kSpsSeg]
   __shared__ double den[kMaxWidths];
   __shared__ long long ca[kMaxWidths], cb[kMaxWidths];
   __shared__ uint32_t bthr[kMaxWidths];
-  __shared__ uint32_t warp_tot[kSpsThreads / 32];
 
   const int32_t i = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const long long n = a.n;
-  if (n <= 0) return;
   const double thr = (double)a.threshold;
   // Per width k: SNR = (ca[k] * B - cb[k]) / den[k]. Window statistics: ca = n, cb = w * S1,
   // den = sqrt(w) * sqrt(n * S2 - S1^2). Clipped per-width statistics (a.wst): ca = N_k,
@@ -574,46 +664,69 @@ __global__ void __launch_bounds__(kSpsThreads) k_sps(const SpsArgs a) {
     bthr[tid] = !live ? 0xFFFFFFFFu
                       : (tl <= 0.0 ? 0u : (tl >= 4294967295.0 ? 0xFFFFFFFFu : (uint32_t)floor(tl)));
   }
-  const int H = a.hist;
-  const int nw = a.nw;
+  __syncthreads();  // the only CTA barrier: the widths' statistics
+  const long long s0 = ((long long)blockIdx.y * kSpsWarps + wid) * seg;
+  if (s0 >= n) return;
+  const long long s1 = s0 + seg < n ? s0 + seg : n;
+  const int H = a.hist, nw = a.nw;
   const int wmax = a.wd[nw - 1];
-  const int32_t* yi = a.y + (int64_t)i * a.stride;
-  const bool vec = (reinterpret_cast<uintptr_t>(yi) & 15) == 0;
   const int B = a.block;
-  const int q0 = wid * 512 + 4 * lane;  // pass sample of this lane's chunk g = 0
-  // samples before the window are zero: the history of the first pass is all zero
-  for (int k = tid; k <= H; k += kSpsThreads) P[k] = 0;
+  SpsRow R;
+  R.y = a.y + (int64_t)i * a.stride;
+  R.P = Ps + (size_t)wid * sps_row_words(H) + kSpsPad;
+  R.n = n;
+  R.H = H;
+  R.lane = lane;
+  R.vec = (reinterpret_cast<uintptr_t>(R.y) & 15) == 0;
+  const uint32_t* P = R.P;
 
-  for (long long seg0 = 0; seg0 < n; seg0 += kSpsSeg) {
-    uint32_t v[4][4];
-    sps_pass_prefix(yi, vec, n, seg0, q0, lane, wid, H, P, warp_tot, v);
+  uint4 nv[4];
+  R.load_pass(s0, nv);
+  uint32_t run = R.history(s0);
+  for (long long j0 = s0; j0 < s1; j0 += kSpsPass) {
+    uint4 v[4] = {nv[0], nv[1], nv[2], nv[3]};
+    run = R.scan(v, run);
+    R.store_pass(v);
+    __syncwarp();
+    if (j0 + kSpsPass < s1) R.load_pass(j0 + kSpsPass, nv);  // in flight during the boxcars
 
     // ---- filter: every boxcar sum of this lane's samples against the bounds
-    const long long wj0 = seg0 + wid * 512;  // the warp's first sample
-    const bool interior = wj0 >= wmax - 1 && wj0 + 512 <= n;  // every (sample, width) valid
-    unsigned groups = 0;  // 32-sample groups of the warp's 512 samples with a passing sum
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const int idx = 1 + H + q0 + 128 * g;  // entry of this chunk's first sample
-      const long long j = seg0 + q0 + 128 * g;
-      bool hot = false;
-#pragma unroll
-      for (int k = 0; k < kMaxWidths; ++k) {
-        if (k >= nw) break;
+    const bool interior = j0 >= wmax - 1 && j0 + kSpsPass <= n;  // every (sample, width) valid
+    bool hot[4] = {false, false, false, false};
+    if (interior) {
+#pragma unroll 1
+      for (int k = 0; k < nw; ++k) {
         const int w = a.wd[k];
-        const uint4 st = prefix4(P, idx, w);
-        const uint32_t b0 = v[g][0] - st.x, b1 = v[g][1] - st.y;
-        const uint32_t b2 = v[g][2] - st.z, b3 = v[g][3] - st.w;
         const uint32_t t = bthr[k];
-        if (interior) {
-          hot |= (b0 >= t) | (b1 >= t) | (b2 >= t) | (b3 >= t);
-        } else {
-          hot |= (j < n && j >= w - 1 && b0 >= t) | (j + 1 < n && j + 1 >= w - 1 && b1 >= t) |
-                 (j + 2 < n && j + 2 >= w - 1 && b2 >= t) | (j + 3 < n && j + 3 >= w - 1 && b3 >= t);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const uint4 st = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
+          const uint32_t mx = max(max(v[g].x - st.x, v[g].y - st.y),
+                                  max(v[g].z - st.z, v[g].w - st.w));
+          hot[g] |= mx >= t;
         }
       }
-      // lanes 8c .. 8c + 7 of chunk row g cover the warp's 32-sample group 4g + c
-      const unsigned hm = __ballot_sync(0xffffffffu, hot);
+    } else {
+#pragma unroll 1
+      for (int k = 0; k < nw; ++k) {
+        const int w = a.wd[k];
+        const uint32_t t = bthr[k];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const uint4 st = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
+          const long long j = j0 + 4 * lane + 128 * g;
+          hot[g] |= (j < n && j >= w - 1 && v[g].x - st.x >= t) |
+                    (j + 1 < n && j + 1 >= w - 1 && v[g].y - st.y >= t) |
+                    (j + 2 < n && j + 2 >= w - 1 && v[g].z - st.z >= t) |
+                    (j + 3 < n && j + 3 >= w - 1 && v[g].w - st.w >= t);
+        }
+      }
+    }
+    // lanes 8c .. 8c + 7 of chunk row g cover the pass's 32-sample group 4g + c
+    unsigned groups = 0;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const unsigned hm = __ballot_sync(0xffffffffu, hot[g]);
 #pragma unroll
       for (int c = 0; c < 4; ++c) groups |= ((hm >> (8 * c)) & 0xFFu) ? (1u << (4 * g + c)) : 0u;
     }
@@ -622,29 +735,68 @@ __global__ void __launch_bounds__(kSpsThreads) k_sps(const SpsArgs a) {
     while (groups) {
       const int c = __ffs(groups) - 1;
       groups &= groups - 1;
-      const int q = wid * 512 + c * 32 + lane;  // pass sample
-      const long long j = seg0 + q;
+      const int q = c * 32 + lane;  // pass sample
+      const long long j = j0 + q;
       const uint32_t pj = P[1 + H + q];
-      const bool leader = (lane & (B - 1)) == 0;
+      // A width whose largest sum stays below its bound cannot reach the threshold and is left
+      // out before the FP64 division.
+      bool leader = (lane & (B - 1)) == 0;
       double bs = 0.0;
       long long bj = 0;
       int bwid = 0;
       bool have = false;
-      for (int k = 0; k < nw; ++k) {
-        const int w = a.wd[k];
-        const bool valid = (j < n) && (j >= w - 1) && den[k] != 0.0;
-        const uint32_t bw = valid ? pj - P[1 + H + q - w] : 0u;
-        int off;
-        const int best = block_argmax(bw, valid, B, lane, off);
-        if (leader && best >= 0) {
-          const long long num = ca[k] * (long long)best - cb[k];
-          const double snr = (double)num / den[k];
-          const long long jk = j + off;  // the leader holds the block's first sample
-          if (!have || snr > bs || (snr == bs && jk < bj)) {
+      if (B == 32) {
+        // lane k takes width k, so the widths' divisions run at once
+        uint32_t mine = 0;
+        int moff = 0;
+        for (int k = 0; k < nw; ++k) {
+          const int w = a.wd[k];
+          const bool valid = (j < n) && (j >= w - 1) && den[k] != 0.0;
+          uint32_t best;
+          int off;
+          const bool any = block_argmax(valid ? pj - P[1 + H + q - w] : 0u, valid, 32, lane, best,
+                                        off);
+          if (lane == k) {
+            have = any && (int32_t)best >= 0 && best >= bthr[k];
+            mine = best;
+            moff = off;
+          }
+        }
+        int kw = lane;
+        if (have) bs = (double)(ca[lane] * (long long)mine - cb[lane]) / den[lane];
+        // the best width: largest SNR, then the earliest sample, then the smallest width
+        for (int o = 8; o > 0; o >>= 1) {
+          const double os = __shfl_xor_sync(0xffffffffu, bs, o);
+          const int oj = __shfl_xor_sync(0xffffffffu, moff, o);
+          const int ok = __shfl_xor_sync(0xffffffffu, kw, o);
+          const bool oh = __shfl_xor_sync(0xffffffffu, have ? 1 : 0, o) != 0;
+          if (oh && (!have || os > bs || (os == bs && (oj < moff || (oj == moff && ok < kw))))) {
             have = true;
-            bs = snr;
-            bj = jk;
-            bwid = w;
+            bs = os;
+            moff = oj;
+            kw = ok;
+          }
+        }
+        leader = lane == 0;
+        bj = j + moff;
+        bwid = a.wd[kw & (kMaxWidths - 1)];
+      } else {
+        for (int k = 0; k < nw; ++k) {
+          const int w = a.wd[k];
+          const bool valid = (j < n) && (j >= w - 1) && den[k] != 0.0;
+          uint32_t best;
+          int off;
+          const bool any = block_argmax(valid ? pj - P[1 + H + q - w] : 0u, valid, B, lane, best,
+                                        off);
+          if (leader && any && (int32_t)best >= 0 && best >= bthr[k]) {
+            const double snr = (double)(ca[k] * (long long)best - cb[k]) / den[k];
+            const long long jk = j + off;  // the leader holds the block's first sample
+            if (!have || snr > bs || (snr == bs && jk < bj)) {
+              have = true;
+              bs = snr;
+              bj = jk;
+              bwid = w;
+            }
           }
         }
       }
@@ -662,9 +814,8 @@ __global__ void __launch_bounds__(kSpsThreads) k_sps(const SpsArgs a) {
         }
       }
     }
-    __syncthreads();  // every read of this pass's P is done
-    // the last H + 1 entries become the next pass's history (P[kSpsSeg] = sum before it)
-    for (int k = tid; k <= H; k += kSpsThreads) P[k] = P[kSpsSeg + k];
+    __syncwarp();  // every read of this pass's P is done
+    if (j0 + kSpsPass < s1) R.carry();
   }
 }
 
@@ -736,77 +887,127 @@ __global__ void __launch_bounds__(kSpsThreads) k_sps_fused(const SpsFusedArgs a)
 // count, sum, 128-bit sum of squares), then, for up to `iters` steps, again over the values
 // within ceil(mu - kappa*sd) .. floor(mu + kappa*sd) of the previous step's mean and population
 // deviation (FP64, one rounding per operation, as the oracle). A width whose previous step has no
-// values or no variance keeps its statistics. Each step sweeps the series once per group of
-// kClipGroup widths, forming the boxcar sums from the carried prefix sums of the search kernel.
-constexpr int kClipGroup = 8;
+// values or no variance keeps its statistics.
+//
+// Each step sweeps the series once per group of at most kClipGroup widths, each warp over its own
+// eighth of the window (SpsRow). The bounds are whole numbers, so a value is tested and summed as
+// x = B - lo <= hi - lo in 32-bit integers, and the sums of B and B^2 follow exactly from the
+// count and the sums of x and x^2. Bound by instruction issue: about 7 instructions per value,
+// where the test in FP64 was bound by the FP64 pipe.
+constexpr int kClipGroup = 6;
 
-__global__ void __launch_bounds__(kSpsThreads) k_clip_stats(const ClipArgs a) {
+__global__ void __launch_bounds__(kSpsThreads, 2) k_clip_stats(const ClipArgs a) {
   extern __shared__ __align__(16) uint32_t Ps[];
-  uint32_t* P = Ps + kSpsPad;  // [1 + hist + kSpsSeg]
-  __shared__ uint32_t warp_tot[kSpsThreads / 32];
-  __shared__ double lo_b[kMaxWidths], hi_b[kMaxWidths];
-  __shared__ int live[kMaxWidths];
+  __shared__ uint32_t lo_b[kMaxWidths], span_b[kMaxWidths];  // values lo .. lo + span
+  __shared__ int live[kMaxWidths];                           // 0: statistics final
+  __shared__ int some[kMaxWidths];  // 0: the bounds hold no value; 1; 2: 64-bit sums suffice
   __shared__ WidthStats st[kMaxWidths];
-  __shared__ unsigned long long red[kClipGroup][4][kSpsThreads / 32];
+  __shared__ unsigned long long red[kClipGroup][4][kSpsWarps];
 
   const int32_t i = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const long long n = a.n;
   const int nw = a.nw, H = a.hist;
-  const int32_t* yi = a.y + (int64_t)i * a.stride;
-  const bool vec = (reinterpret_cast<uintptr_t>(yi) & 15) == 0;
-  const int q0 = wid * 512 + 4 * lane;
+  const int wmax = a.wd[nw - 1];
+  SpsRow R;
+  R.y = a.y + (int64_t)i * a.stride;
+  R.P = Ps + (size_t)wid * sps_row_words(H) + kSpsPad;
+  R.n = n;
+  R.H = H;
+  R.lane = lane;
+  R.vec = (reinterpret_cast<uintptr_t>(R.y) & 15) == 0;
+  const uint32_t* P = R.P;
+  const long long per = ((n + kSpsWarps - 1) / kSpsWarps + 127) / 128 * 128;
+  const long long s0 = min(n, wid * per), s1 = min(n, s0 + per);
+  // a lane's sums of squares over its part of a sweep stay below 2^64, its sums of four values
+  // below 2^32
+  const double lane_values = 16.0 * (double)((per + kSpsPass - 1) / kSpsPass);
+  auto narrow = [&](uint32_t span) {
+    return (double)span * (double)span * lane_values < 1.8e19 && span < (1u << 30);
+  };
   if (tid < kMaxWidths) {
-    lo_b[tid] = -1.0;  // step 0: every value (all boxcar sums are >= 0)
-    hi_b[tid] = 1e300;
+    lo_b[tid] = 0u;  // step 0: every value (all boxcar sums are >= 0)
+    span_b[tid] = tid < nw ? (uint32_t)a.wd[tid] * a.vmax : 0u;
     live[tid] = tid < nw ? 1 : 0;
+    some[tid] = narrow(span_b[tid]) ? 2 : 1;
     st[tid] = WidthStats{0, 0, 0, 0};
   }
   __syncthreads();
+  const int ngrp = (nw + kClipGroup - 1) / kClipGroup, per_grp = (nw + ngrp - 1) / ngrp;
   for (int step = 0; step <= a.iters; ++step) {
-    for (int g0 = 0; g0 < nw; g0 += kClipGroup) {
+    for (int g0 = 0; g0 < nw; g0 += per_grp) {
+      const int ng = min(per_grp, nw - g0);
       bool any = false;
-      for (int k = g0; k < min(nw, g0 + kClipGroup); ++k) any |= live[k] != 0;
+      for (int k = g0; k < g0 + ng; ++k) any |= live[k] != 0;
       if (!any) continue;  // uniform: every thread reads the same flags
-      uint32_t cn[kClipGroup];
-      unsigned long long c1[kClipGroup], c2l[kClipGroup], c2h[kClipGroup];
+      uint32_t cn[kClipGroup], c2h[kClipGroup];
+      unsigned long long c1[kClipGroup], c2l[kClipGroup];
 #pragma unroll
-      for (int kk = 0; kk < kClipGroup; ++kk) cn[kk] = 0, c1[kk] = c2l[kk] = c2h[kk] = 0;
-      for (int k = tid; k <= H; k += kSpsThreads) P[k] = 0;  // samples before the window
-      for (long long seg0 = 0; seg0 < n; seg0 += kSpsSeg) {
-        uint32_t v[4][4];
-        sps_pass_prefix(yi, vec, n, seg0, q0, lane, wid, H, P, warp_tot, v);
+      for (int kk = 0; kk < kClipGroup; ++kk) cn[kk] = c2h[kk] = 0, c1[kk] = c2l[kk] = 0;
+      if (s0 < s1) {
+        uint4 nv[4];
+        R.load_pass(s0, nv);
+        uint32_t run = R.history(s0);
+        for (long long j0 = s0; j0 < s1; j0 += kSpsPass) {
+          uint4 v[4] = {nv[0], nv[1], nv[2], nv[3]};
+          run = R.scan(v, run);
+          R.store_pass(v);
+          __syncwarp();
+          if (j0 + kSpsPass < s1) R.load_pass(j0 + kSpsPass, nv);
+          const bool interior = j0 >= wmax - 1 && j0 + kSpsPass <= s1;
 #pragma unroll
-        for (int kk = 0; kk < kClipGroup; ++kk) {
-          const int k = g0 + kk;
-          const bool on = k < nw && live[min(k, kMaxWidths - 1)];
-          const int w = on ? a.wd[k] : 1;
-          const double lo = on ? lo_b[k] : 1.0, hi = on ? hi_b[k] : 0.0;  // empty when off
+          for (int kk = 0; kk < kClipGroup; ++kk) {
+            if (kk >= ng) break;
+            const int k = g0 + kk;
+            if (!live[k] || !some[k]) continue;  // uniform
+            const int w = a.wd[k];
+            const uint32_t lo = lo_b[k], span = span_b[k];
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int idx = 1 + H + q0 + 128 * g;
-            const uint4 s4 = prefix4(P, idx, w);
-            const long long j = seg0 + q0 + 128 * g;
+            for (int g = 0; g < 4; ++g) {
+              const uint4 s4 = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
+              uint32_t x[4] = {v[g].x - s4.x - lo, v[g].y - s4.y - lo, v[g].z - s4.z - lo,
+                               v[g].w - s4.w - lo};
+              bool in[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const uint32_t b = v[g][e] - (e == 0 ? s4.x : e == 1 ? s4.y : e == 2 ? s4.z : s4.w);
-              const double bd = (double)b;
-              if (j + e < n && j + e >= w - 1 && bd >= lo && bd <= hi) {
-                const unsigned long long sq = (unsigned long long)b * b;
-                cn[kk] += 1;
-                c1[kk] += b;
-                c2l[kk] += sq;
-                c2h[kk] += (c2l[kk] < sq) ? 1ull : 0ull;
+              for (int e = 0; e < 4; ++e) in[e] = x[e] <= span;
+              if (!interior) {
+                const long long j = j0 + 4 * lane + 128 * g;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) in[e] = in[e] && j + e < s1 && j + e >= w - 1;
               }
+              if (some[k] == 2) {
+                uint32_t sum = 0;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const uint32_t m = in[e] ? x[e] : 0u;
+                  cn[kk] += in[e] ? 1u : 0u;
+                  sum += m;
+                  c2l[kk] += (unsigned long long)m * m;
+                }
+                c1[kk] += sum;
+                continue;
+              }
+              unsigned long long sum = 0, sq = 0;  // four values below 2^31: sq below 2^64
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const uint32_t m = in[e] ? x[e] : 0u;
+                cn[kk] += in[e] ? 1u : 0u;
+                sum += m;
+                sq += (unsigned long long)m * m;
+              }
+              c1[kk] += sum;
+              c2l[kk] += sq;
+              c2h[kk] += (c2l[kk] < sq) ? 1u : 0u;
             }
           }
+          __syncwarp();  // every read of this pass's P is done
+          if (j0 + kSpsPass < s1) R.carry();
         }
-        __syncthreads();  // every read of this pass's P is done
-        for (int k = tid; k <= H; k += kSpsThreads) P[k] = P[kSpsSeg + k];
       }
-      // block sums of the group's widths: warp butterflies, then one lane per width
+      // CTA sums of the group's widths: warp butterflies, then one thread per width
 #pragma unroll
       for (int kk = 0; kk < kClipGroup; ++kk) {
+        if (kk >= ng) break;
         unsigned long long x0 = cn[kk], x1 = c1[kk], lo = c2l[kk], hi = c2h[kk];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
@@ -826,16 +1027,24 @@ __global__ void __launch_bounds__(kSpsThreads) k_clip_stats(const ClipArgs a) {
         }
       }
       __syncthreads();
-      if (tid < kClipGroup && g0 + tid < nw && live[g0 + tid]) {
-        unsigned long long x0 = 0, x1 = 0, lo = 0, hi = 0;
-        for (int q = 0; q < kSpsThreads / 32; ++q) {
-          x0 += red[tid][0][q];
+      if (tid < ng && live[g0 + tid]) {
+        unsigned long long c = 0, x1 = 0, lo = 0, hi = 0;
+        for (int q = 0; q < kSpsWarps; ++q) {
+          c += red[tid][0][q];
           x1 += red[tid][1][q];
           const unsigned long long nlo = lo + red[tid][2][q];
           hi = hi + red[tid][3][q] + (nlo < lo ? 1ull : 0ull);
           lo = nlo;
         }
-        st[g0 + tid] = WidthStats{(long long)x0, (long long)x1, lo, hi};
+        // sums of B = x + l over c values: T1 = X1 + c l, T2 = X2 + 2 l X1 + c l^2 (128 bits)
+        const unsigned long long l = lo_b[g0 + tid];
+        const unsigned long long t1 = x1 + c * l;
+        const unsigned long long a0 = 2 * l * x1, a1 = __umul64hi(2 * l, x1);
+        const unsigned long long b0 = l * l * c, b1 = __umul64hi(l * l, c);
+        unsigned long long r0 = lo + a0, r1 = hi + a1 + (r0 < lo ? 1ull : 0ull);
+        r1 += b1 + (r0 + b0 < r0 ? 1ull : 0ull);
+        r0 += b0;
+        st[g0 + tid] = WidthStats{(long long)c, (long long)t1, r0, r1};
       }
       __syncthreads();
     }
@@ -855,8 +1064,13 @@ __global__ void __launch_bounds__(kSpsThreads) k_clip_stats(const ClipArgs a) {
         const double mu = __ddiv_rn(__ll2double_rn(s.t1), dn);
         const double sd = __ddiv_rn(__dsqrt_rn(u128_to_f64(v_hi, v_lo)), dn);
         const double ks = __dmul_rn(a.kappa, sd);
-        lo_b[tid] = ceil(__dsub_rn(mu, ks));
-        hi_b[tid] = floor(__dadd_rn(mu, ks));
+        const double lo = ceil(__dsub_rn(mu, ks)), hi = floor(__dadd_rn(mu, ks));
+        // the whole-number bounds on values 0 .. 2^31 - 1
+        const double top = 2147483647.0;
+        const uint32_t l = lo <= 0.0 ? 0u : (lo <= top ? (uint32_t)lo : 0u);
+        lo_b[tid] = l;
+        span_b[tid] = hi >= top ? 0x7FFFFFFFu - l : (hi >= (double)l ? (uint32_t)hi - l : 0u);
+        some[tid] = lo <= top && hi >= 0.0 && lo <= hi ? (narrow(span_b[tid]) ? 2 : 1) : 0;
       }
     }
     __syncthreads();
@@ -866,19 +1080,31 @@ __global__ void __launch_bounds__(kSpsThreads) k_clip_stats(const ClipArgs a) {
 
 cudaError_t launch_clip_stats(const ClipArgs& a, cudaStream_t st) {
   if (a.n <= 0 || a.n_trials <= 0 || a.nw <= 0) return cudaSuccess;
-  if (a.hist < 0 || a.hist % 4 || a.hist + 1 > kSpsSeg || a.iters < 0 || !(a.kappa > 0))
+  if (a.hist < 0 || a.hist % 256 || a.hist > 1024 || a.iters < 0 || !(a.kappa > 0))
     return cudaErrorInvalidValue;
-  const size_t smem = sizeof(uint32_t) * (size_t)(kSpsPad + 1 + a.hist + kSpsSeg);
+  const size_t smem = sizeof(uint32_t) * (size_t)sps_row_words(a.hist) * kSpsWarps;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_clip_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
   k_clip_stats<<<a.n_trials, kSpsThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sps(const SpsArgs& a, cudaStream_t st) {
   if (a.n <= 0 || a.n_trials <= 0 || a.nw <= 0) return cudaSuccess;
-  if (a.hist < 0 || a.hist % 4 || a.hist + 1 > kSpsSeg || a.block < 1 || a.block > 32)
+  if (a.hist < 0 || a.hist % 256 || a.hist > 1024 || a.block < 1 || a.block > 32)
     return cudaErrorInvalidValue;
-  const size_t smem = sizeof(uint32_t) * (size_t)(kSpsPad + 1 + a.hist + kSpsSeg);
-  k_sps<<<a.n_trials, kSpsThreads, smem, st>>>(a);
+  const size_t smem = sizeof(uint32_t) * (size_t)sps_row_words(a.hist) * kSpsWarps;
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_sps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t seg = sps_segment(a.n_trials, a.n, a.hist);
+  const int64_t rows = (a.n + seg * kSpsWarps - 1) / (seg * kSpsWarps);
+  k_sps<<<dim3((unsigned)a.n_trials, (unsigned)rows), kSpsThreads, smem, st>>>(a, seg);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,125 @@
+"""Kernels at the sizes where their tiling can go wrong, against the oracle: the search and the
+clipped statistics at the edges of a warp's passes and segments, the corner turn of spectra that
+start at any byte, the staged direct kernel with and without a split of the channels, and the
+128-trial tile. Series, moments and statistics are whole numbers and are compared exactly."""
+import numpy as np
+import pytest
+
+import oracle
+from synth import configs
+from _parity import clipped_trial_snr, compare_candidates
+
+torch = pytest.importorskip("torch")
+import paper_2101_00941_gb300 as dd  # noqa: E402
+from _gpu_check import _arrivals, check  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    dd.build()
+    dd.lib()
+
+
+def _series(trials, n, seed):
+    rng = np.random.default_rng(seed)
+    y = np.rint(rng.normal(60000.0, 300.0, (trials, n))).astype(np.int32)
+    for t in range(trials):  # pulses at the window's ends and inside
+        for j in (0, n // 2, n - 1):
+            y[t, max(0, j - 2):j + 3] += 900
+    return y
+
+
+# a warp's pass is 512 samples, a segment 2 to 16 passes; rows that start off a 16-byte boundary
+@pytest.mark.parametrize("n", [1, 31, 512, 513, 1023, 4097, 20001, 65541])
+@pytest.mark.parametrize("widths,block,shift", [((1, 2, 4, 8, 16, 32, 64, 128, 256), 32, 0),
+                                                ((1, 3, 5, 600, 1024), 8, 1), ((1,), 1, 3)])
+def test_search_window_edges(n, widths, block, shift):
+    trials, d = 3, 1
+    y = _series(trials, n, 70 + n)
+    stride = n + shift + 4
+    buf = torch.zeros(trials * stride, dtype=torch.int32, device="cuda")
+    view = buf.as_strided((trials, n), (stride, 1), shift)
+    view.copy_(torch.from_numpy(y))
+    cap = trials * n
+    cands = torch.zeros(cap * dd.CAND_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    thr = 4.0
+    torch.cuda.synchronize()
+    dd.dd_sps_static(view.data_ptr(), trials, n, stride, 0, d, 17, widths, thr, block,
+                     cands.data_ptr(), cap, count.data_ptr())
+    torch.cuda.synchronize()
+    got = cands.cpu().numpy().view(dd.CAND_DTYPE)[:int(count.item())]
+    w = [k for k in widths if k <= n]
+    want = oracle.sps(y, np.arange(trials), 0, d, 17, w, block, thr) if w else got[:0]
+    order = lambda c: c[np.lexsort((c["width"], c["t_start"], c["trial"]))]
+    got, want = order(got), order(want)
+    assert got.size == want.size
+    for f in ("trial", "t_start", "width", "snr"):
+        np.testing.assert_array_equal(got[f], want[f], err_msg=f)
+
+
+def _coarse(ranges, nchans, nsamp, index, bw=300.0):
+    w = configs.mid(nsamp=nsamp, chunk_len=4096, n_streams=2, npulses=3, nchans=4096,
+                    ranges=ranges, index=index)
+    w.nchans, w.foff = nchans, -bw / nchans
+    w.pulses = tuple(configs.PulseSpec(p.dm * 0.05, min(p.t_ref, nsamp // 2), p.width,
+                                       p.amp * 8.0) for p in w.pulses)
+    return w
+
+
+@pytest.mark.parametrize("widths,sizes", [
+    ((1, 2, 4, 7, 12, 24, 48, 96, 100, 128, 200, 256, 500, 512, 1000, 1024), [4000, 4096, 3000]),
+    ((2,), [130, 4096])])
+def test_clipped_statistics_edges(widths, sizes):
+    """16 widths (three groups a sweep) with a 1024-sample history, and one width; windows that
+    end inside a pass."""
+    w = _coarse((configs.DMRange(0.0, 1.0, 5, 1), configs.DMRange(5.0, 2.0, 3, 2)), 64, 1 << 14, 71)
+    w.widths, w.threshold = widths, 4.0
+    x = w.generate(_arrivals(w))
+    ranges = w.ranges_array()
+    ref = oracle.run(x[:sum(sizes)], w.freqs(), w.tsamp, ranges, widths, w.threshold, 32, sizes)
+    plan = dd.Plan(w.freqs(), w.tsamp, ranges, 4096, n_streams=1, max_width=max(widths))
+    try:
+        xs, T = torch.from_numpy(x).cuda(), 0
+        for n, per in zip(sizes, ref["chunks"]):
+            seq = plan.run(xs[T:T + n], n)
+            T += n
+            plan.search(widths, w.threshold, estimator=dd.DD_EST_CLIPPED)
+            got, want = plan.candidates(seq), []
+            for r in range(len(ranges)):
+                y, d = per[r]["series"], int(ranges[r][3])
+                wd = [k for k in oracle.widths_for_range(widths, d) if k <= y.shape[1]]
+                if y.shape[1] and wd:
+                    want.append(oracle.sps_clipped(y, per[r]["trials"], r, d, per[r]["J0"], wd, 32,
+                                                   w.threshold))
+            want = np.concatenate(want) if want else got[:0]
+            compare_candidates(got, want, w.threshold, 32,
+                               lambda r, t, per=per: per[r]["series"][t],
+                               lambda r, per=per: per[r]["J0"], lambda r: int(ranges[r][3]),
+                               trial_snr=clipped_trial_snr(3.0, 3))
+    finally:
+        plan.close()
+
+
+@pytest.mark.parametrize("nchans", [17, 63, 80, 129])
+@pytest.mark.parametrize("offset", [0, 1, 6])
+def test_corner_turn_any_start(nchans, offset):
+    """Spectra of any length from a chunk at any byte address (chunks of 4-sample and ragged
+    lengths): one trial of DM 0 is the sum over channels."""
+    n = 1024
+    x = np.random.default_rng(72).integers(0, 256, (n, nchans), dtype=np.uint8)
+    f = 1500.0 - np.arange(nchans) * 1.0
+    plan = dd.Plan(f, 64e-6, [(0.0, 1.0, 1, 1)], n, n_streams=1, max_width=4)
+    try:
+        buf = torch.zeros(offset + n * nchans, dtype=torch.uint8, device="cuda")
+        buf[offset:] = torch.from_numpy(x.reshape(-1)).cuda()
+        at = 0
+        for m in (1, 258, 63, 702):
+            plan.run(buf[offset + at * nchans:offset + (at + m) * nchans].view(m, nchans), m)
+            np.testing.assert_array_equal(plan.series(0)[0].cpu().numpy()[0],
+                                          x[at:at + m].sum(1, dtype=np.int64))
+            at += m
+    finally:
+        plan.close()
