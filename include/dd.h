@@ -533,11 +533,11 @@ void dd_serve_destroy(dd_server_t server);
  * verifies them against it: each trial's pair words lie in one plane (even or odd words) of its
  * delay class and stand for class words that add, in every channel, the sample at that trial's
  * own delay; class word ranges are aligned; every read stays inside the staged rows; the build
- * work lists cover every block of every class once.
+ * tasks reach every class by its own channel steps and store every unit of it once.
  *   shifts       : int32 [n_trials][cpad], delays of one range in decimated samples, channels
  *                  padded to cpad (a multiple of 8) by repeating the last channel
  *   tile_samples : 512 or 256 (outputs per time tile)
- *   tile_trials  : 64 or 32 (trials per tile)
+ *   tile_trials  : 128 (with 256 outputs), 64 or 32 (trials per tile)
  *   ok           : receives 1 if the tiled kernel can run the range, else 0
  *   violations   : receives the number of violated checks (0 expected; 0 when ok is 0)
  * Errors: DD_ERR_ARG.

@@ -322,7 +322,9 @@ int plan_tiled_shape(const int32_t* tab, int ntr, int cpad, int d, int tt, int t
 }
 
 // Tile shapes (outputs, trials, threads per CTA) in the order a plan tries them.
-constexpr int kShapes[4][3] = {{512, 64, 512}, {512, 64, 1024}, {256, 64, 512}, {256, 32, 512}};
+constexpr int kNumShapes = 5;
+constexpr int kShapes[kNumShapes][3] = {
+    {512, 64, 512}, {256, 128, 512}, {512, 64, 1024}, {256, 64, 512}, {256, 32, 512}};
 
 // Turn recorded event pairs into intervals relative to the reference event.
 int harvest_timing(dd_plan_s* p) {
@@ -471,7 +473,7 @@ int plan_autotune(dd_plan_s* p) {
     }
     float best_ms = 1e30f;
     RangeKernel best = cur;
-    for (int shape = 0; shape < 4; ++shape) {
+    for (int shape = 0; shape < kNumShapes; ++shape) {
       const int tt = kShapes[shape][0], trials = kShapes[shape][1], nt = kShapes[shape][2];
       RangeKernel k = cur;
       if (tt != cur.tt || trials != cur.trials || nt != cur.threads) {
@@ -625,6 +627,10 @@ int dd_plan(const double* freqs_mhz, int32_t nchans, double tsamp_s, const dd_ra
 
   dd_plan_s* p = new dd_plan_s();
   p->device = o.device;
+  if (cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, o.device) != cudaSuccess) {
+    delete p;
+    return fail(DD_ERR_CUDA, "device attributes could not be read");
+  }
   p->C = nchans;
   p->Cp = (int32_t)round_up(nchans, 8);
   p->tsamp = tsamp_s;
@@ -715,9 +721,25 @@ int dd_plan(const double* freqs_mhz, int32_t nchans, double tsamp_s, const dd_ra
       for (int r = 0; r < nranges; ++r) {
         // the first shape that fits, in kShapes order; testing aids force the 256-output tile
         // (DD_FLAG_TILE256) or the 32-trial tile (DD_FLAG_TRIALS32)
-        for (int shape = 0; shape < 4 && !p->rk[r].tiled; ++shape) {
+        // 128 trials x 256 outputs share each class's words among more trials than 64 x 512, but
+        // round the trials up to 128 and see a wider spread of delays: by the estimated work of
+        // the launch (tiled_cost). Both measured on the 4096-channel plan, x1 / x2 / x4 / x8:
+        // 17.0 / 5.5 / 2.9 / 2.0 ms with 64 x 512 (about), 15.5 / 4.7 / 2.5 / 1.7 with 128 x 256;
+        // on the 1024-channel plan, whose spread per trial is as large and whose classes are more,
+        // 2.39 / 0.80 / 0.39 against 2.38 / 0.77 / 0.36
+        const int64_t nout = o.chunk_len / ranges[r].decimation;
+        const int32_t* rt = &full[(size_t)p->row0[r] * p->Cp];
+        const double c64 = ddk::tiled_cost(rt, ranges[r].n_trials, p->Cp, ranges[r].decimation,
+                                           512, 64, 512, nout, p->sms);
+        const double c128 = ddk::tiled_cost(rt, ranges[r].n_trials, p->Cp, ranges[r].decimation,
+                                            256, 128, 512, nout, p->sms);
+        // (a launch that leaves SMs idle keeps the 512-output tile)
+        const bool fills = (int64_t)((ranges[r].n_trials + 63) / 64) * ((nout + 511) / 512) >= p->sms;
+        const bool wide = fills && c128 >= 0 && (c64 < 0 || c128 < 0.97 * c64);
+        for (int k = 0; k < kNumShapes && !p->rk[r].tiled; ++k) {
+          const int shape = wide && k < 2 ? 1 - k : k;
           const int tt = kShapes[shape][0], trials = kShapes[shape][1], nt = kShapes[shape][2];
-          if ((o.flags & DD_FLAG_TILE256) && tt != 256) continue;
+          if ((o.flags & DD_FLAG_TILE256) && (tt != 256 || trials == 128)) continue;
           if ((o.flags & DD_FLAG_TRIALS32) && trials != 32) continue;
           if ((o.flags & DD_FLAG_WARPS32) != 0 && nt != 1024) continue;
           bool ok = false;
@@ -886,7 +908,6 @@ int dd_fuse_search(dd_plan_t p, const int32_t* widths, int32_t nwidths, uint32_t
     return fail(DD_ERR_STATE, "dd_fuse_search must come before the plan's first dd_run");
   if (!p->fused_widths.empty()) return fail(DD_ERR_STATE, "the plan's search is already fused");
   DD_CK(cudaSetDevice(p->device));
-  DD_CK(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
   const bool keep = (fuse_flags & DD_FUSE_KEEP_SERIES) != 0;
   const int nr = (int)p->ranges.size();
   std::vector<int32_t> full;  // the delay table at the padded stride, for re-planning a range
@@ -1131,10 +1152,12 @@ static int run_impl(dd_plan_t p, const uint8_t* chunk, int64_t nsamp, void* cuda
         }
         DD_CK(ddk::launch_fused(A, F, R.is_u16, K.fsmem, st));
         p->launches += F.nsegs > 1 ? 2 : 1;
-      } else if (defer && K.tt == 512 && K.trials == 64 && K.threads == 512) {
+      } else if (defer && K.threads == 512 && K.tt * K.trials == 512 * 64) {
         ddk::DeferredTile dt;
         dt.args = A;
         dt.is_u16 = R.is_u16;
+        dt.tt = K.tt;
+        dt.trials = K.trials;
         dt.nstage = K.nstage;
         dt.smem = K.smem;
         defer->push_back(dt);
@@ -1356,9 +1379,9 @@ int dd_tiled_plan_check(const int32_t* shifts, int32_t n_trials, int32_t cpad,
                         int32_t* ok, int64_t* violations) {
   if (!shifts || !ok || !violations) return fail(DD_ERR_ARG, "NULL argument");
   if (n_trials < 1 || cpad < 8 || cpad % 8 || (tile_samples != 256 && tile_samples != 512) ||
-      (tile_trials != 32 && tile_trials != 64))
+      (tile_trials != 32 && tile_trials != 64 && tile_trials != 128))
     return fail(DD_ERR_ARG, "need n_trials >= 1, cpad a multiple of 8, tile_samples 256 or 512, "
-                            "tile_trials 32 or 64");
+                            "tile_trials 32, 64 or 128");
   int k = 0;
   *violations = ddk::tiled_plan_check(shifts, n_trials, cpad, decimation, tile_samples,
                                       tile_trials, &k);

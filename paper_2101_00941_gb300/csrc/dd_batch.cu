@@ -147,28 +147,30 @@ int enqueue_step_persistent(dd_batch_s* b) {
     if (rc) break;
     if ((int64_t)defs.size() > b->max_descs)
       return ddk::report_error(DD_ERR_STATE, "dd_batch: more deferred launches than planned");
-    // the round's work lists: one per instance (uint8/uint16 x 3/4 staging buffers), each a run
-    // of segments (one per deferred launch: all its tiles)
+    // the round's work lists: one per instance (uint8/uint16 x 3/4 staging buffers x tile shape),
+    // each a run of segments (one per deferred launch: all its tiles)
     ddk::TiledArgs* hd = b->h_descs + c * b->max_descs;
     int32_t* hs = b->h_segd + c * b->max_descs;
-    int64_t* hf = b->h_segf + c * (b->max_descs + 4);
+    int64_t* hf = b->h_segf + c * (b->max_descs + 8);
     for (size_t k = 0; k < defs.size(); ++k) hd[k] = defs[k].args;
     int nseg_total = 0;
     int64_t fpos = 0;
     struct Inst {
-      int is_u16, nstage, nseg, seg0;
+      int is_u16, nstage, tt, trials, nseg, seg0;
       int64_t f0;
       size_t smem;
     };
     std::vector<Inst> insts;
     for (int u16 = 0; u16 < 2; ++u16)
-      for (int ns = 3; ns <= 4; ++ns) {
-        Inst in{u16, ns, 0, nseg_total, fpos, 0};
+      for (int v = 0; v < 4; ++v) {
+        const int ns = 3 + v % 2, tt = v < 2 ? 512 : 256, trials = v < 2 ? 64 : 128;
+        Inst in{u16, ns, tt, trials, 0, nseg_total, fpos, 0};
         int64_t first = 0;
         for (size_t k = 0; k < defs.size(); ++k) {
-          if (defs[k].is_u16 != u16 || defs[k].nstage != ns) continue;
+          if (defs[k].is_u16 != u16 || defs[k].nstage != ns || defs[k].tt != tt) continue;
           const ddk::TiledArgs& a = defs[k].args;
-          const int64_t tiles = (int64_t)((a.n_trials + 63) / 64) * ((a.nout + 511) / 512);
+          const int64_t tiles =
+              (int64_t)((a.n_trials + trials - 1) / trials) * ((a.nout + tt - 1) / tt);
           hs[nseg_total + in.nseg] = (int32_t)k;
           hf[fpos + in.nseg] = first;
           first += tiles;
@@ -183,7 +185,7 @@ int enqueue_step_persistent(dd_batch_s* b) {
       }
     ddk::TiledArgs* dd_ = b->d_descs + c * b->max_descs;
     int32_t* ds = b->d_segd + c * b->max_descs;
-    int64_t* df = b->d_segf + c * (b->max_descs + 4);
+    int64_t* df = b->d_segf + c * (b->max_descs + 8);
     // (a round whose ranges all run on the direct kernel has no work list, only searches)
     if (!defs.empty()) {
       rc = ck(cudaMemcpyAsync(dd_, hd, sizeof(ddk::TiledArgs) * defs.size(),
@@ -197,7 +199,7 @@ int enqueue_step_persistent(dd_batch_s* b) {
         rc = ck(cudaMemcpyAsync(df, hf, sizeof(int64_t) * fpos, cudaMemcpyHostToDevice, b->root),
                 "work list");
       if (rc == DD_OK)
-        rc = ck(cudaMemsetAsync(b->d_counters + 4 * c, 0, 4 * sizeof(unsigned long long),
+        rc = ck(cudaMemsetAsync(b->d_counters + 8 * c, 0, 8 * sizeof(unsigned long long),
                                 b->root),
                 "counters");
     }
@@ -209,9 +211,9 @@ int enqueue_step_persistent(dd_batch_s* b) {
       pa.seg_first = df + in.f0;
       pa.nseg = in.nseg;
       pa.pad = 0;
-      pa.counter = b->d_counters + 4 * c + g;
-      rc = ck(ddk::launch_tiled_persistent(pa, in.is_u16, 512, in.nstage, 64, 512, in.smem,
-                                           b->sms, b->root),
+      pa.counter = b->d_counters + 8 * c + g;
+      rc = ck(ddk::launch_tiled_persistent(pa, in.is_u16, in.tt, in.nstage, in.trials, 512,
+                                           in.smem, b->sms, b->root),
               "persistent dedispersion");
     }
     for (size_t i = 0; rc == DD_OK && i < b->plans.size(); ++i) {
@@ -319,7 +321,7 @@ int dd_batch_create(int32_t nbeams, const dd_batch_beam_t* beams, const dd_range
     for (auto n : b->nchunks) b->rounds = std::max(b->rounds, n);
     b->max_descs = (int64_t)b->plans.size() * nranges;
     const size_t nd = (size_t)(b->rounds * b->max_descs);
-    const size_t nf = (size_t)(b->rounds * (b->max_descs + 4));
+    const size_t nf = (size_t)(b->rounds * (b->max_descs + 8));
     if (cudaMallocHost(&b->h_descs, sizeof(ddk::TiledArgs) * std::max<size_t>(nd, 1)) !=
             cudaSuccess ||
         cudaMallocHost(&b->h_segd, sizeof(int32_t) * std::max<size_t>(nd, 1)) != cudaSuccess ||
@@ -328,7 +330,7 @@ int dd_batch_create(int32_t nbeams, const dd_batch_beam_t* beams, const dd_range
             cudaSuccess ||
         cudaMalloc(&b->d_segd, sizeof(int32_t) * std::max<size_t>(nd, 1)) != cudaSuccess ||
         cudaMalloc(&b->d_segf, sizeof(int64_t) * std::max<size_t>(nf, 1)) != cudaSuccess ||
-        cudaMalloc(&b->d_counters, sizeof(unsigned long long) * 4 *
+        cudaMalloc(&b->d_counters, sizeof(unsigned long long) * 8 *
                                        std::max<size_t>((size_t)b->rounds, 1)) != cudaSuccess) {
       cudaGetLastError();
       rc = ddk::report_error(DD_ERR_NOMEM, "dd_batch_create: persistent work lists");

@@ -48,6 +48,9 @@
 #include <cstddef>
 #include <cstring>
 #include <mutex>
+#include <new>
+#include <system_error>
+#include <thread>
 
 #include "dd_internal.h"
 
@@ -55,7 +58,8 @@ namespace ddk {
 
 namespace {
 
-constexpr int kMaxTileTrials = 64;         // trials per tile: 64 or 32
+constexpr int kMaxTileTrials = 128;        // trials per tile: 128, 64 or 32
+constexpr int kFusedTrials = 64;           // ... of the fused form
 constexpr int kThreads = 512;               // threads of the 16-warp shapes
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxWarps = 32;
@@ -63,9 +67,9 @@ constexpr int kG = 8;                       // channels per group (one delay cla
 constexpr int kNG = 2;                      // groups per stage
 constexpr int kRows = kG * kNG;             // channel rows per stage
 constexpr int kMaxNStage = 4;               // staging buffers (rows + class table), at most
-constexpr int kMaxCls = 16;                 // classes per group
+constexpr int kMaxCls = 24;                 // classes per group
 constexpr int kMaxSteps = 3;                // channel steps between chained classes
-constexpr int kMaxLinks = 2 * kMaxCls;      // chain links (classes and in-between steps) per group
+constexpr int kMaxLinks = 32;               // chain links (classes and in-between steps) per group
 constexpr int kMaxTasks = 112;              // build tasks per stage
 constexpr int kBlock = 31;                  // build units stored per 32-lane block
 constexpr int kSegBytes = 128;              // inner extent of a staged-row copy (tensor map)
@@ -74,7 +78,7 @@ constexpr size_t kSmemLimit2 = 110 * 1024;  // ... when two CTAs share an SM
 
 // CTAs per SM a tile shape is compiled for (its register budget: 65536 / (NT x CTAs)).
 __host__ __device__ constexpr int tile_ctas(int D, int TT, int NT) {
-  return (NT == 1024 || (D == 64 && TT == 512)) ? 1 : 2;
+  return (NT == 1024 || D * TT == 64 * 512) ? 1 : 2;
 }
 
 // Entry of trial t of a tile in StageTab::zstart for a CTA of W warps with tpw trials per warp:
@@ -444,7 +448,7 @@ __device__ __forceinline__ uint32_t group_max(uint32_t key, int B, int lane, int
 
 // Head and tail buffers of CTA (trial tile bx, segment seg): [64][hist] each.
 __device__ __forceinline__ uint32_t* fused_edge(const FusedArgs& f, int ntx, int bx, int seg) {
-  return f.edge + ((size_t)seg * ntx + bx) * 2 * kMaxTileTrials * (size_t)f.hist;
+  return f.edge + ((size_t)seg * ntx + bx) * 2 * kFusedTrials * (size_t)f.hist;
 }
 
 template <int TT, int W, int kTPW, int KT>
@@ -456,10 +460,10 @@ __device__ __forceinline__ void fused_search(const TiledArgs& a, const FusedArgs
   constexpr int KP = KT / 2;
   const int hist = f.hist, HP = f.hp, Bk = f.block, nw = f.nw;
   const int wmax = f.wd[nw - 1];
-  const int ntx = (a.n_trials + kMaxTileTrials - 1) / kMaxTileTrials;
+  const int ntx = (a.n_trials + kFusedTrials - 1) / kFusedTrials;
   const int seg = by / f.seg_tiles;
   uint32_t* head = fused_edge(f, ntx, bx, seg);
-  uint32_t* tail = head + kMaxTileTrials * (size_t)hist;
+  uint32_t* tail = head + kFusedTrials * (size_t)hist;
   uint32_t* E = reinterpret_cast<uint32_t*>(smem + f.e_off) + (size_t)warp * (HP + TT) + HP;
   const int64_t nout = a.nout;
   const uint64_t pol = l2_keep_policy();
@@ -591,11 +595,11 @@ __global__ void __launch_bounds__(512) k_fused_edges(const __grid_constant__ Til
   const int ntx = gridDim.x / 4;
   const int hist = f.hist, Bk = f.block;
   const int t = quarter * kEdgeTrials + warp;  // trial within the trial tile
-  const int trial = bx * kMaxTileTrials + t;
+  const int trial = bx * kFusedTrials + t;
   if (trial >= a.n_trials) return;  // warp-uniform; no barrier follows
   const uint32_t* hd = fused_edge(f, ntx, bx, seg) + (size_t)t * hist;
   const uint32_t* tl =
-      fused_edge(f, ntx, bx, seg - 1) + kMaxTileTrials * (size_t)hist + (size_t)t * hist;
+      fused_edge(f, ntx, bx, seg - 1) + kFusedTrials * (size_t)hist + (size_t)t * hist;
   uint32_t* H = edge_rows + (size_t)warp * 2 * hist;
   uint32_t* T = H + hist;
 #pragma unroll 4
@@ -624,16 +628,31 @@ __global__ void __launch_bounds__(512) k_fused_edges(const __grid_constant__ Til
   }
 }
 
-// Word 32k + lane of every trial's sequence in both groups (shared-memory addresses of word 0)
-// added to the packed sums.
-template <int KP, int kTPW>
-__device__ __forceinline__ void add_words(const uint32_t (&zp)[kTPW], const uint32_t (&zq)[kTPW],
+// Words 32k + lane of N trials' sequences in both groups (or, both = false, in the first) added
+// to the packed sums of trials q0 ..; tc: shared address of the trials' word offsets, zs: of the
+// stage's words at the lane.
+template <int KP, int N, int kTPW>
+__device__ __forceinline__ void add_words(uint32_t zs, uint32_t tc, bool both, int q0,
                                           uint32_t (&pk)[kTPW][KP]) {
+  uint32_t zp[N], zq[N];  // N trials' words in group 0 and 1
 #pragma unroll
-  for (int k = 0; k < KP; ++k)
+  for (int q = 0; q < N; q += 2) {
+    const uint32_t e = lds<0>(tc + 2 * q), f = lds<2 * kMaxTileTrials>(tc + 2 * q);
+    zp[q] = zs + 4u * (e & 0xFFFFu), zp[q + 1] = zs + 4u * (e >> 16);
+    zq[q] = zs + 4u * (f & 0xFFFFu), zq[q + 1] = zs + 4u * (f >> 16);
+  }
+  if (both) {
 #pragma unroll
-    for (int q = 0; q < kTPW; ++q)
-      pk[q][k] += lds<0>(zp[q] + 128 * k) + lds<0>(zq[q] + 128 * k);
+    for (int k = 0; k < KP; ++k)
+#pragma unroll
+      for (int q = 0; q < N; ++q)
+        pk[q0 + q][k] += lds<0>(zp[q] + 128 * k) + lds<0>(zq[q] + 128 * k);
+  } else {
+#pragma unroll
+    for (int k = 0; k < KP; ++k)
+#pragma unroll
+      for (int q = 0; q < N; ++q) pk[q0 + q][k] += lds<0>(zp[q] + 128 * k);
+  }
 }
 
 template <typename T, int TT, int NS, int D, int NT, bool FUSED = false>
@@ -728,24 +747,10 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
       const uint32_t tc = stab + b0 * tab_step + (uint32_t)offsetof(StageTab, zstart) +
                           2u * kTPW * warp;
       const uint32_t zs = zcur + 4u * lane;
-      uint32_t zp[kTPW], zq[kTPW];
-      static_assert(kTPW == 4 || kTPW == 2, "a warp's offsets are one 8- or 4-byte load");
-      const uint32_t e0 = lds<0>(tc), e1 = lds<2 * kMaxTileTrials>(tc);
-      zp[0] = zs + 4u * (e0 & 0xFFFFu); zp[1] = zs + 4u * (e0 >> 16);
-      zq[0] = zs + 4u * (e1 & 0xFFFFu); zq[1] = zs + 4u * (e1 >> 16);
-      if constexpr (kTPW == 4) {
-        const uint32_t e2 = lds<4>(tc), e3 = lds<2 * kMaxTileTrials + 4>(tc);
-        zp[2] = zs + 4u * (e2 & 0xFFFFu); zp[3] = zs + 4u * (e2 >> 16);
-        zq[2] = zs + 4u * (e3 & 0xFFFFu); zq[3] = zs + 4u * (e3 >> 16);
-      }
-      if (ng == kNG) {  // uniform; only the last stage may hold one group
-        add_words<KP, kTPW>(zp, zq, pk);
-      } else {
+      constexpr int N = kTPW < 4 ? kTPW : 4;  // trials at a time: eight row addresses
 #pragma unroll
-        for (int k = 0; k < KP; ++k)
-#pragma unroll
-          for (int q = 0; q < kTPW; ++q) pk[q][k] += lds<0>(zp[q] + 128 * k);
-      }
+      for (int q = 0; q < kTPW; q += N)  // only the last stage may hold one group
+        add_words<KP, N>(zs, tc + 2u * q, ng == kNG, q, pk);
       if (--left == 0 || s + 1 == nstages) {  // uniform
         left = a.flush;
 #pragma unroll
@@ -927,14 +932,14 @@ constexpr BuildCost kCostU8{100, 16, 18}, kCostU16{80, 13, 14};
 // Deal a stage's build work to W warps: per group and block of 31 units, the chain of links,
 // from and to classes that store units in the block, cut where the plan breaks the chain
 // (link without a step) and where a warp has its share. The share is the smallest, found by
-// bisection, with which W warps suffice. False if the task list overflows.
-bool deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
+// bisection, with which W warps suffice. Returns it, or 0 if the task list overflows.
+int deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
   const int first[kNG + 1] = {0, st.nlink[0], st.nlink[0] + st.nlink[1]};
   int nblk[kNG] = {0, 0};
   for (int gl = 0; gl < kNG; ++gl)
     for (int p = first[gl]; p < first[gl + 1]; ++p)
       nblk[gl] = std::max(nblk[gl], (int)(cls[p].ulo() + cls[p].un() + kBlock - 1) / kBlock);
-  if (nblk[0] > kMaxBlocks || nblk[1] > kMaxBlocks) return false;
+  if (nblk[0] > kMaxBlocks || nblk[1] > kMaxBlocks) return 0;
   auto stores = [&](int p, int b) {
     return cls[p].un() && (int)cls[p].ulo() < (b + 1) * kBlock &&
            (int)(cls[p].ulo() + cls[p].un()) > b * kBlock;
@@ -988,7 +993,7 @@ bool deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
     const int mid = (lo + hi) / 2;
     if (deal(mid, false) > W) lo = mid; else hi = mid;
   }
-  return deal(hi, true) > 0;
+  return deal(hi, true) > 0 ? hi : 0;
 }
 
 int stage_tasks(const StageTab& st) {
@@ -1062,18 +1067,156 @@ static void tiled_smem_work(TiledPlan& P, int ntiles, int nstages, int ngroups, 
 // 255 x decimation, so decimation must stay at or below 16; delays must be monotone in the trial
 // within a channel; classes, tasks and the staged rows must fit their fixed-size tables and
 // shared memory.
+namespace {
+
+// A stage's table with room for every link, and what the plan needs to know of it.
+struct StagePlan {
+  StageTab st;
+  ClsLink cls[kNG * kMaxLinks];
+  int words, links;  // pair words and links used
+  int share;         // the largest warp's build work (BuildCost units)
+};
+
+bool plan_stage(const int32_t* tab, int t0, int n, int cpad, int s, bool u16, int tt, int D,
+                int W, int row_slot, StagePlan& F) {
+  const int U = u16 ? Word<uint16_t>::kUnit : Word<uint8_t>::kUnit;
+  const int es = u16 ? 2 : 1, ngroups = cpad / kG;
+  std::memset(&F, 0, sizeof F);
+  StageTab& st = F.st;
+  int32_t xmin = INT32_MAX;
+  for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
+    xmin = std::min(xmin, tab[(int64_t)t0 * cpad + c]);
+  st.xmin = xmin;
+  int words = 0, nl = 0;  // words and links of the groups before
+  for (int gl = 0; gl < kNG && s * kNG + gl < ngroups; ++gl) {
+    const int g = s * kNG + gl;
+    int b[kMaxTileTrials], cls_of[kMaxTileTrials];
+    int32_t ckey[kMaxCls][kG];
+    int cmin[kMaxCls], cmax[kMaxCls], csum[kMaxCls];
+    int ncls = 0, prev = 0, f0 = INT32_MAX;
+    const int nl0 = nl;
+    for (int i = 0; i < n; ++i) {
+      const int32_t* sv = tab + (int64_t)(t0 + i) * cpad + kG * g;
+      b[i] = *std::min_element(sv, sv + kG);
+      f0 = std::min(f0, b[i]);
+      int32_t key[kG];
+      int sum = 0;
+      for (int q = 0; q < kG; ++q) {
+        const int64_t r = (int64_t)sv[q] - b[i];
+        if (r > 32767) return false;
+        key[q] = (int32_t)r;
+        sum += (int)r;
+      }
+      int p = 0;
+      while (p < ncls && !(csum[p] == sum && std::equal(key, key + kG, ckey[p]))) ++p;
+      if (p == ncls) {
+        if (ncls == kMaxCls) return false;
+        std::copy(key, key + kG, ckey[ncls]);
+        cmin[ncls] = cmax[ncls] = b[i];
+        csum[ncls] = sum;
+        ++ncls;
+      } else {
+        cmin[p] = std::min(cmin[p], b[i]);
+        cmax[p] = std::max(cmax[p], b[i]);
+      }
+      cls_of[i] = p;
+    }
+    int order[kMaxCls], zoff[kMaxCls], zlens[kMaxCls], ulos[kMaxCls];
+    for (int p = 0; p < ncls; ++p) order[p] = p;
+    std::stable_sort(order, order + ncls, [&](int x, int y) { return csum[x] < csum[y]; });
+    for (int k = 0; k < ncls; ++k) {
+      const int p = order[k];
+      const int ulo = (cmin[p] - f0) / U;
+      if (ulo > 32767 || cmax[p] - f0 + tt > 65535) return false;
+      int un = (cmax[p] - f0 + tt + U - 1) / U - ulo;
+      if (u16) un += un & 1;  // 16-byte aligned classes
+      zoff[p] = words;
+      zlens[p] = un * U;
+      ulos[p] = ulo;
+      int32_t key[kG];  // walks from the preceding class to this one
+      std::copy(ckey[k > 0 ? prev : p], ckey[k > 0 ? prev : p] + kG, key);
+      auto at_row = [&](int q, int r) {
+        return 8u * es * (uint32_t)((gl * kG + q) * row_slot + f0 + r - xmin);
+      };
+      int dist = 0;
+      for (int q = 0; q < kG; ++q) dist += std::abs(ckey[p][q] - key[q]);
+      if (k == 0 || dist > kMaxSteps || nl - nl0 + dist + ncls - k - 1 > kMaxLinks) {
+        std::copy(ckey[p], ckey[p] + kG, key);  // a chain starts here
+        for (int q = 0; q < kG; ++q) F.cls[nl].off[q] = at_row(q, key[q]);
+        ++nl;
+      }
+      for (int q = 0; q < kG; ++q)
+        while (key[q] != ckey[p][q]) {
+          const bool up = ckey[p][q] > key[q];
+          F.cls[nl].step = (up ? kStepAdd : kStepSub) | at_row(q, up ? key[q] : key[q] - 1);
+          key[q] += up ? 1 : -1;
+          for (int c = 0; c < kG; ++c) F.cls[nl].off[c] = at_row(c, key[c]);
+          ++nl;
+        }
+      ClsLink& e = F.cls[nl - 1];
+      e.ev = 4 * (words - ulo * U / 2);
+      e.od = e.ev + 2 * zlens[p];
+      e.range = (uint32_t)ulo | (uint32_t)un << 16;
+      prev = p;
+      words += zlens[p];
+      if (words > 32767) return false;
+    }
+    for (int i = 0; i < n; ++i) {
+      const int p = cls_of[i], o = b[i] - f0 - ulos[p] * U;
+      st.zstart[gl][trial_slot(i, W, D / W)] =
+          (int16_t)(zoff[p] + (o % 2) * (zlens[p] / 2) + o / 2);
+    }
+    st.nlink[gl] = (uint8_t)(nl - nl0);
+  }
+  F.words = words;
+  F.links = nl;
+  F.share = deal_work(st, F.cls, W, u16 ? kCostU16 : kCostU8);
+  return F.share > 0;
+}
+
+bool shape_exists(int tt, int D, int nt) {
+  return (tt == 512 && D == 64 && (nt == 512 || nt == 1024)) ||
+         (tt == 256 && (D == 128 || D == 64 || D == 32) && nt == 512);
+}
+
+}  // namespace
+
+double tiled_cost(const int32_t* tab, int ntr, int cpad, int decimation, int tt, int D, int nt,
+                  int64_t nout, int sms) {
+  if (decimation < 1 || kRows * 255 * decimation > 65535 || cpad % kG || !shape_exists(tt, D, nt))
+    return -1.0;
+  const int nstages = (cpad / kG + kNG - 1) / kNG, ntiles = (ntr + D - 1) / D;
+  const int W = nt / 32;
+  StagePlan F;
+  double sum = 0;
+  int count = 0;
+  for (int a = 0; a < std::min(ntiles, 4); ++a)
+    for (int b = 0; b < std::min(nstages, 16); ++b) {
+      const int ti = (int)((int64_t)a * ntiles / std::min(ntiles, 4));
+      const int s = (int)((int64_t)b * nstages / std::min(nstages, 16));
+      if (!plan_stage(tab, ti * D, std::min(D, ntr - ti * D), cpad, s, decimation > 1, tt, D, W, 0,
+                      F))
+        return -1.0;
+      sum += F.share;
+      ++count;
+    }
+  // the rest of a stage, per warp: kTPW x KP words (two loads and an add each) and about 100
+  // instructions of waits, addresses and barrier
+  const double stage = sum / count + (D / W) * (tt / 64) * 3 + 100;
+  const int64_t ctas = ntiles * ((nout + tt - 1) / tt), slots = (int64_t)sms * tile_ctas(D, tt, nt);
+  return stage * nstages * (double)((ctas + slots - 1) / slots) * tile_ctas(D, tt, nt);
+}
+
 TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int tt, int D,
                      int nt) {
   TiledPlan P;
   P.ok = false;
   const bool u16 = decimation > 1;
   if (decimation < 1 || kRows * 255 * decimation > 65535 || cpad % kG) return P;
-  if ((D != 64 && D != 32) || (tt != 512 && tt != 256) || (nt != 512 && nt != 1024)) return P;
-  const int NG = kNG, U = u16 ? Word<uint16_t>::kUnit : Word<uint8_t>::kUnit;
+  if (!shape_exists(tt, D, nt)) return P;
   const int es = u16 ? 2 : 1, W = nt / 32;
-  const int ngroups = cpad / kG, nstages = (ngroups + NG - 1) / NG;
+  const int ngroups = cpad / kG, nstages = (ngroups + kNG - 1) / kNG;
   const int ntiles = (ntr + D - 1) / D;
-  const BuildCost cost = u16 ? kCostU16 : kCostU8;
   // staged rows: a stage's common copy window runs from the smallest first-trial delay to the
   // largest last-trial delay of its channels
   int64_t spread = 0, span = 0;
@@ -1081,9 +1224,12 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
     const int t0 = ti * D, n = std::min(D, ntr - t0);
     const int32_t* a = tab + (int64_t)t0 * cpad;
     const int32_t* z = tab + (int64_t)(t0 + n - 1) * cpad;
-    for (int i = 1; i < n; ++i)
+    for (int i = 1; i < n; ++i) {
+      bool down = false;
       for (int c = 0; c < cpad; ++c)
-        if (a[(int64_t)i * cpad + c] < a[(int64_t)(i - 1) * cpad + c]) return P;
+        down |= a[(int64_t)i * cpad + c] < a[(int64_t)(i - 1) * cpad + c];
+      if (down) return P;
+    }
     for (int c0 = 0; c0 < cpad; c0 += kRows) {
       int32_t xmin = INT32_MAX, xmax = 0;
       for (int c = c0; c < std::min(cpad, c0 + kRows); ++c) {
@@ -1106,125 +1252,76 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
   P.nseg = (int)std::min<int64_t>((span + tt + 32 + 2 * SEG - 2) / SEG, 256);
   if (P.nseg > 255) return P;
   P.row_slot = P.nseg * SEG;
-  // row offsets and their phase fit the 16-bit byte offsets the plan counts with
+  // a stage buffer's byte offsets fit 16 bits (ClsLink's fields count on it)
   if ((size_t)kRows * P.row_slot * es > 65535) return P;
 
-  // tables at the largest pitch first, repacked below
-  struct Full {
-    StageTab st;
-    ClsLink cls[kNG * kMaxLinks];
+  // the tables, each as long as its links: host threads take runs of trial tiles
+  struct Part {
+    std::vector<uint8_t> bytes;
+    std::vector<uint32_t> len;
+    int words = 0;
+    bool ok = true, nomem = false;
   };
-  std::vector<uint8_t> out;
-  std::vector<size_t> at((size_t)ntiles * nstages + 1, 0);
-  out.reserve((size_t)ntiles * nstages * (sizeof(StageTab) + 18 * sizeof(ClsLink)));
-  int64_t zcap = 0;
-  size_t most = 0;
-  Full F;
-  for (int ti = 0; ti < ntiles; ++ti) {
-    const int t0 = ti * D, n = std::min(D, ntr - t0);
-    for (int s = 0; s < nstages; ++s) {
-      std::memset(&F, 0, sizeof F);
-      StageTab& st = F.st;
-      int32_t xmin = INT32_MAX;
-      for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
-        xmin = std::min(xmin, tab[(int64_t)t0 * cpad + c]);
-      st.xmin = xmin;
-      int words = 0, nl = 0;  // words and links of the groups before
-      for (int gl = 0; gl < NG && s * NG + gl < ngroups; ++gl) {
-        const int g = s * NG + gl;
-        int b[kMaxTileTrials], cls_of[kMaxTileTrials];
-        int32_t ckey[kMaxCls][kG];
-        int cmin[kMaxCls], cmax[kMaxCls], csum[kMaxCls];
-        int ncls = 0, prev = 0, f0 = INT32_MAX;
-        const int nl0 = nl;
-        for (int i = 0; i < n; ++i) {
-          const int32_t* sv = tab + (int64_t)(t0 + i) * cpad + kG * g;
-          b[i] = *std::min_element(sv, sv + kG);
-          f0 = std::min(f0, b[i]);
-          int32_t key[kG];
-          int sum = 0;
-          for (int q = 0; q < kG; ++q) {
-            const int64_t r = (int64_t)sv[q] - b[i];
-            if (r > 32767) return P;
-            key[q] = (int32_t)r;
-            sum += (int)r;
-          }
-          int p = 0;
-          while (p < ncls && !(csum[p] == sum && std::equal(key, key + kG, ckey[p]))) ++p;
-          if (p == ncls) {
-            if (ncls == kMaxCls) return P;
-            std::copy(key, key + kG, ckey[ncls]);
-            cmin[ncls] = cmax[ncls] = b[i];
-            csum[ncls] = sum;
-            ++ncls;
-          } else {
-            cmin[p] = std::min(cmin[p], b[i]);
-            cmax[p] = std::max(cmax[p], b[i]);
-          }
-          cls_of[i] = p;
+  const int want = std::min(ntiles, (int)std::min<int64_t>((int64_t)ntiles * nstages / 256 + 1, 8));
+  const int hw = (int)std::thread::hardware_concurrency();
+  const int nth = std::max(1, std::min(want, hw));
+  std::vector<Part> parts(nth);
+  auto run = [&](int k) {
+    Part& q = parts[k];
+    try {
+      StagePlan F;
+      const int a = (int)((int64_t)ntiles * k / nth), z = (int)((int64_t)ntiles * (k + 1) / nth);
+      q.len.reserve((size_t)(z - a) * nstages);
+      q.bytes.reserve((size_t)(z - a) * nstages * (sizeof(StageTab) + 18 * sizeof(ClsLink)));
+      for (int ti = a; ti < z && q.ok; ++ti)
+        for (int s = 0; s < nstages && q.ok; ++s) {
+          q.ok = plan_stage(tab, ti * D, std::min(D, ntr - ti * D), cpad, s, u16, tt, D, W,
+                            P.row_slot, F);
+          if (!q.ok) break;
+          const size_t len = sizeof(StageTab) + F.links * sizeof(ClsLink), at = q.bytes.size();
+          q.bytes.resize(at + len);
+          std::memcpy(q.bytes.data() + at, &F.st, sizeof(StageTab));
+          std::memcpy(q.bytes.data() + at + sizeof(StageTab), F.cls, F.links * sizeof(ClsLink));
+          q.len.push_back((uint32_t)len);
+          q.words = std::max(q.words, F.words);
         }
-        int order[kMaxCls], zoff[kMaxCls], zlens[kMaxCls], ulos[kMaxCls];
-        for (int p = 0; p < ncls; ++p) order[p] = p;
-        std::stable_sort(order, order + ncls, [&](int x, int y) { return csum[x] < csum[y]; });
-        for (int k = 0; k < ncls; ++k) {
-          const int p = order[k];
-          const int ulo = (cmin[p] - f0) / U;
-          if (ulo > 32767 || cmax[p] - f0 + tt > 65535) return P;
-          int un = (cmax[p] - f0 + tt + U - 1) / U - ulo;
-          if (u16) un += un & 1;  // 16-byte aligned classes
-          zoff[p] = words;
-          zlens[p] = un * U;
-          ulos[p] = ulo;
-          int32_t key[kG];  // walks from the preceding class to this one
-          std::copy(ckey[k > 0 ? prev : p], ckey[k > 0 ? prev : p] + kG, key);
-          auto at_row = [&](int q, int r) {
-            return 8u * es * (uint32_t)((gl * kG + q) * P.row_slot + f0 + r - xmin);
-          };
-          int dist = 0;
-          for (int q = 0; q < kG; ++q) dist += std::abs(ckey[p][q] - key[q]);
-          if (k == 0 || dist > kMaxSteps || nl - nl0 + dist + ncls - k - 1 > kMaxLinks) {
-            std::copy(ckey[p], ckey[p] + kG, key);  // a chain starts here
-            for (int q = 0; q < kG; ++q) F.cls[nl].off[q] = at_row(q, key[q]);
-            ++nl;
-          }
-          for (int q = 0; q < kG; ++q)
-            while (key[q] != ckey[p][q]) {
-              const bool up = ckey[p][q] > key[q];
-              F.cls[nl].step = (up ? kStepAdd : kStepSub) | at_row(q, up ? key[q] : key[q] - 1);
-              key[q] += up ? 1 : -1;
-              for (int c = 0; c < kG; ++c) F.cls[nl].off[c] = at_row(c, key[c]);
-              ++nl;
-            }
-          ClsLink& e = F.cls[nl - 1];
-          e.ev = 4 * (words - ulo * U / 2);
-          e.od = e.ev + 2 * zlens[p];
-          e.range = (uint32_t)ulo | (uint32_t)un << 16;
-          prev = p;
-          words += zlens[p];
-          if (words > 32767) return P;
-        }
-        for (int i = 0; i < n; ++i) {
-          const int p = cls_of[i], o = b[i] - f0 - ulos[p] * U;
-          st.zstart[gl][trial_slot(i, W, D / W)] =
-              (int16_t)(zoff[p] + (o % 2) * (zlens[p] / 2) + o / 2);
-        }
-        st.nlink[gl] = (uint8_t)(nl - nl0);
-      }
-      if (!deal_work(st, F.cls, W, cost)) return P;
-      zcap = std::max<int64_t>(zcap, words);
-      const size_t bytes = sizeof(StageTab) + nl * sizeof(ClsLink);
-      most = std::max(most, bytes);
-      const size_t i = (size_t)ti * nstages + s;
-      at[i + 1] = at[i] + bytes;
-      out.insert(out.end(), (uint8_t*)&F, (uint8_t*)&F + bytes);
+    } catch (const std::bad_alloc&) {
+      q.nomem = true;
     }
+  };
+  {
+    std::vector<std::thread> th;
+    th.reserve(nth);
+    int k = 1;
+    try {
+      for (; k < nth; ++k) th.emplace_back(run, k);
+    } catch (const std::system_error&) {  // no more threads: this one does the rest
+    }
+    run(0);
+    for (; k < nth; ++k) run(k);
+    for (auto& t : th) t.join();
   }
-  P.zcap = (int)((std::max<int64_t>(zcap, 4) + 3) / 4 * 4);
+  size_t most = 0;
+  int zcap = 4;
+  for (const Part& q : parts) {
+    if (q.nomem) throw std::bad_alloc();
+    if (!q.ok) return P;
+    for (uint32_t l : q.len) most = std::max<size_t>(most, l);
+    zcap = std::max(zcap, q.words);
+  }
+  P.zcap = (zcap + 3) / 4 * 4;
   P.tab_pitch = (int)most;
   P.tab_bytes = most * ntiles * nstages;
   P.tabs.resize(P.tab_bytes);
-  for (size_t i = 0; i + 1 < at.size(); ++i)
-    std::memcpy(P.tabs.data() + i * most, out.data() + at[i], at[i + 1] - at[i]);
+  uint8_t* to = P.tabs.data();
+  for (const Part& q : parts) {
+    const uint8_t* from = q.bytes.data();
+    for (uint32_t l : q.len) {
+      std::memcpy(to, from, l);
+      from += l;
+      to += most;
+    }
+  }
   // as many staging buffers as fit (4, else 3: a copy is then issued two stages ahead)
   const size_t limit = P.ctas == 2 ? kSmemLimit2 : kSmemLimit;
   for (int nst = kMaxNStage; nst >= 3 && !P.ok; --nst) {
@@ -1237,15 +1334,18 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
 }
 
 // Instances: uint8/uint16 data x 4/3 staging buffers x the tile shapes (outputs, trials,
-// threads): 512 x 64 with 512 or 1024 threads, 256 x 64 and 256 x 32 with 512.
+// threads): 512 x 64 with 512 or 1024 threads, 256 x 128, 256 x 64 and 256 x 32 with 512.
 #define DD_TILED_SHAPES(X, T, U16)                                                  \
   X(T, U16, 512, 4, 64, 512) X(T, U16, 512, 3, 64, 512) X(T, U16, 512, 4, 64, 1024) \
   X(T, U16, 512, 3, 64, 1024) X(T, U16, 256, 4, 64, 512) X(T, U16, 256, 3, 64, 512) \
+  X(T, U16, 256, 4, 128, 512) X(T, U16, 256, 3, 128, 512)                           \
   X(T, U16, 256, 4, 32, 512) X(T, U16, 256, 3, 32, 512)
 #define DD_TILED_INSTANCES(X) DD_TILED_SHAPES(X, uint8_t, 0) DD_TILED_SHAPES(X, uint16_t, 1)
-// The persistent form exists for the 64 x 512 tile with 16 warps (the shape every plan measured
-// so far runs fastest on).
+// The persistent form exists for the 64 x 512 and 128 x 256 tiles with 16 warps, the shapes a
+// plan chooses between.
 #define DD_PERSIST_INSTANCES(X)                                                   \
+  X(uint8_t, 0, 256, 4, 128, 512) X(uint8_t, 0, 256, 3, 128, 512)                 \
+  X(uint16_t, 1, 256, 4, 128, 512) X(uint16_t, 1, 256, 3, 128, 512)               \
   X(uint8_t, 0, 512, 4, 64, 512) X(uint8_t, 0, 512, 3, 64, 512)                   \
   X(uint16_t, 1, 512, 4, 64, 512) X(uint16_t, 1, 512, 3, 64, 512)
 
@@ -1504,7 +1604,7 @@ int fused_segments(int ntx, int ntt, int sms, int smax) {
 cudaError_t launch_fused(const TiledArgs& a, const FusedArgs& f, int is_u16, size_t smem,
                          cudaStream_t st) {
   if (a.nout <= 0 || a.n_trials <= 0) return cudaSuccess;
-  const int ntx = (a.n_trials + kMaxTileTrials - 1) / kMaxTileTrials;
+  const int ntx = (a.n_trials + kFusedTrials - 1) / kFusedTrials;
   const int ntt = (int)((a.nout + 511) / 512);
   if (f.nsegs < 1 || (int64_t)f.nsegs * f.seg_tiles < ntt ||
       (int64_t)(f.nsegs - 1) * f.seg_tiles >= ntt || f.hist < 1 || f.hist > 512 ||

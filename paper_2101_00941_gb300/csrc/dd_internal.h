@@ -166,7 +166,7 @@ struct PersistArgs {
 struct TiledPlan {
   bool ok = false;
   int tt = 0;
-  int trials = 0;          // trials per tile (64 or 32)
+  int trials = 0;          // trials per tile (128, 64 or 32)
   int threads = 0;         // threads per CTA (512 or 1024)
   int ctas = 0;            // CTAs per SM the tile shape is compiled for
   int nseg = 0;            // 128-byte segments per staged channel row
@@ -188,6 +188,10 @@ struct TiledPlan {
 
 TiledPlan tiled_plan(const int32_t* shifts, int ntr, int cpad, int decimation, int tt,
                      int trials, int threads);
+// Estimate of a shape's launch over a window of nout outputs, in instructions of a warp per SM,
+// from a sample of the range's stages (up to 4 trial tiles x 16 stages); < 0: does not fit.
+double tiled_cost(const int32_t* shifts, int ntr, int cpad, int decimation, int tt, int trials,
+                  int threads, int64_t nout, int sms);
 int64_t tiled_plan_check(const int32_t* shifts, int ntr, int cpad, int decimation, int tt,
                          int trials, int* ok);
 cudaError_t prepare_tiled(int is_u16, int tt, int nstage, int trials, int threads, size_t smem);
@@ -246,11 +250,12 @@ void plan_redirect_errors(dd_plan_s* plan, int32_t* err);
 struct DeferredTile {
   TiledArgs args;
   int32_t is_u16;
+  int32_t tt, trials;  // tile shape
   int32_t nstage;
   size_t smem;
 };
-// dd_run on stream `st`, except that the range launches of the 64 x 512 x 512 tile shape are
-// appended to *out instead of being made (every other launch is made as dd_run makes it).
+// dd_run on stream `st`, except that the range launches of the 64 x 512 and 128 x 256 tile shapes
+// with 512 threads are appended to *out instead of being made (every other launch is made as dd_run makes it).
 int run_deferred(dd_plan_s* plan, const uint8_t* chunk, int64_t nsamp, cudaStream_t st,
                  std::vector<DeferredTile>* out);
 // Serving support: make the next dd_run's dedispersion wait (once) for an event of another

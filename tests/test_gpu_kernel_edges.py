@@ -123,3 +123,24 @@ def test_corner_turn_any_start(nchans, offset):
             at += m
     finally:
         plan.close()
+
+
+@pytest.mark.parametrize("trials,sizes", [(1024, [10240, 10240]), (1000, [10240, 10238, 9000])])
+def test_wide_trial_tile(trials, sizes):
+    """Plans that take the 128-trial tile, for uint8 and uint16 data: full and ragged last tiles,
+    odd last windows, fifteen groups of channels (the last stage holds one)."""
+    ranges = (configs.DMRange(0.0, 0.05, trials, 1), configs.DMRange(50.0, 0.1, trials, 2))
+    w = configs.mid(nsamp=1 << 15, chunk_len=4096, n_streams=2, npulses=4, nchans=4096,
+                    ranges=ranges, index=74)
+    w.nchans, w.foff = 120, -300.0 / 4096
+    w.pulses = tuple(configs.PulseSpec(p.dm * 0.05, min(p.t_ref, 25000), p.width, p.amp * 6.0)
+                     for p in w.pulses)
+    x = w.generate(_arrivals(w))
+    plan = dd.Plan(w.freqs(), w.tsamp, w.ranges_array(), 10240, n_streams=1, max_width=256)
+    try:
+        for r in range(2):
+            assert plan.model(r, 512)["tile_trials"] == 128
+            assert plan.kernel(r) == (dd.DD_KERNEL_TILED, 256)
+    finally:
+        plan.close()
+    check(w, x[:sum(sizes)], sizes, 2)

@@ -86,3 +86,30 @@ def test_coarse_channels_and_bad_tables_are_refused():
     assert dd.dd_tiled_plan_check(mid, 1, 512) == (0, 0)
     with pytest.raises(dd.DDError):
         dd.dd_tiled_plan_check(np.zeros((4, 12), np.int32), 1, 512)  # 12 channels: not padded
+
+
+@pytest.mark.parametrize("tt,trials", SHAPES + [(256, 128)])
+@pytest.mark.parametrize("decimation", [1, 2, 16])
+def test_chains_on_jittered_tables(tt, trials, decimation):
+    """Delay tables whose groups' classes lie zero to many channel steps apart (chains with
+    in-between links, broken chains, one class): the plan is either refused or free of
+    violations, and the smooth tables are accepted."""
+    rng = np.random.default_rng(75)
+    accepted = 0
+    for jitter in (0.0, 0.3, 1.0, 2.0):
+        for ntr, cpad in ((130, 40), (64, 8), (1, 24)):
+            slope = np.linspace(0.9, 0.93, cpad)
+            t = np.arange(ntr)[:, None] * slope + rng.random(cpad) * 3
+            t = np.floor(t + jitter * rng.random((ntr, cpad)))
+            tab = np.maximum.accumulate(t, axis=0).astype(np.int32)
+            ok, bad = dd.dd_tiled_plan_check(tab, decimation, tt, trials)
+            assert bad == 0, (jitter, ntr, cpad)
+            accepted += ok
+            assert ok or jitter > 0
+    assert accepted > 3
+
+
+def test_128_trial_tile_on_the_workloads():
+    for w in (configs.mid(nsamp=1 << 17), configs.out_of_core(nsamp=1 << 20)):
+        for tab, r in list(zip(_tables(w), w.ranges))[::3]:
+            assert dd.dd_tiled_plan_check(tab, r.decimation, 256, 128) == (1, 0), r
