@@ -160,10 +160,12 @@ struct Slot {
 }  // namespace
 
 // How one range is dedispersed: the tiled delay-class kernel (with its tile shape, staging
-// buffers and shared-memory sizes) or, when the plan does not fit it, the direct kernel (the
+// buffers and shared-memory sizes) or, when the plan does not fit it, a direct kernel: the staged
+// one, or the cached-read one where 64 trials' delays spread too far for shared memory (the
 // one-thread-per-output kernel with DD_FLAG_NAIVE).
 struct RangeKernel {
   bool tiled = false;
+  int frame = 0;              // staged direct kernel: pair words per channel (0: not used)
   int tt = 0;
   int trials = 0;             // trials per tile
   int threads = 0;            // threads per CTA
@@ -751,6 +753,15 @@ int dd_plan(const double* freqs_mhz, int32_t nchans, double tsamp_s, const dd_ra
             return rc2;
           }
         }
+        RangeKernel& K = p->rk[r];
+        if (!K.tiled && ddk::staged_plan(rt, ranges[r].n_trials, p->Cp, ranges[r].decimation,
+                                         &K.frame)) {
+          const cudaError_t e2 = ddk::prepare_staged(ranges[r].decimation > 1);
+          if (e2 != cudaSuccess) {
+            free_plan(p);
+            return fail(DD_ERR_CUDA, "staged kernel set-up: %s", cudaGetErrorString(e2));
+          }
+        }
       }
     }
   }
@@ -1167,12 +1178,29 @@ static int run_impl(dd_plan_t p, const uint8_t* chunk, int64_t nsamp, void* cuda
       }
     } else if (p->opts.flags & DD_FLAG_NAIVE) {
       DD_CK(ddk::launch_dedisp_naive(R, p->Cp, st));
+    } else if (K.frame) {
+      ddk::StagedArgs A;
+      A.xd = R.xd;
+      A.xd_stride = R.xd_stride;
+      A.m0 = R.m0;
+      A.nout = R.nout;
+      A.y = R.y;
+      A.y_stride = R.y_stride;
+      A.mom = R.mom;
+      A.shifts = R.shifts;
+      A.n_trials = R.n_trials;
+      A.cpad = p->Cp;
+      A.frame = K.frame;
+      A.flush = 65535 / (8 * 255 * d);
+      int nl = 0;
+      DD_CK(ddk::launch_staged(A, R.is_u16, p->sms, st, &nl));
+      p->launches += nl;
     } else {
       DD_CK(ddk::launch_dedisp_direct(R, p->Cp, st));
     }
     rc = timing_end(p, st, ts);
     if (rc) return rc;
-    if (!K.tiled) {
+    if (!K.tiled && !K.frame) {
       DD_CK(ddk::launch_moments(R.y, R.n_trials, R.nout, R.y_stride, R.mom, st));
       p->launches += 2;
     }

@@ -628,6 +628,60 @@ __global__ void __launch_bounds__(512) k_fused_edges(const __grid_constant__ Til
   }
 }
 
+// A tile's outputs: the series (if `store`) and the exact moments. Lane l of warp v holds outputs
+// 2(l + 32k) and 2(l + 32k) + 1 of trials v, v + W, ... of the tile.
+template <int W, int kTPW, int KT>
+__device__ __forceinline__ void store_tile(const uint32_t (&acc)[kTPW][KT], int32_t* y,
+                                           int64_t y_stride, Moments* mom, int64_t nout,
+                                           int trial0, int ntr, int64_t j0, int warp, int lane,
+                                           bool store) {
+  constexpr int KP = KT / 2;
+#pragma unroll
+  for (int q = 0; q < kTPW; ++q) {
+    const int t = warp + W * q;
+    if (t < ntr) {
+      int32_t* yr = y + (int64_t)(trial0 + t) * y_stride;
+      unsigned long long s1 = 0, lo = 0, hi = 0;
+#pragma unroll
+      for (int k = 0; k < KP; ++k) {
+        const int64_t j = j0 + 2 * (lane + 32 * k);
+        if (!store) {
+        } else if (j + 1 < nout) {
+          *reinterpret_cast<int2*>(yr + j) = make_int2((int32_t)acc[q][2 * k],
+                                                       (int32_t)acc[q][2 * k + 1]);
+        } else if (j < nout) {
+          yr[j] = (int32_t)acc[q][2 * k];
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (j + h < nout) {
+            const uint32_t v = acc[q][2 * k + h];
+            s1 += v;
+            const unsigned long long sq = (unsigned long long)v * v;
+            lo += sq;
+            hi += (lo < sq) ? 1ull : 0ull;
+          }
+        }
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        const unsigned long long olo = __shfl_xor_sync(0xffffffffu, lo, off);
+        const unsigned long long ohi = __shfl_xor_sync(0xffffffffu, hi, off);
+        const unsigned long long nlo = lo + olo;
+        hi = hi + ohi + (nlo < lo ? 1ull : 0ull);
+        lo = nlo;
+      }
+      if (lane == 0) {
+        Moments* m = mom + trial0 + t;
+        atomicAdd(&m->s1, s1);
+        const unsigned long long old = atomicAdd(&m->s2lo, lo);
+        atomicAdd(&m->s2hi, hi + ((old + lo < old) ? 1ull : 0ull));
+      }
+    }
+  }
+}
+
 // Words 32k + lane of N trials' sequences in both groups (or, both = false, in the first) added
 // to the packed sums of trials q0 ..; tc: shared address of the trials' word offsets, zs: of the
 // stage's words at the lane.
@@ -783,52 +837,8 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
     return false;
   }
 
-  // ---- epilogue: series + exact moments
-#pragma unroll
-  for (int q = 0; q < kTPW; ++q) {
-    const int t = warp + W * q;
-    if (t < ntr) {
-      int32_t* yr = a.y + (int64_t)(trial0 + t) * a.y_stride;
-      unsigned long long s1 = 0, lo = 0, hi = 0;
-      const bool store = !FUSED || f->keep_series;
-#pragma unroll
-      for (int k = 0; k < KP; ++k) {
-        const int64_t j = j0 + 2 * (lane + 32 * k);
-        if (!store) {
-        } else if (j + 1 < a.nout) {
-          *reinterpret_cast<int2*>(yr + j) = make_int2((int32_t)acc[q][2 * k],
-                                                       (int32_t)acc[q][2 * k + 1]);
-        } else if (j < a.nout) {
-          yr[j] = (int32_t)acc[q][2 * k];
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (j + h < a.nout) {
-            const uint32_t v = acc[q][2 * k + h];
-            s1 += v;
-            const unsigned long long sq = (unsigned long long)v * v;
-            lo += sq;
-            hi += (lo < sq) ? 1ull : 0ull;
-          }
-        }
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-        const unsigned long long olo = __shfl_xor_sync(0xffffffffu, lo, off);
-        const unsigned long long ohi = __shfl_xor_sync(0xffffffffu, hi, off);
-        const unsigned long long nlo = lo + olo;
-        hi = hi + ohi + (nlo < lo ? 1ull : 0ull);
-        lo = nlo;
-      }
-      if (lane == 0) {
-        Moments* m = a.mom + trial0 + t;
-        atomicAdd(&m->s1, s1);
-        const unsigned long long old = atomicAdd(&m->s2lo, lo);
-        atomicAdd(&m->s2hi, hi + ((old + lo < old) ? 1ull : 0ull));
-      }
-    }
-  }
+  store_tile<W, kTPW, KT>(acc, a.y, a.y_stride, a.mom, a.nout, trial0, ntr, j0, warp, lane,
+                          !FUSED || f->keep_series);
   if constexpr (FUSED)
     fused_search<TT, W, kTPW, KT>(a, *f, acc, smem, bx, by, first, trial0, ntr, j0, warp, lane);
   return true;
@@ -888,6 +898,195 @@ __global__ void __launch_bounds__(512, 1)
   for (int y = y0; y < y1; ++y)
     if (!tile_body<T, 512, NS, 64, 512, true>(a, blockIdx.x, y, smem, y > y0, &f, y == y0))
       break;  // a bounded wait ran out (uniform): the error bit is set
+}
+
+// ---- staged direct kernel: ranges without shared delay classes (coarse channels, whose
+// neighbouring trials differ by several samples within a group, or decimation above x16)
+//
+// CTA (x, y): 64 trials x 512 outputs, 16 warps, warp v the trials v, v + 16, ... of the tile as in
+// the tiled kernel. Per stage of kSC channels the rows' windows (512 samples plus the tile's delay
+// spread) come to shared memory by 16-byte asynchronous copies, are turned once into single-channel
+// pair words x[v] | x[v + 1] << 16 in an even and an odd plane, and every trial adds the words of
+// its own offset: one 32-bit shared-memory load per two channel-adds, conflict free, into packed
+// 16-bit sums that go to the 32-bit outputs before they can overflow. Bound by the shared-memory
+// pipe at 64 channel-adds per SM-clock; reading each trial's samples through the read-only cache
+// with funnel shifts (k_dedisp_direct) was bound by instruction issue at about half of that (256
+// channels of 1.6 MHz, 800 trials x 131072 at x1 and 400 at x2: 5.47 -> 3.00 ms, 1.1e13 channel-adds
+// per second).
+// Copies of stage s + 2, words of stage s + 1 and sums of stage s share one barrier per stage.
+// Where the tiles are too few for the chip, blockIdx.z takes a share of the channels and the
+// shares' sums are added to a zeroed series.
+constexpr int kSC = 8;        // channels per stage
+constexpr int kStTrials = 64, kStOut = 512;
+
+struct StagedLayout {
+  size_t z, off, total;
+  int row;  // bytes of a staged row
+};
+
+// frame: pair words per channel, a multiple of 8; the raw rows come first
+__host__ __device__ inline StagedLayout staged_layout(int es, int frame) {
+  StagedLayout L;
+  L.row = (int)align16((size_t)(frame + 16) * es);
+  L.z = (size_t)2 * kSC * L.row;
+  L.off = L.z + (size_t)2 * kSC * frame * 4;
+  L.total = L.off + (size_t)2 * kStTrials * kSC * 4;
+  return L;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(512, 1) k_dedisp_staged(const StagedArgs a) {
+  constexpr int es = (int)sizeof(T);
+  constexpr int kTPW = kStTrials / 16, KT = kStOut / 32, KP = kStOut / 64;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const StagedLayout SL = staged_layout(es, a.frame);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int trial0 = blockIdx.x * kStTrials;
+  const int ntr = min(kStTrials, a.n_trials - trial0);
+  const int64_t j0 = (int64_t)blockIdx.y * kStOut;
+  const int all = a.cpad / kSC;  // stages; this CTA's: sb .. sb + nstages - 1
+  const int sb = (int)((int64_t)all * blockIdx.z / gridDim.z);
+  const int nstages = (int)((int64_t)all * (blockIdx.z + 1) / gridDim.z) - sb;
+  uint32_t sraw = smem_addr(smem);
+  asm volatile("" : "+r"(sraw));
+  const uint32_t sz = sraw + (uint32_t)SL.z, soff = sraw + (uint32_t)SL.off;
+  const uint32_t zbytes = (uint32_t)(kSC * a.frame * 4);
+  // the tile's smallest delays
+  const int32_t* first = a.shifts + (int64_t)trial0 * a.cpad + sb * kSC;
+
+  // copies: 64 threads per row
+  const int crow = tid >> 6, cchunk = tid & 63;
+  auto copy_rows = [&](int s, int32_t sfirst) {
+    const int64_t byte = (a.m0 + j0 + sfirst) * es & ~(int64_t)15;
+    const unsigned char* src = static_cast<const unsigned char*>(a.xd) +
+                               (int64_t)((sb + s) * kSC + crow) * a.xd_stride * es + byte;
+    const uint32_t dst = sraw + (uint32_t)((s & 1) * kSC + crow) * (uint32_t)SL.row;
+    for (int c = 16 * cchunk; c < SL.row; c += 16 * 64)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + c), "l"(src + c)
+                   : "memory");
+  };
+  // offsets: thread (trial, channel); byte offset of the trial's words in the stage's planes
+  const int ot = tid >> 3, oc = tid & 7;
+  auto offset = [&](int32_t st, int32_t sf) {
+    const int ph = (int)(((a.m0 + j0 + sf) * es & 15) / es);
+    const int o = (ot < ntr ? st - sf : 0) + ph;
+    return (uint32_t)(oc * a.frame * 4 + (o & 1) * a.frame * 2 + (o >> 1) * 4);
+  };
+  const int32_t* myrow = a.shifts + (int64_t)(trial0 + min(ot, ntr - 1)) * a.cpad + sb * kSC + oc;
+  auto build = [&](int s) {
+    // each warp half a channel's units: one row word per unit and the next one
+    const int ch = warp >> 1;
+    const uint32_t row = sraw + (uint32_t)((s & 1) * kSC + ch) * (uint32_t)SL.row;
+    const uint32_t ev = sz + (s & 1) * zbytes + (uint32_t)(ch * a.frame * 4);
+    const uint32_t od = ev + (uint32_t)a.frame * 2;
+    constexpr int U = 4 / es;  // samples per row word
+    for (int u = (warp & 1) * 32 + lane; u * U < a.frame; u += 64) {
+      const uint32_t w0 = lds<0>(row + 4 * u), w1 = lds<4>(row + 4 * u);
+      if constexpr (es == 1) {
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(ev + 8 * u),
+                     "r"(__byte_perm(w0, 0, 0x4140)), "r"(__byte_perm(w0, 0, 0x4342))
+                     : "memory");
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(od + 8 * u),
+                     "r"(__byte_perm(w0, 0, 0x4241)),
+                     "r"(__byte_perm(__funnelshift_r(w0, w1, 24), 0, 0x4140))
+                     : "memory");
+      } else {
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(ev + 4 * u), "r"(w0) : "memory");
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(od + 4 * u), "r"(__byte_perm(w0, w1, 0x5432))
+                     : "memory");
+      }
+    }
+  };
+  auto put_offset = [&](int s, uint32_t v) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(soff + (uint32_t)((s & 1) * 512 + tid) * 4u),
+                 "r"(v)
+                 : "memory");
+  };
+
+  // prologue: rows of stages 0 and 1, words and offsets of stage 0
+  copy_rows(0, __ldg(first + crow));
+  if (nstages > 1) copy_rows(1, __ldg(first + kSC + crow));
+  put_offset(0, offset(__ldg(myrow), __ldg(first + oc)));
+  int32_t nst = 0, nsf = 0, ncf = 0;  // delays for the next offsets and the next copy
+  if (nstages > 1) nst = __ldg(myrow + kSC), nsf = __ldg(first + kSC + oc);
+  if (nstages > 2) ncf = __ldg(first + 2 * kSC + crow);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  build(0);
+  __syncthreads();
+
+  uint32_t acc[kTPW][KT], pk[kTPW][KP];
+#pragma unroll
+  for (int q = 0; q < kTPW; ++q) {
+#pragma unroll
+    for (int k = 0; k < KT; ++k) acc[q][k] = 0;
+#pragma unroll
+    for (int k = 0; k < KP; ++k) pk[q][k] = 0;
+  }
+  int left = a.flush;
+  for (int s = 0; s < nstages; ++s) {
+    if (s + 2 < nstages) {
+      copy_rows(s + 2, ncf);  // into the rows of stage s, whose words are built
+      if (s + 3 < nstages) ncf = __ldg(first + (s + 3) * kSC + crow);
+    }
+    if (s + 1 < nstages) {
+      put_offset(s + 1, offset(nst, nsf));
+      if (s + 2 < nstages)
+        nst = __ldg(myrow + (s + 2) * kSC), nsf = __ldg(first + (s + 2) * kSC + oc);
+      build(s + 1);
+    }
+    const uint32_t zs = sz + (s & 1) * zbytes + 4u * lane;
+#pragma unroll
+    for (int q = 0; q < kTPW; ++q) {
+      const uint32_t ob = soff + (uint32_t)((s & 1) * 512 + (warp + 16 * q) * kSC) * 4u;
+      const uint4 oa = lds128(ob), oz = lds128(ob + 16);
+      const uint32_t zp[kSC] = {zs + oa.x, zs + oa.y, zs + oa.z, zs + oa.w,
+                                zs + oz.x, zs + oz.y, zs + oz.z, zs + oz.w};
+      if (a.flush > 0) {
+#pragma unroll
+        for (int c = 0; c < kSC; c += 2)
+#pragma unroll
+          for (int k = 0; k < KP; ++k)
+            pk[q][k] += lds<0>(zp[c] + 128 * k) + lds<0>(zp[c + 1] + 128 * k);
+      } else {  // eight channels' sum does not fit a 16-bit lane
+#pragma unroll 1
+        for (int c = 0; c < kSC; ++c) {
+          const uint32_t z = zs + lds<0>(ob + 4 * c);
+#pragma unroll
+          for (int k = 0; k < KP; ++k)
+            pair_add(lds<0>(z + 128 * k), acc[q][2 * k], acc[q][2 * k + 1]);
+        }
+      }
+    }
+    if (a.flush > 0 && (--left == 0 || s + 1 == nstages)) {
+      left = a.flush;
+#pragma unroll
+      for (int k = 0; k < KP; ++k)
+#pragma unroll
+        for (int q = 0; q < kTPW; ++q) {
+          pair_add(pk[q][k], acc[q][2 * k], acc[q][2 * k + 1]);
+          pk[q][k] = 0;
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+  }
+  if (gridDim.z > 1) {  // moments follow from the complete series
+#pragma unroll
+    for (int q = 0; q < kTPW; ++q) {
+      const int t = warp + 16 * q;
+      if (t >= ntr) continue;
+      int32_t* yr = a.y + (int64_t)(trial0 + t) * a.y_stride;
+#pragma unroll
+      for (int k = 0; k < KP; ++k) {
+        const int64_t j = j0 + 2 * (lane + 32 * k);
+        if (j < a.nout) atomicAdd(yr + j, (int32_t)acc[q][2 * k]);
+        if (j + 1 < a.nout) atomicAdd(yr + j + 1, (int32_t)acc[q][2 * k + 1]);
+      }
+    }
+    return;
+  }
+  store_tile<16, kTPW, KT>(acc, a.y, a.y_stride, a.mom, a.nout, trial0, ntr, j0, warp, lane, true);
 }
 
 template <typename T, int TT, int NS, int D, int NT>
@@ -1621,6 +1820,65 @@ cudaError_t launch_fused(const TiledArgs& a, const FusedArgs& f, int is_u16, siz
   const size_t esmem = (size_t)(512 / 32) * 2 * f.hist * sizeof(uint32_t);
   k_fused_edges<<<dim3((unsigned)ntx * 4, (unsigned)(f.nsegs - 1)), 512, esmem, st>>>(a, f);
   return cudaGetLastError();
+}
+
+int staged_plan(const int32_t* tab, int ntr, int cpad, int decimation, int* frame) {
+  if (cpad % kSC) return 0;
+  int64_t spread = 0;
+  for (int t0 = 0; t0 < ntr; t0 += kStTrials) {
+    const int n = std::min(kStTrials, ntr - t0);
+    for (int i = 0; i < n; ++i)
+      for (int c = 0; c < cpad; ++c) {
+        const int64_t o = (int64_t)tab[(int64_t)(t0 + i) * cpad + c] - tab[(int64_t)t0 * cpad + c];
+        if (o < 0) return 0;
+        spread = std::max(spread, o);
+      }
+  }
+  // a row may start up to 15 samples before the tile's first one
+  const int64_t f = (spread + 15 + kStOut + 7) / 8 * 8;
+  if (f > 4096) return 0;
+  const int es = decimation > 1 ? 2 : 1;
+  if (staged_layout(es, (int)f).total > kSmemLimit) return 0;
+  *frame = (int)f;
+  return 1;
+}
+
+cudaError_t prepare_staged(int is_u16) {
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  return is_u16 ? cudaFuncSetAttribute(k_dedisp_staged<uint16_t>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, optin)
+                : cudaFuncSetAttribute(k_dedisp_staged<uint8_t>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+}
+
+cudaError_t launch_staged(const StagedArgs& a, int is_u16, int sms, cudaStream_t st,
+                          int* launches) {
+  *launches = 0;
+  if (a.nout <= 0 || a.n_trials <= 0) return cudaSuccess;
+  dim3 grid((unsigned)((a.n_trials + kStTrials - 1) / kStTrials),
+            (unsigned)((a.nout + kStOut - 1) / kStOut), 1);
+  // shares of at least four stages while the chip has room for them
+  const int64_t ctas = (int64_t)grid.x * grid.y;
+  if (2 * ctas <= sms) grid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>(sms / ctas, a.cpad / kSC / 4));
+  const size_t smem = staged_layout(is_u16 ? 2 : 1, a.frame).total;
+  cudaError_t e = cudaSuccess;
+  if (grid.z > 1)
+    e = cudaMemset2DAsync(a.y, a.y_stride * sizeof(int32_t), 0, a.nout * sizeof(int32_t),
+                          a.n_trials, st);
+  if (e != cudaSuccess) return e;
+  if (is_u16) k_dedisp_staged<uint16_t><<<grid, 512, smem, st>>>(a);
+  else k_dedisp_staged<uint8_t><<<grid, 512, smem, st>>>(a);
+  *launches = 1;
+  e = cudaGetLastError();
+  if (e == cudaSuccess && grid.z > 1) {
+    e = launch_moments(a.y, a.n_trials, a.nout, a.y_stride, a.mom, st);
+    *launches = 2;
+  }
+  return e;
 }
 
 cudaError_t launch_tiled(const TiledArgs& a, int is_u16, int tt, int D, int nt,

@@ -106,6 +106,22 @@ struct TiledArgs {
   CUtensorMap rows;        // the ring as [Cp][xd_stride / seg][seg] (make_ring_map)
 };
 
+// Arguments of the staged direct kernel (dd_dedisp.cu), one launch per range.
+struct StagedArgs {
+  const void* xd;          // decimated ring, uint8 (d == 1) or uint16, [Cp][xd_stride]
+  int64_t xd_stride;       // elements
+  int64_t m0;              // ring column of window sample 0
+  int64_t nout;            // window length
+  int32_t* y;              // [n_trials][y_stride]
+  int64_t y_stride;
+  Moments* mom;            // [n_trials], zeroed before the launch
+  const int32_t* shifts;   // [n_trials][Cp], non-decreasing in the trial index
+  int32_t n_trials;
+  int32_t cpad;
+  int32_t frame;           // pair words per channel (staged_plan)
+  int32_t flush;           // stages whose sums fit the packed 16-bit lanes: 65535 / (8 * 255 * d)
+};
+
 // Search fused into the tiled kernel (64 x 512 tiles, 16 warps): one CTA walks a segment of
 // consecutive time tiles of one trial tile and, after each tile, records per (trial, width,
 // peak block) the block's largest boxcar sum and its earliest sample. Boxcars that reach back
@@ -218,6 +234,14 @@ int fused_segments(int ntx, int ntt, int sms, int smax);
 cudaError_t launch_fused(const TiledArgs& a, const FusedArgs& f, int is_u16, size_t smem,
                          cudaStream_t st);
 cudaError_t launch_sps_fused(const SpsFusedArgs& a, cudaStream_t st);
+
+// Whether a range's delays fit the staged direct kernel (no delay falls with the trial, and the
+// rows of 64 trials fit shared memory); *frame: StagedArgs::frame.
+int staged_plan(const int32_t* shifts, int ntr, int cpad, int decimation, int* frame);
+cudaError_t prepare_staged(int is_u16);
+// *launches: kernels launched (more than one where few tiles split the channels among CTAs).
+cudaError_t launch_staged(const StagedArgs& a, int is_u16, int sms, cudaStream_t st,
+                          int* launches);
 
 // Tensor map of a channel-major ring (uint8, or uint16 when is_u16) for the tiled kernel's
 // stage copies: dims {128-byte segment, segments per row, cpad rows}, box {segment, nseg, 16}.

@@ -125,6 +125,30 @@ def test_corner_turn_any_start(nchans, offset):
         plan.close()
 
 
+@pytest.mark.parametrize("nchans,trials,sizes", [
+    (200, 70, [4096, 4096]),    # few tiles: the channels split among CTAs
+    (200, 70, [4096, 1280, 256]),
+    (41, 2500, [2048, 2048]),   # 40 trial tiles: whole channel sums, seven padding channels
+])
+def test_staged_direct_kernel(nchans, trials, sizes):
+    """Coarse channels at x1, x2, x32 (last decimation whose eight-channel sums are packed), x64
+    and x256: every series and moment."""
+    ranges = (configs.DMRange(0.0, 0.5, trials, 1), configs.DMRange(10.0, 1.0, 65, 2),
+              configs.DMRange(20.0, 4.0, 20, 32), configs.DMRange(30.0, 8.0, 9, 64),
+              configs.DMRange(40.0, 20.0, 3, 256))
+    if trials > 1000:
+        ranges = (configs.DMRange(0.0, 0.02, trials, 1), configs.DMRange(10.0, 1.0, 65, 64))
+    w = _coarse(ranges, nchans, 1 << 13, 73)
+    w.widths = (1, 4, 64, 256)
+    x = w.generate(_arrivals(w))
+    plan = dd.Plan(w.freqs(), w.tsamp, w.ranges_array(), 4096, n_streams=1, max_width=256)
+    try:
+        assert plan.kernel(0)[0] == plan.kernel(len(ranges) - 1)[0] == dd.DD_KERNEL_DIRECT
+    finally:
+        plan.close()
+    check(w, x[:sum(sizes)], sizes, 1)
+
+
 @pytest.mark.parametrize("trials,sizes", [(1024, [10240, 10240]), (1000, [10240, 10238, 9000])])
 def test_wide_trial_tile(trials, sizes):
     """Plans that take the 128-trial tile, for uint8 and uint16 data: full and ragged last tiles,
