@@ -889,20 +889,24 @@ __global__ void __launch_bounds__(kSpsThreads) k_sps_fused(const SpsFusedArgs a)
 // deviation (FP64, one rounding per operation, as the oracle). A width whose previous step has no
 // values or no variance keeps its statistics.
 //
-// Each step sweeps the series once per group of at most kClipGroup widths, each warp over its own
-// eighth of the window (SpsRow). The bounds are whole numbers, so a value is tested and summed as
-// x = B - lo <= hi - lo in 32-bit integers, and the sums of B and B^2 follow exactly from the
-// count and the sums of x and x^2. Bound by instruction issue: about 7 instructions per value,
-// where the test in FP64 was bound by the FP64 pipe.
-constexpr int kClipGroup = 6;
+// Each step sweeps the series once, each warp over its own eighth of the window (SpsRow). The
+// bounds are whole numbers, so a value is tested and summed as x = B - lo <= hi - lo in 32-bit
+// integers, and the sums of B and B^2 follow exactly from the count and the sums of x and x^2. A
+// lane's sums of a width wait in shared memory between passes, so the width loop stays rolled:
+// unrolled over widths with the sums in registers it outgrew the instruction cache and took 18
+// instructions a value (4.2 ms for the 1024-channel beam's three ranges, 9 widths x 4 sweeps, 2.9 so; in
+// FP64 it was bound by the FP64 pipe, 44 ms).
+struct ClipSum {
+  unsigned long long c1, c2;  // sums of x and (low half) of x^2
+};
 
-__global__ void __launch_bounds__(kSpsThreads, 2) k_clip_stats(const ClipArgs a) {
+__global__ void __launch_bounds__(kSpsThreads, 3) k_clip_stats(const ClipArgs a) {
   extern __shared__ __align__(16) uint32_t Ps[];
   __shared__ uint32_t lo_b[kMaxWidths], span_b[kMaxWidths];  // values lo .. lo + span
   __shared__ int live[kMaxWidths];                           // 0: statistics final
   __shared__ int some[kMaxWidths];  // 0: the bounds hold no value; 1; 2: 64-bit sums suffice
   __shared__ WidthStats st[kMaxWidths];
-  __shared__ unsigned long long red[kClipGroup][4][kSpsWarps];
+  __shared__ unsigned long long red[kMaxWidths][4][kSpsWarps];
 
   const int32_t i = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -917,13 +921,20 @@ __global__ void __launch_bounds__(kSpsThreads, 2) k_clip_stats(const ClipArgs a)
   R.lane = lane;
   R.vec = (reinterpret_cast<uintptr_t>(R.y) & 15) == 0;
   const uint32_t* P = R.P;
+  // this lane's sums of width k: sums[32 k], cnts[32 k] (count; carries of c2 in cnts[32 (nw + k)])
+  ClipSum* sums = reinterpret_cast<ClipSum*>(Ps + (size_t)kSpsWarps * sps_row_words(H)) +
+                  (size_t)wid * nw * 32 + lane;
+  uint32_t* cnts = reinterpret_cast<uint32_t*>(
+                       reinterpret_cast<ClipSum*>(Ps + (size_t)kSpsWarps * sps_row_words(H)) +
+                       (size_t)kSpsWarps * nw * 32) +
+                   (size_t)wid * nw * 64 + lane;
   const long long per = ((n + kSpsWarps - 1) / kSpsWarps + 127) / 128 * 128;
   const long long s0 = min(n, wid * per), s1 = min(n, s0 + per);
-  // a lane's sums of squares over its part of a sweep stay below 2^64, its sums of four values
+  // a lane's sums of squares over its part of a sweep stay below 2^64, its sums over a pass
   // below 2^32
   const double lane_values = 16.0 * (double)((per + kSpsPass - 1) / kSpsPass);
   auto narrow = [&](uint32_t span) {
-    return (double)span * (double)span * lane_values < 1.8e19 && span < (1u << 30);
+    return (double)span * (double)span * lane_values < 1.8e19 && span < (1u << 28);
   };
   if (tid < kMaxWidths) {
     lo_b[tid] = 0u;  // step 0: every value (all boxcar sums are >= 0)
@@ -933,144 +944,143 @@ __global__ void __launch_bounds__(kSpsThreads, 2) k_clip_stats(const ClipArgs a)
     st[tid] = WidthStats{0, 0, 0, 0};
   }
   __syncthreads();
-  const int ngrp = (nw + kClipGroup - 1) / kClipGroup, per_grp = (nw + ngrp - 1) / ngrp;
   for (int step = 0; step <= a.iters; ++step) {
-    for (int g0 = 0; g0 < nw; g0 += per_grp) {
-      const int ng = min(per_grp, nw - g0);
-      bool any = false;
-      for (int k = g0; k < g0 + ng; ++k) any |= live[k] != 0;
-      if (!any) continue;  // uniform: every thread reads the same flags
-      uint32_t cn[kClipGroup], c2h[kClipGroup];
-      unsigned long long c1[kClipGroup], c2l[kClipGroup];
-#pragma unroll
-      for (int kk = 0; kk < kClipGroup; ++kk) cn[kk] = c2h[kk] = 0, c1[kk] = c2l[kk] = 0;
-      if (s0 < s1) {
-        uint4 nv[4];
-        R.load_pass(s0, nv);
-        uint32_t run = R.history(s0);
-        for (long long j0 = s0; j0 < s1; j0 += kSpsPass) {
-          uint4 v[4] = {nv[0], nv[1], nv[2], nv[3]};
-          run = R.scan(v, run);
-          R.store_pass(v);
-          __syncwarp();
-          if (j0 + kSpsPass < s1) R.load_pass(j0 + kSpsPass, nv);
-          const bool interior = j0 >= wmax - 1 && j0 + kSpsPass <= s1;
-#pragma unroll
-          for (int kk = 0; kk < kClipGroup; ++kk) {
-            if (kk >= ng) break;
-            const int k = g0 + kk;
-            if (!live[k] || !some[k]) continue;  // uniform
-            const int w = a.wd[k];
-            const uint32_t lo = lo_b[k], span = span_b[k];
+    bool any = false;
+    for (int k = 0; k < nw; ++k) any |= live[k] != 0;
+    if (!any) break;  // uniform: every thread reads the same flags
+    for (int k = 0; k < nw; ++k) {
+      sums[32 * k] = ClipSum{0, 0};
+      cnts[32 * k] = cnts[32 * (nw + k)] = 0;
+    }
+    if (s0 < s1) {
+      uint4 nv[4];
+      R.load_pass(s0, nv);
+      uint32_t run = R.history(s0);
+      for (long long j0 = s0; j0 < s1; j0 += kSpsPass) {
+        uint4 v[4] = {nv[0], nv[1], nv[2], nv[3]};
+        run = R.scan(v, run);
+        R.store_pass(v);
+        __syncwarp();
+        if (j0 + kSpsPass < s1) R.load_pass(j0 + kSpsPass, nv);
+        const bool interior = j0 >= wmax - 1 && j0 + kSpsPass <= s1;
+#pragma unroll 1
+        for (int k = 0; k < nw; ++k) {
+          const int how = live[k] ? some[k] : 0;
+          if (how == 0) continue;  // uniform
+          const int w = a.wd[k];
+          const uint32_t lo = lo_b[k], span = span_b[k];
+          ClipSum c = sums[32 * k];
+          uint32_t cn = cnts[32 * k];
+          if (how == 2 && interior) {
+            uint32_t sum = 0;
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
               const uint4 s4 = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
-              uint32_t x[4] = {v[g].x - s4.x - lo, v[g].y - s4.y - lo, v[g].z - s4.z - lo,
-                               v[g].w - s4.w - lo};
-              bool in[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) in[e] = x[e] <= span;
-              if (!interior) {
-                const long long j = j0 + 4 * lane + 128 * g;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) in[e] = in[e] && j + e < s1 && j + e >= w - 1;
-              }
-              if (some[k] == 2) {
-                uint32_t sum = 0;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const uint32_t m = in[e] ? x[e] : 0u;
-                  cn[kk] += in[e] ? 1u : 0u;
-                  sum += m;
-                  c2l[kk] += (unsigned long long)m * m;
-                }
-                c1[kk] += sum;
-                continue;
-              }
-              unsigned long long sum = 0, sq = 0;  // four values below 2^31: sq below 2^64
+              const uint32_t x[4] = {v[g].x - s4.x - lo, v[g].y - s4.y - lo, v[g].z - s4.z - lo,
+                                     v[g].w - s4.w - lo};
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                const uint32_t m = in[e] ? x[e] : 0u;
-                cn[kk] += in[e] ? 1u : 0u;
+                const uint32_t m = x[e] <= span ? x[e] : 0u;
+                if (x[e] <= span) ++cn;
                 sum += m;
-                sq += (unsigned long long)m * m;
+                c.c2 += (unsigned long long)m * m;
               }
-              c1[kk] += sum;
-              c2l[kk] += sq;
-              c2h[kk] += (c2l[kk] < sq) ? 1u : 0u;
             }
+            c.c1 += sum;
+          } else {
+            uint32_t carry = 0;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              const uint4 s4 = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
+              const uint32_t x[4] = {v[g].x - s4.x - lo, v[g].y - s4.y - lo, v[g].z - s4.z - lo,
+                                     v[g].w - s4.w - lo};
+              const long long j = j0 + 4 * lane + 128 * g;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const bool in = x[e] <= span && j + e < s1 && j + e >= w - 1;
+                const uint32_t m = in ? x[e] : 0u;
+                const unsigned long long sq = (unsigned long long)m * m;
+                if (in) ++cn;
+                c.c1 += m;
+                c.c2 += sq;
+                carry += c.c2 < sq ? 1u : 0u;
+              }
+            }
+            if (carry) cnts[32 * (nw + k)] += carry;
           }
-          __syncwarp();  // every read of this pass's P is done
-          if (j0 + kSpsPass < s1) R.carry();
+          sums[32 * k] = c;
+          cnts[32 * k] = cn;
         }
+        __syncwarp();  // every read of this pass's P is done
+        if (j0 + kSpsPass < s1) R.carry();
       }
-      // CTA sums of the group's widths: warp butterflies, then one thread per width
-#pragma unroll
-      for (int kk = 0; kk < kClipGroup; ++kk) {
-        if (kk >= ng) break;
-        unsigned long long x0 = cn[kk], x1 = c1[kk], lo = c2l[kk], hi = c2h[kk];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          x0 += __shfl_xor_sync(0xffffffffu, x0, off);
-          x1 += __shfl_xor_sync(0xffffffffu, x1, off);
-          const unsigned long long olo = __shfl_xor_sync(0xffffffffu, lo, off);
-          const unsigned long long ohi = __shfl_xor_sync(0xffffffffu, hi, off);
-          const unsigned long long nlo = lo + olo;
-          hi = hi + ohi + (nlo < lo ? 1ull : 0ull);
-          lo = nlo;
-        }
-        if (lane == 0) {
-          red[kk][0][wid] = x0;
-          red[kk][1][wid] = x1;
-          red[kk][2][wid] = lo;
-          red[kk][3][wid] = hi;
-        }
-      }
-      __syncthreads();
-      if (tid < ng && live[g0 + tid]) {
-        unsigned long long c = 0, x1 = 0, lo = 0, hi = 0;
-        for (int q = 0; q < kSpsWarps; ++q) {
-          c += red[tid][0][q];
-          x1 += red[tid][1][q];
-          const unsigned long long nlo = lo + red[tid][2][q];
-          hi = hi + red[tid][3][q] + (nlo < lo ? 1ull : 0ull);
-          lo = nlo;
-        }
-        // sums of B = x + l over c values: T1 = X1 + c l, T2 = X2 + 2 l X1 + c l^2 (128 bits)
-        const unsigned long long l = lo_b[g0 + tid];
-        const unsigned long long t1 = x1 + c * l;
-        const unsigned long long a0 = 2 * l * x1, a1 = __umul64hi(2 * l, x1);
-        const unsigned long long b0 = l * l * c, b1 = __umul64hi(l * l, c);
-        unsigned long long r0 = lo + a0, r1 = hi + a1 + (r0 < lo ? 1ull : 0ull);
-        r1 += b1 + (r0 + b0 < r0 ? 1ull : 0ull);
-        r0 += b0;
-        st[g0 + tid] = WidthStats{(long long)c, (long long)t1, r0, r1};
-      }
-      __syncthreads();
     }
-    // bounds of the next step from this step's statistics
-    if (step < a.iters && tid < nw && live[tid]) {
-      const WidthStats s = st[tid];
-      const unsigned long long un = (unsigned long long)s.n, ut1 = (unsigned long long)s.t1;
-      const unsigned long long p_lo = un * s.t2lo;
-      const unsigned long long p_hi = __umul64hi(un, s.t2lo) + un * s.t2hi;
-      const unsigned long long q_lo = ut1 * ut1, q_hi = __umul64hi(ut1, ut1);
-      const unsigned long long v_lo = p_lo - q_lo;
-      const unsigned long long v_hi = p_hi - q_hi - (p_lo < q_lo ? 1ull : 0ull);
-      if (s.n == 0 || (v_lo | v_hi) == 0) {
-        live[tid] = 0;
-      } else {
-        const double dn = __ll2double_rn(s.n);
-        const double mu = __ddiv_rn(__ll2double_rn(s.t1), dn);
-        const double sd = __ddiv_rn(__dsqrt_rn(u128_to_f64(v_hi, v_lo)), dn);
-        const double ks = __dmul_rn(a.kappa, sd);
-        const double lo = ceil(__dsub_rn(mu, ks)), hi = floor(__dadd_rn(mu, ks));
-        // the whole-number bounds on values 0 .. 2^31 - 1
-        const double top = 2147483647.0;
-        const uint32_t l = lo <= 0.0 ? 0u : (lo <= top ? (uint32_t)lo : 0u);
-        lo_b[tid] = l;
-        span_b[tid] = hi >= top ? 0x7FFFFFFFu - l : (hi >= (double)l ? (uint32_t)hi - l : 0u);
-        some[tid] = lo <= top && hi >= 0.0 && lo <= hi ? (narrow(span_b[tid]) ? 2 : 1) : 0;
+    // CTA sums of the widths: warp butterflies, then one thread per width
+#pragma unroll 1
+    for (int k = 0; k < nw; ++k) {
+      unsigned long long x0 = cnts[32 * k], x1 = sums[32 * k].c1, lo = sums[32 * k].c2;
+      unsigned long long hi = cnts[32 * (nw + k)];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        x0 += __shfl_xor_sync(0xffffffffu, x0, off);
+        x1 += __shfl_xor_sync(0xffffffffu, x1, off);
+        const unsigned long long olo = __shfl_xor_sync(0xffffffffu, lo, off);
+        const unsigned long long ohi = __shfl_xor_sync(0xffffffffu, hi, off);
+        const unsigned long long nlo = lo + olo;
+        hi = hi + ohi + (nlo < lo ? 1ull : 0ull);
+        lo = nlo;
+      }
+      if (lane == 0) {
+        red[k][0][wid] = x0;
+        red[k][1][wid] = x1;
+        red[k][2][wid] = lo;
+        red[k][3][wid] = hi;
+      }
+    }
+    __syncthreads();
+    if (tid < nw && live[tid]) {
+      unsigned long long c = 0, x1 = 0, lo = 0, hi = 0;
+      for (int q = 0; q < kSpsWarps; ++q) {
+        c += red[tid][0][q];
+        x1 += red[tid][1][q];
+        const unsigned long long nlo = lo + red[tid][2][q];
+        hi = hi + red[tid][3][q] + (nlo < lo ? 1ull : 0ull);
+        lo = nlo;
+      }
+      // sums of B = x + l over c values: T1 = X1 + c l, T2 = X2 + 2 l X1 + c l^2 (128 bits)
+      const unsigned long long l = lo_b[tid];
+      const unsigned long long t1 = x1 + c * l;
+      const unsigned long long a0 = 2 * l * x1, a1 = __umul64hi(2 * l, x1);
+      const unsigned long long b0 = l * l * c, b1 = __umul64hi(l * l, c);
+      unsigned long long r0 = lo + a0, r1 = hi + a1 + (r0 < lo ? 1ull : 0ull);
+      r1 += b1 + (r0 + b0 < r0 ? 1ull : 0ull);
+      r0 += b0;
+      const WidthStats s = WidthStats{(long long)c, (long long)t1, r0, r1};
+      st[tid] = s;
+      // bounds of the next step from this step's statistics
+      if (step < a.iters) {
+        const unsigned long long un = c, ut1 = t1;
+        const unsigned long long p_lo = un * s.t2lo;
+        const unsigned long long p_hi = __umul64hi(un, s.t2lo) + un * s.t2hi;
+        const unsigned long long q_lo = ut1 * ut1, q_hi = __umul64hi(ut1, ut1);
+        const unsigned long long v_lo = p_lo - q_lo;
+        const unsigned long long v_hi = p_hi - q_hi - (p_lo < q_lo ? 1ull : 0ull);
+        if (s.n == 0 || (v_lo | v_hi) == 0) {
+          live[tid] = 0;
+        } else {
+          const double dn = __ll2double_rn(s.n);
+          const double mu = __ddiv_rn(__ll2double_rn(s.t1), dn);
+          const double sd = __ddiv_rn(__dsqrt_rn(u128_to_f64(v_hi, v_lo)), dn);
+          const double ks = __dmul_rn(a.kappa, sd);
+          const double lo = ceil(__dsub_rn(mu, ks)), hi = floor(__dadd_rn(mu, ks));
+          // the whole-number bounds on values 0 .. 2^31 - 1
+          const double top = 2147483647.0;
+          const uint32_t l2 = lo <= 0.0 ? 0u : (lo <= top ? (uint32_t)lo : 0u);
+          lo_b[tid] = l2;
+          span_b[tid] =
+              hi >= top ? 0x7FFFFFFFu - l2 : (hi >= (double)l2 ? (uint32_t)hi - l2 : 0u);
+          some[tid] = lo <= top && hi >= 0.0 && lo <= hi ? (narrow(span_b[tid]) ? 2 : 1) : 0;
+        }
       }
     }
     __syncthreads();
@@ -1082,7 +1092,9 @@ cudaError_t launch_clip_stats(const ClipArgs& a, cudaStream_t st) {
   if (a.n <= 0 || a.n_trials <= 0 || a.nw <= 0) return cudaSuccess;
   if (a.hist < 0 || a.hist % 256 || a.hist > 1024 || a.iters < 0 || !(a.kappa > 0))
     return cudaErrorInvalidValue;
-  const size_t smem = sizeof(uint32_t) * (size_t)sps_row_words(a.hist) * kSpsWarps;
+  const size_t smem = (sizeof(uint32_t) * (size_t)sps_row_words(a.hist) +
+                       32 * (size_t)a.nw * (sizeof(ClipSum) + 2 * sizeof(uint32_t))) *
+                      kSpsWarps;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(
         k_clip_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
