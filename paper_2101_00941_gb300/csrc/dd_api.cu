@@ -741,6 +741,7 @@ int dd_plan(const double* freqs_mhz, int32_t nchans, double tsamp_s, const dd_ra
         for (int k = 0; k < kNumShapes && !p->rk[r].tiled; ++k) {
           const int shape = wide && k < 2 ? 1 - k : k;
           const int tt = kShapes[shape][0], trials = kShapes[shape][1], nt = kShapes[shape][2];
+          if (trials == 128 && !wide) continue;
           if ((o.flags & DD_FLAG_TILE256) && (tt != 256 || trials == 128)) continue;
           if ((o.flags & DD_FLAG_TRIALS32) && trials != 32) continue;
           if ((o.flags & DD_FLAG_WARPS32) != 0 && nt != 1024) continue;

@@ -67,13 +67,14 @@ constexpr int kG = 8;                       // channels per group (one delay cla
 constexpr int kNG = 2;                      // groups per stage
 constexpr int kRows = kG * kNG;             // channel rows per stage
 constexpr int kMaxNStage = 4;               // staging buffers (rows + class table), at most
-constexpr int kMaxCls = 24;                 // classes per group
+constexpr int kMaxCls = 24;                 // classes per group of a 128-trial tile
+constexpr int kMaxCls64 = 16;               // ... of a smaller one
 constexpr int kMaxSteps = 3;                // channel steps between chained classes
 constexpr int kMaxLinks = 32;               // chain links (classes and in-between steps) per group
-constexpr int kMaxTasks = 112;              // build tasks per stage
 constexpr int kBlock = 31;                  // build units stored per 32-lane block
 constexpr int kSegBytes = 128;              // inner extent of a staged-row copy (tensor map)
-constexpr size_t kSmemLimit = 220 * 1024;   // dynamic shared memory a CTA may plan for
+constexpr size_t kSmemLimit = 226 * 1024;   // dynamic shared memory a CTA may plan for: 227 KB
+                                            // less the persistent form's static 1 KB
 constexpr size_t kSmemLimit2 = 110 * 1024;  // ... when two CTAs share an SM
 
 // CTAs per SM a tile shape is compiled for (its register budget: 65536 / (NT x CTAs)).
@@ -81,7 +82,7 @@ __host__ __device__ constexpr int tile_ctas(int D, int TT, int NT) {
   return (NT == 1024 || D * TT == 64 * 512) ? 1 : 2;
 }
 
-// Entry of trial t of a tile in StageTab::zstart for a CTA of W warps with tpw trials per warp:
+// Entry of trial t of a tile in a stage's word offsets for a CTA of W warps with tpw trials per warp:
 // warp t mod W reads its trials t, t + W, ... as tpw consecutive entries.
 __host__ __device__ constexpr int trial_slot(int t, int W, int tpw) { return (t % W) * tpw + t / W; }
 
@@ -89,11 +90,11 @@ __host__ __device__ constexpr int trial_slot(int t, int W, int tpw) { return (t 
 // channel steps apart (un = 0: it stores nothing). A group's classes share a frame of pair words:
 // frame word v of a class is the sum that a trial of smallest delay b in the class uses for
 // output v - (b - F), F being the group's smallest delay. A unit is 4 (uint8) or 2 (uint16)
-// consecutive frame words; the class stores units ulo .. ulo + un - 1. Row offsets are 8 x a byte
-// offset within the stage buffer for frame word 0, before the copy's phase is added: the low five
-// bits of 8 x (offset + phase) are the funnel shift, the rest the row word. step: the channel
-// step that leads here from the preceding link, the row offset of x[r] of x[r + 1] - x[r] with
-// the step's sign in the top two bits (01: add, 11: subtract); 0 for the first link of a chain.
+// consecutive frame words; the class stores units ulo .. ulo + un - 1. Row offsets are byte
+// offsets within the stage buffer for frame word 0, before the copy's phase is added. step: the
+// channel step that leads here from the preceding link, the row offset of x[r] of x[r + 1] - x[r]
+// with the step's sign in the top two bits (01: add, 11: subtract); 0 for the first link of a
+// chain.
 struct ClsLink {
   uint32_t off[kG];
   uint32_t step;
@@ -103,24 +104,30 @@ struct ClsLink {
   __host__ __device__ uint32_t un() const { return range >> 16; }
 };
 static_assert(sizeof(ClsLink) == 48, "read as three 16-byte words");
-constexpr uint32_t kStepOff = 0x000FFFFFu, kStepAdd = 0x40000000u, kStepSub = 0xC0000000u;
+constexpr uint32_t kStepOff = 0x0000FFFFu, kStepAdd = 0x40000000u, kStepSub = 0xC0000000u;
 
-// Head of a stage's table, followed by its links (group 0's, then group 1's).
-// A build task is one block of 31 units of a run of chained links of one group:
-// first link | (links - 1) << 6 | block << 10; warp w runs the tasks of wtask[w].
+// A build task: units u0 .. u0 + 30 of a run of chained links of one group. link: byte offset of
+// the first link in the stage's table | (links - 1) << 16.
+struct BuildTask {
+  uint32_t link, u0;
+};
+
+// A stage's table: this head, the byte offset of each trial's sequence in the stage's words
+// (uint32 [kNG][trials per tile], entry trial_slot(t); 0: no trial), the links (group 0's, then
+// group 1's) and the build tasks. Warp w runs the tasks of wtask[w].
 struct StageTab {
-  int16_t zstart[kNG][kMaxTileTrials];  // stage word offset of each trial's sequence (0: no
-                                        // trial), entry trial_slot(t)
-  uint16_t task[kMaxTasks];
-  uint16_t wtask[kMaxWarps];            // first task | tasks << 8
+  uint32_t wtask[kMaxWarps];  // byte offset of the first task in the table | tasks << 16
   uint8_t nlink[kNG];
   uint8_t pad[6];
   int32_t xmin;  // smallest delay of the stage's rows for the tile's first trial
   int32_t pad1;
 };
 static_assert(sizeof(StageTab) % 16 == 0, "class tables are copied in 16-byte units");
-static_assert(kNG * kMaxLinks <= 64, "a task's fields");
-constexpr int kMaxRun = 16, kMaxBlocks = 64;
+// where the links of a table for D trials start
+__host__ __device__ constexpr uint32_t links_at(int D) {
+  return (uint32_t)sizeof(StageTab) + 4u * kNG * (uint32_t)D;
+}
+constexpr int kMaxRun = 16;
 
 __host__ __device__ constexpr size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
 
@@ -252,13 +259,16 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 template <typename T>
 struct Word;
 
-// The two row words holding a lane's samples of one channel: bits 0 .. 19 of w8 are 8 x the byte
-// offset of the lane-0 sample in the stage buffer (below 2^16 bytes plus a phase below 2^7; a
-// step's sign sits above), base is the buffer's address plus one word per unit.
-__device__ __forceinline__ void row_words(uint32_t base, uint32_t w8, uint32_t& w0, uint32_t& w1) {
-  const uint32_t addr = base + ((w8 >> 3) & 0x1FFFCu);
+// The two row words holding a lane's samples of one channel: off is the row offset (a step's sign
+// may sit above bit 29), base the stage buffer's shared address plus the copy's phase and one word
+// per unit. The sum's low two bits and its low five bits times eight are the byte and the funnel
+// shift; a shared address has 18 bits. Returns 8 x the sum (shift amounts are taken modulo 32).
+__device__ __forceinline__ uint32_t row_words(uint32_t base, uint32_t off, uint32_t& w0,
+                                              uint32_t& w1) {
+  const uint32_t at = base + off, addr = at & 0x3FFFCu;
   w0 = lds<0>(addr);
   w1 = lds<4>(addr);
+  return at << 3;
 }
 
 // uint8 data. Unit u covers pair words 4u .. 4u + 3, i.e. the eight-channel sums
@@ -273,17 +283,17 @@ template <>
 struct Word<uint8_t> {
   static constexpr int kUnit = 4;  // pair words per unit
   uint32_t e = 0, o = 0;           // samples (0, 2) and (1, 3) in 16-bit lanes
-  __device__ __forceinline__ void add(uint32_t base, uint32_t w8) {
+  __device__ __forceinline__ void add(uint32_t base, uint32_t off) {
     uint32_t w0, w1;
-    row_words(base, w8, w0, w1);
+    const uint32_t w8 = row_words(base, off, w0, w1);
     const uint32_t a = __funnelshift_r(w0, w1, w8);  // samples 0..3 in bytes 0..3
     e += a & 0x00FF00FFu;
     o += __byte_perm(a, 0, 0x4341);
   }
   // one channel's samples r .. r + 3 replaced by r + 1 .. r + 4 (sign 1) or the reverse (-1)
-  __device__ __forceinline__ void step(uint32_t base, uint32_t w8, int sign) {
+  __device__ __forceinline__ void step(uint32_t base, uint32_t off, int sign) {
     uint32_t w0, w1;
-    row_words(base, w8, w0, w1);
+    const uint32_t w8 = row_words(base, off, w0, w1);
     const uint32_t a = __funnelshift_r(w0, w1, w8);
     const uint32_t x4 = __funnelshift_r(w1, w1, w8);               // sample 4 in byte 0
     const uint32_t a02 = a & 0x00FF00FFu, a13 = __byte_perm(a, 0, 0x4341);
@@ -314,14 +324,14 @@ template <>
 struct Word<uint16_t> {
   static constexpr int kUnit = 2;
   uint32_t e = 0;  // samples 0, 1
-  __device__ __forceinline__ void add(uint32_t base, uint32_t w8) {
+  __device__ __forceinline__ void add(uint32_t base, uint32_t off) {
     uint32_t w0, w1;
-    row_words(base, w8, w0, w1);
+    const uint32_t w8 = row_words(base, off, w0, w1);
     e += __funnelshift_r(w0, w1, w8);
   }
-  __device__ __forceinline__ void step(uint32_t base, uint32_t w8, int sign) {
+  __device__ __forceinline__ void step(uint32_t base, uint32_t off, int sign) {
     uint32_t w0, w1;
-    row_words(base, w8, w0, w1);
+    const uint32_t w8 = row_words(base, off, w0, w1);
     const uint32_t a = __funnelshift_r(w0, w1, w8);
     const uint32_t x2 = __funnelshift_r(w1, w1, w8);  // sample 2 in the low half
     e += (__byte_perm(a, x2, 0x5432) - a) * (uint32_t)sign;
@@ -357,48 +367,48 @@ template <typename T>
 __device__ __forceinline__ void build_stage(uint32_t tabp, uint32_t rawb, uint32_t zb,
                                             uint32_t pos, int warp, int lane) {
   constexpr uint32_t SEG = kSegBytes / sizeof(T);
+  constexpr uint32_t ZU = 4u * (Word<T>::kUnit / 2);  // plane bytes per unit
   uint32_t wt;
-  asm volatile("ld.shared.u16 %0, [%1];"
+  asm volatile("ld.shared.u32 %0, [%1];"
                : "=r"(wt)
-               : "r"(tabp + (uint32_t)offsetof(StageTab, wtask) + 2u * warp));
+               : "r"(tabp + (uint32_t)offsetof(StageTab, wtask) + 4u * warp));
   const uint32_t xmin = lds<offsetof(StageTab, xmin)>(tabp);
-  const uint32_t ph8 = ((pos + xmin) & (SEG - 1)) * 8u * (uint32_t)sizeof(T);
-  uint32_t tp = tabp + (uint32_t)offsetof(StageTab, task) + 2u * (wt & 0xFFu);
-  for (uint32_t left = __reduce_max_sync(0xffffffffu, wt >> 8); left > 0; --left, tp += 2) {
-    uint32_t tk;
-    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(tk) : "r"(tp));
-    tk = __reduce_max_sync(0xffffffffu, tk);
-    uint32_t cp = tabp + (uint32_t)sizeof(StageTab) + (tk & 63u) * (uint32_t)sizeof(ClsLink);
-    const uint32_t u = (tk >> 10) * kBlock + lane;
-    const uint32_t us = lane < kBlock ? u : 0x80000000u;  // lane 31 stores nothing
-    const uint32_t base = rawb + 4u * u;
-    const uint32_t zl = zb + (uint32_t)sizeof(uint32_t) * (Word<T>::kUnit / 2) * u;
+  const uint32_t base0 =
+      rawb + ((pos + xmin) & (SEG - 1)) * (uint32_t)sizeof(T) + 4u * (uint32_t)lane;
+  const uint32_t zl0 = zb + ZU * (uint32_t)lane;
+  const uint32_t us0 = lane < kBlock ? (uint32_t)lane : 0x80000000u;  // lane 31 stores nothing
+  uint32_t tp = tabp + (wt & 0xFFFFu);
+  for (uint32_t left = __reduce_max_sync(0xffffffffu, wt >> 16); left > 0; --left, tp += 8) {
+    uint32_t tl, u0;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(tl), "=r"(u0) : "r"(tp));
+    uint32_t n = __reduce_max_sync(0xffffffffu, tl >> 16);
+    uint32_t cp = tabp + (tl & 0xFFFFu);
+    const uint32_t us = us0 + u0, base = base0 + 4u * u0, zl = zl0 + ZU * u0;
     Word<T> w;
     const uint4 a = lds128(cp), b = lds128(cp + 16);
     uint4 lk = lds128(cp + 32);
-    w.add(base, a.x + ph8);
-    w.add(base, a.y + ph8);
-    w.add(base, a.z + ph8);
-    w.add(base, a.w + ph8);
-    w.add(base, b.x + ph8);
-    w.add(base, b.y + ph8);
-    w.add(base, b.z + ph8);
-    w.add(base, b.w + ph8);
+    w.add(base, a.x);
+    w.add(base, a.y);
+    w.add(base, a.z);
+    w.add(base, a.w);
+    w.add(base, b.x);
+    w.add(base, b.y);
+    w.add(base, b.z);
+    w.add(base, b.w);
     // the next link's record is loaded before this one's stores
-    uint32_t n = (tk >> 6) & 15u;
 #pragma unroll 1
     for (; n >= 2; n -= 2, cp += 2u * (uint32_t)sizeof(ClsLink)) {
       const uint4 l1 = lds128(cp + 32 + sizeof(ClsLink));
       w.emit(zl + lk.y, zl + lk.z, us - (lk.w & 0xFFFFu), lk.w >> 16);
-      w.step(base, l1.x + ph8, (int32_t)l1.x >> 30);
+      w.step(base, l1.x, (int32_t)l1.x >> 30);
       lk = lds128(cp + 32 + 2 * sizeof(ClsLink));
       w.emit(zl + l1.y, zl + l1.z, us - (l1.w & 0xFFFFu), l1.w >> 16);
-      w.step(base, lk.x + ph8, (int32_t)lk.x >> 30);
+      w.step(base, lk.x, (int32_t)lk.x >> 30);
     }
     w.emit(zl + lk.y, zl + lk.z, us - (lk.w & 0xFFFFu), lk.w >> 16);
     if (n) {
       lk = lds128(cp + 32 + sizeof(ClsLink));
-      w.step(base, lk.x + ph8, (int32_t)lk.x >> 30);
+      w.step(base, lk.x, (int32_t)lk.x >> 30);
       w.emit(zl + lk.y, zl + lk.z, us - (lk.w & 0xFFFFu), lk.w >> 16);
     }
   }
@@ -685,15 +695,20 @@ __device__ __forceinline__ void store_tile(const uint32_t (&acc)[kTPW][KT], int3
 // Words 32k + lane of N trials' sequences in both groups (or, both = false, in the first) added
 // to the packed sums of trials q0 ..; tc: shared address of the trials' word offsets, zs: of the
 // stage's words at the lane.
-template <int KP, int N, int kTPW>
+template <int D, int KP, int N, int kTPW>
 __device__ __forceinline__ void add_words(uint32_t zs, uint32_t tc, bool both, int q0,
                                           uint32_t (&pk)[kTPW][KP]) {
   uint32_t zp[N], zq[N];  // N trials' words in group 0 and 1
+  if constexpr (N == 4) {
+    const uint4 e = lds128(tc), f = lds128(tc + 4 * D);
+    zp[0] = zs + e.x, zp[1] = zs + e.y, zp[2] = zs + e.z, zp[3] = zs + e.w;
+    zq[0] = zs + f.x, zq[1] = zs + f.y, zq[2] = zs + f.z, zq[3] = zs + f.w;
+  } else {
 #pragma unroll
-  for (int q = 0; q < N; q += 2) {
-    const uint32_t e = lds<0>(tc + 2 * q), f = lds<2 * kMaxTileTrials>(tc + 2 * q);
-    zp[q] = zs + 4u * (e & 0xFFFFu), zp[q + 1] = zs + 4u * (e >> 16);
-    zq[q] = zs + 4u * (f & 0xFFFFu), zq[q + 1] = zs + 4u * (f >> 16);
+    for (int q = 0; q < N; ++q) {
+      zp[q] = zs + lds<0>(tc + 4 * q);
+      zq[q] = zs + lds<4 * D>(tc + 4 * q);
+    }
   }
   if (both) {
 #pragma unroll
@@ -771,12 +786,14 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
     for (int k = 0; k < KP; ++k) pk[q][k] = 0;
   int left = a.flush;  // stages until the packed sums go to the 32-bit outputs
   const uint32_t raw_step = (uint32_t)(stage_elems * sizeof(T)), tab_step = (uint32_t)a.tab_pitch;
-  int b0 = 0, b1 = 1;     // staging buffers of stages s and s + 1
-  uint32_t par1 = 0;      // barrier parity of stage s + 1
+  // of stage s: staging buffer; of stage s + 1: staging buffer, its rows and table, barrier parity
+  int b0 = 0, b1 = 1;
+  uint32_t tcur = stab, rnext = sraw + raw_step, tnext = stab + tab_step, par1 = 0;
   uint32_t zcur = sz, znext = sz + a.zcap * 4u;  // word buffers of stages s and s + 1
+  const uint32_t zrow = (uint32_t)sizeof(StageTab) + 4u * kTPW * warp;
+  const int lone = (ngroups & 1) ? nstages - 1 : nstages;  // the stage holding one group
 
   for (int s = 0; s < nstages && !aborted; ++s) {
-    const int ng = min(kNG, ngroups - s * kNG);
     // (1) TMA for stage s + NS - 1 into the buffers stage s - 1 used (its words were built
     //     during stage s - 2 and its table last read by the accumulation of stage s - 1)
     if (s >= 1 && s + NS - 1 < nstages) {
@@ -788,36 +805,41 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
       }
       issued = s + NS;
     }
-    // (2) pair words of stage s + 1
     bool ok = true;
-    if (s + 1 < nstages) {
-      ok = mbar_try_wait(&mbar[b1], par1) || mbar_wait_bounded(&mbar[b1], par1);
-      if (ok)
-        build_stage<T>(stab + b1 * tab_step, sraw + b1 * raw_step, znext, pos, warp, lane);
-    }
-    // (3) accumulate stage s: lane l of the warp reads, for each of its trials, pair word
-    //     l + 32k of the trial's plane in both groups (outputs 2(l + 32k) and 2(l + 32k) + 1)
+    if (s + 1 < nstages) ok = mbar_try_wait(&mbar[b1], par1) || mbar_wait_bounded(&mbar[b1], par1);
+    // (2) pair words of stage s + 1, and
+    // (3) accumulation of stage s: lane l of the warp reads, for each of its trials, pair word
+    //     l + 32k of the trial's plane in both groups (outputs 2(l + 32k) and 2(l + 32k) + 1).
+    // Half of each scheduler's warps take (3) first: the build is bound by instruction issue, the
+    // accumulation by the shared-memory pipe.
+    if (ok && s + 1 < nstages) build_stage<T>(tnext, rnext, znext, pos, warp, lane);
     {
-      const uint32_t tc = stab + b0 * tab_step + (uint32_t)offsetof(StageTab, zstart) +
-                          2u * kTPW * warp;
-      const uint32_t zs = zcur + 4u * lane;
+      const uint32_t zs = zcur + 4u * lane, tc = tcur + zrow;
       constexpr int N = kTPW < 4 ? kTPW : 4;  // trials at a time: eight row addresses
 #pragma unroll
-      for (int q = 0; q < kTPW; q += N)  // only the last stage may hold one group
-        add_words<KP, N>(zs, tc + 2u * q, ng == kNG, q, pk);
-      if (--left == 0 || s + 1 == nstages) {  // uniform
-        left = a.flush;
+      for (int q = 0; q < kTPW; q += N) add_words<D, KP, N>(zs, tc + 4u * q, s != lone, q, pk);
+    }
+    if (--left == 0 || s + 1 == nstages) {  // uniform
+      left = a.flush;
 #pragma unroll
-        for (int k = 0; k < KP; ++k)
+      for (int k = 0; k < KP; ++k)
 #pragma unroll
-          for (int q = 0; q < kTPW; ++q) {
-            pair_add(pk[q][k], acc[q][2 * k], acc[q][2 * k + 1]);
-            pk[q][k] = 0;
-          }
-      }
+        for (int q = 0; q < kTPW; ++q) {
+          pair_add(pk[q][k], acc[q][2 * k], acc[q][2 * k + 1]);
+          pk[q][k] = 0;
+        }
     }
     b0 = b1;
-    if (++b1 == NS) b1 = 0, par1 ^= 1u;
+    tcur = tnext;
+    if (++b1 == NS) {
+      b1 = 0;
+      par1 ^= 1u;
+      rnext = sraw;
+      tnext = stab;
+    } else {
+      rnext += raw_step;
+      tnext += tab_step;
+    }
     const uint32_t zt = zcur;
     zcur = znext;
     znext = zt;
@@ -1131,22 +1153,26 @@ constexpr BuildCost kCostU8{100, 16, 18}, kCostU16{80, 13, 14};
 // Deal a stage's build work to W warps: per group and block of 31 units, the chain of links,
 // from and to classes that store units in the block, cut where the plan breaks the chain
 // (link without a step) and where a warp has its share. The share is the smallest, found by
-// bisection, with which W warps suffice. Returns it, or 0 if the task list overflows.
-int deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
+// bisection, with which W warps suffice. Returns it.
+int deal_work(StageTab& st, const ClsLink* cls, int D, std::vector<BuildTask>& tasks, int W,
+              const BuildCost& C) {
   const int first[kNG + 1] = {0, st.nlink[0], st.nlink[0] + st.nlink[1]};
+  const uint32_t l0 = links_at(D), t0 = l0 + (uint32_t)(first[kNG] * sizeof(ClsLink));
   int nblk[kNG] = {0, 0};
   for (int gl = 0; gl < kNG; ++gl)
     for (int p = first[gl]; p < first[gl + 1]; ++p)
       nblk[gl] = std::max(nblk[gl], (int)(cls[p].ulo() + cls[p].un() + kBlock - 1) / kBlock);
-  if (nblk[0] > kMaxBlocks || nblk[1] > kMaxBlocks) return 0;
   auto stores = [&](int p, int b) {
     return cls[p].un() && (int)cls[p].ulo() < (b + 1) * kBlock &&
            (int)(cls[p].ulo() + cls[p].un()) > b * kBlock;
   };
-  // deal with a given share; returns the warps used (-1 if the task list overflows)
+  // deal with a given share; returns the warps used
   auto deal = [&](int share, bool out) {
     int w = 0, load = 0, nt = 0;
-    if (out) std::memset(st.wtask, 0, sizeof st.wtask);
+    if (out) {
+      tasks.clear();
+      std::memset(st.wtask, 0, sizeof st.wtask);
+    }
     for (int gl = 0; gl < kNG; ++gl)
       for (int b = 0; b < nblk[gl]; ++b) {
         int p = first[gl];
@@ -1157,7 +1183,6 @@ int deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
           }
           if (load > 0 && load + C.base + C.emit > share) {
             ++w;
-            if (out) st.wtask[w] = (uint16_t)nt;
             load = 0;
           }
           // a run from p: extend while the links chain and fit the share
@@ -1173,9 +1198,10 @@ int deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
             }
           }
           if (out) {
-            if (nt == kMaxTasks) return -1;
-            st.task[nt] = (uint16_t)(p | (last - p) << 6 | b << 10);
-            st.wtask[w] += 1 << 8;
+            if (st.wtask[w] == 0) st.wtask[w] = t0 + (uint32_t)(nt * sizeof(BuildTask));
+            st.wtask[w] += 1u << 16;
+            tasks.push_back({(uint32_t)(l0 + p * sizeof(ClsLink)) | (uint32_t)(last - p) << 16,
+                             (uint32_t)(b * kBlock)});
           }
           ++nt;
           p = last + 1;
@@ -1192,13 +1218,24 @@ int deal_work(StageTab& st, const ClsLink* cls, int W, const BuildCost& C) {
     const int mid = (lo + hi) / 2;
     if (deal(mid, false) > W) lo = mid; else hi = mid;
   }
-  return deal(hi, true) > 0 ? hi : 0;
+  deal(hi, true);
+  return hi;
 }
 
+// Tasks of a stage, and where they lie in its table for D trials.
 int stage_tasks(const StageTab& st) {
   int n = 0;
-  for (int w = 0; w < kMaxWarps; ++w) n += st.wtask[w] >> 8;
+  for (int w = 0; w < kMaxWarps; ++w) n += (int)(st.wtask[w] >> 16);
   return n;
+}
+
+const ClsLink* table_links(const uint8_t* tab, int D) {
+  return reinterpret_cast<const ClsLink*>(tab + links_at(D));
+}
+
+const BuildTask* table_tasks(const uint8_t* tab, int D) {
+  const StageTab& st = *reinterpret_cast<const StageTab*>(tab);
+  return reinterpret_cast<const BuildTask*>(table_links(tab, D) + st.nlink[0] + st.nlink[1]);
 }
 
 // Self-test of the bounded wait above: one thread arms a fresh mbarrier that nothing ever
@@ -1241,10 +1278,10 @@ static void tiled_smem_work(TiledPlan& P, int ntiles, int nstages, int ngroups, 
       const StageTab& st = *reinterpret_cast<const StageTab*>(tp);
       const int ng = std::min(kNG, ngroups - s * kNG);
       lsu += (int64_t)W * kTPW * KP * ng;             // accumulation words
-      lsu += (int64_t)W * ng * (kTPW / 2);            // zstart entries (two a load)
+      lsu += (int64_t)W * ng * ((kTPW + 3) / 4);      // zstart entries (four a load)
       lsu += 2 * W;                                   // wtask, xmin
       for (int t = 0; t < stage_tasks(st); ++t) {
-        const int n = (st.task[t] >> 6) & 15;         // links after the first
+        const int n = (int)(table_tasks(tp, P.trials)[t].link >> 16);  // links after the first
         lsu += 3 + 2 * kG;                            // descriptor, row offsets, row words
         lsu += (int64_t)(n + 1) * (1 + sts_per_class) + 2 * n;
       }
@@ -1271,7 +1308,9 @@ namespace {
 // A stage's table with room for every link, and what the plan needs to know of it.
 struct StagePlan {
   StageTab st;
+  uint32_t zstart[kNG][kMaxTileTrials];
   ClsLink cls[kNG * kMaxLinks];
+  std::vector<BuildTask> tasks;
   int words, links;  // pair words and links used
   int share;         // the largest warp's build work (BuildCost units)
 };
@@ -1279,8 +1318,11 @@ struct StagePlan {
 bool plan_stage(const int32_t* tab, int t0, int n, int cpad, int s, bool u16, int tt, int D,
                 int W, int row_slot, StagePlan& F) {
   const int U = u16 ? Word<uint16_t>::kUnit : Word<uint8_t>::kUnit;
-  const int es = u16 ? 2 : 1, ngroups = cpad / kG;
-  std::memset(&F, 0, sizeof F);
+  const int ngroups = cpad / kG;
+  const uint32_t es = u16 ? 2 : 1;
+  std::memset(&F.st, 0, sizeof F.st);
+  std::memset(F.zstart, 0, sizeof F.zstart);
+  std::memset(F.cls, 0, sizeof F.cls);
   StageTab& st = F.st;
   int32_t xmin = INT32_MAX;
   for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
@@ -1309,7 +1351,7 @@ bool plan_stage(const int32_t* tab, int t0, int n, int cpad, int s, bool u16, in
       int p = 0;
       while (p < ncls && !(csum[p] == sum && std::equal(key, key + kG, ckey[p]))) ++p;
       if (p == ncls) {
-        if (ncls == kMaxCls) return false;
+        if (ncls == (D > 64 ? kMaxCls : kMaxCls64)) return false;
         std::copy(key, key + kG, ckey[ncls]);
         cmin[ncls] = cmax[ncls] = b[i];
         csum[ncls] = sum;
@@ -1335,7 +1377,7 @@ bool plan_stage(const int32_t* tab, int t0, int n, int cpad, int s, bool u16, in
       int32_t key[kG];  // walks from the preceding class to this one
       std::copy(ckey[k > 0 ? prev : p], ckey[k > 0 ? prev : p] + kG, key);
       auto at_row = [&](int q, int r) {
-        return 8u * es * (uint32_t)((gl * kG + q) * row_slot + f0 + r - xmin);
+        return es * (uint32_t)((gl * kG + q) * row_slot + f0 + r - xmin);
       };
       int dist = 0;
       for (int q = 0; q < kG; ++q) dist += std::abs(ckey[p][q] - key[q]);
@@ -1362,15 +1404,15 @@ bool plan_stage(const int32_t* tab, int t0, int n, int cpad, int s, bool u16, in
     }
     for (int i = 0; i < n; ++i) {
       const int p = cls_of[i], o = b[i] - f0 - ulos[p] * U;
-      st.zstart[gl][trial_slot(i, W, D / W)] =
-          (int16_t)(zoff[p] + (o % 2) * (zlens[p] / 2) + o / 2);
+      F.zstart[gl][trial_slot(i, W, D / W)] =
+          4u * (uint32_t)(zoff[p] + (o % 2) * (zlens[p] / 2) + o / 2);
     }
     st.nlink[gl] = (uint8_t)(nl - nl0);
   }
   F.words = words;
   F.links = nl;
-  F.share = deal_work(st, F.cls, W, u16 ? kCostU16 : kCostU8);
-  return F.share > 0;
+  F.share = deal_work(st, F.cls, D, F.tasks, W, u16 ? kCostU16 : kCostU8);
+  return true;
 }
 
 bool shape_exists(int tt, int D, int nt) {
@@ -1471,16 +1513,22 @@ TiledPlan tiled_plan(const int32_t* tab, int ntr, int cpad, int decimation, int 
       StagePlan F;
       const int a = (int)((int64_t)ntiles * k / nth), z = (int)((int64_t)ntiles * (k + 1) / nth);
       q.len.reserve((size_t)(z - a) * nstages);
-      q.bytes.reserve((size_t)(z - a) * nstages * (sizeof(StageTab) + 18 * sizeof(ClsLink)));
+      q.bytes.reserve((size_t)(z - a) * nstages * (links_at(D) + 24 * sizeof(ClsLink)));
       for (int ti = a; ti < z && q.ok; ++ti)
         for (int s = 0; s < nstages && q.ok; ++s) {
           q.ok = plan_stage(tab, ti * D, std::min(D, ntr - ti * D), cpad, s, u16, tt, D, W,
                             P.row_slot, F);
           if (!q.ok) break;
-          const size_t len = sizeof(StageTab) + F.links * sizeof(ClsLink), at = q.bytes.size();
+          const size_t zlen = 4 * (size_t)D, links = F.links * sizeof(ClsLink);
+          const size_t tasks = F.tasks.size() * sizeof(BuildTask);
+          const size_t at = q.bytes.size(), len = align16(links_at(D) + links + tasks);
           q.bytes.resize(at + len);
-          std::memcpy(q.bytes.data() + at, &F.st, sizeof(StageTab));
-          std::memcpy(q.bytes.data() + at + sizeof(StageTab), F.cls, F.links * sizeof(ClsLink));
+          uint8_t* to = q.bytes.data() + at;
+          std::memcpy(to, &F.st, sizeof(StageTab));
+          for (int gl = 0; gl < kNG; ++gl)
+            std::memcpy(to + sizeof(StageTab) + gl * zlen, F.zstart[gl], zlen);
+          std::memcpy(to + links_at(D), F.cls, links);
+          std::memcpy(to + links_at(D) + links, F.tasks.data(), tasks);
           q.len.push_back((uint32_t)len);
           q.words = std::max(q.words, F.words);
         }
@@ -1576,9 +1624,12 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
     for (int s = 0; s < nstages; ++s) {
       const uint8_t* tp = P.tabs.data() + ((size_t)ti * nstages + s) * P.tab_pitch;
       const StageTab& st = *reinterpret_cast<const StageTab*>(tp);
-      const ClsLink* cls = reinterpret_cast<const ClsLink*>(tp + sizeof(StageTab));
+      const ClsLink* cls = table_links(tp, D);
+      const BuildTask* task = table_tasks(tp, D);
+      const uint32_t* zst = reinterpret_cast<const uint32_t*>(tp + sizeof(StageTab));
       const int ncls = st.nlink[0] + st.nlink[1];
-      bad += sizeof(StageTab) + ncls * sizeof(ClsLink) > (size_t)P.tab_pitch;
+      const size_t tasks0 = (const uint8_t*)task - tp;
+      bad += tasks0 + stage_tasks(st) * sizeof(BuildTask) > (size_t)P.tab_pitch;
       int32_t xmin = INT32_MAX;
       for (int c = s * kRows; c < std::min(cpad, (s + 1) * kRows); ++c)
         xmin = std::min(xmin, tab[(int64_t)t0 * cpad + c]);
@@ -1600,13 +1651,14 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
         for (int v = z0; v < z0 + zlen; ++v) bad += words[v]++ != 0;
       }
       for (int w = 0, t = 0; w < kWarps; ++w) {  // the warps' tasks follow one another
-        bad += (st.wtask[w] >> 8) && (st.wtask[w] & 255) != t;
-        t += st.wtask[w] >> 8;
+        bad += (st.wtask[w] >> 16) && (st.wtask[w] & 0xFFFFu) != tasks0 + t * sizeof(BuildTask);
+        t += (int)(st.wtask[w] >> 16);
       }
       for (int w = kWarps; w < kMaxWarps; ++w) bad += st.wtask[w] != 0;
-      bad += stage_tasks(st) > kMaxTasks;
-      for (int t = 0; t < std::min(stage_tasks(st), kMaxTasks); ++t) {
-        const int p0 = st.task[t] & 63, np = ((st.task[t] >> 6) & 15) + 1, b = st.task[t] >> 10;
+      for (int t = 0; t < stage_tasks(st); ++t) {
+        const int p0 = (int)((task[t].link & 0xFFFFu) - links_at(D)) / (int)sizeof(ClsLink);
+        const int np = (int)(task[t].link >> 16) + 1, u0 = (int)task[t].u0;
+        bad += (task[t].link & 0xFFFFu) != links_at(D) + p0 * sizeof(ClsLink);
         const int gl = p0 >= st.nlink[0];
         if (p0 + np > (gl ? ncls : (int)st.nlink[0])) {
           ++bad;
@@ -1621,21 +1673,21 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
             bad += !up && (sw & ~kStepOff) != kStepSub;
             int hit = 0;
             for (int q = 0; q < kG && !hit; ++q)
-              if (off[q] == (up ? at : at + 8u * es)) {
-                off[q] = up ? at + 8u * es : at;
+              if (off[q] == (up ? at : at + es)) {
+                off[q] = up ? at + es : at;
                 ++hit;
               }
             bad += hit != 1;
           }
           bad += !std::equal(off, off + kG, cls[p].off);
           for (int l = 0; l < kBlock; ++l) {
-            const int v = b * kBlock + l - (int)cls[p].ulo();
+            const int v = u0 + l - (int)cls[p].ulo();
             if (v >= 0 && v < (int)cls[p].un()) bad += stored[p][v]++ != 0;
           }
           // lane 31's second row word at the largest phase
           for (int q = 0; q < kG; ++q)
             bad += L.raw + (size_t)(P.nstage - 1) * kRows * P.row_slot * es +
-                       4u * (uint32_t)(b * kBlock + 31) + cls[p].off[q] / 8 + (SEG - 1) * es + 8 >
+                       4u * (uint32_t)(u0 + 31) + cls[p].off[q] + (SEG - 1) * es + 8 >
                    L.total;
         }
       }
@@ -1646,7 +1698,9 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
         const int c0 = (s * kNG + gl) * kG, g0 = p1;
         p1 += st.nlink[gl];
         for (int i = 0; i < n; ++i) {
-          const int z = st.zstart[gl][trial_slot(i, kWarps, D / kWarps)];
+          const uint32_t zb = zst[gl * D + trial_slot(i, kWarps, D / kWarps)];
+          bad += zb % 4 != 0;
+          const int z = (int)zb / 4;
           int p = g0, v = -1;
           for (; p < p1; ++p) {
             const int zo = cls[p].ev / 4 + (int)cls[p].ulo() * U / 2;
@@ -1665,7 +1719,7 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
             continue;
           }
           for (int q = 0; q < kG; ++q)
-            bad += (int64_t)cls[p].off[q] / (8 * es) + v !=
+            bad += (int64_t)cls[p].off[q] / es + v !=
                    (int64_t)(gl * kG + q) * P.row_slot +
                        tab[(int64_t)(t0 + i) * cpad + c0 + q] - xmin;
         }

@@ -93,7 +93,8 @@ def test_coarse_channels_and_bad_tables_are_refused():
 def test_chains_on_jittered_tables(tt, trials, decimation):
     """Delay tables whose groups' classes lie zero to many channel steps apart (chains with
     in-between links, broken chains, one class): the plan is either refused or free of
-    violations, and the smooth tables are accepted."""
+    violations, and smooth tables are accepted up to the tile's class limit (16 per group, 24 with
+    128 trials)."""
     rng = np.random.default_rng(75)
     accepted = 0
     for jitter in (0.0, 0.3, 1.0, 2.0):
@@ -105,7 +106,10 @@ def test_chains_on_jittered_tables(tt, trials, decimation):
             ok, bad = dd.dd_tiled_plan_check(tab, decimation, tt, trials)
             assert bad == 0, (jitter, ntr, cpad)
             accepted += ok
-            assert ok or jitter > 0
+            most = max(len(np.unique(g - g.min(1, keepdims=True), axis=0))
+                       for t0 in range(0, ntr, trials)
+                       for c in range(0, cpad, 8) for g in [tab[t0:t0 + trials, c:c + 8]])
+            assert ok or jitter > 0 or most > (24 if trials == 128 else 16)
     assert accepted > 3
 
 
