@@ -461,6 +461,95 @@ __device__ __forceinline__ uint32_t* fused_edge(const FusedArgs& f, int ntx, int
   return f.edge + ((size_t)seg * ntx + bx) * 2 * kFusedTrials * (size_t)f.hist;
 }
 
+// A warp's prefix-sum row is padded by four words after every 16, so that lanes reading 16-byte
+// chunks 16 samples apart touch every bank once: place of entry j, and of the first entry of
+// 4-entry chunk c.
+__host__ __device__ constexpr int fused_row_words(int hp) { return (hp + 512) / 4 * 5; }
+__device__ __forceinline__ int row_at(int j) { return j + 4 * (j >> 4); }
+__device__ __forceinline__ int chunk_at(int c) { return 4 * c + 4 * (c >> 2); }
+
+// d = p - the sixteen entries from M entries past chunk x on (of the lane's part e of a row).
+template <int M>
+__device__ __forceinline__ void row_diffs(const uint32_t (&p)[16], const uint32_t* e, int x,
+                                          uint32_t (&d)[16]) {
+  uint4 v[5];
+#pragma unroll
+  for (int i = 0; i < (M ? 5 : 4); ++i)
+    v[i] = *reinterpret_cast<const uint4*>(e + chunk_at(x + i));
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const uint4 c = v[(i + M) / 4];
+    const int r = (i + M) % 4;
+    d[i] = p[i] - (r == 0 ? c.x : r == 1 ? c.y : r == 2 ? c.z : c.w);
+  }
+}
+
+// Peak blocks of 16 or 32 samples: lane l takes samples 16 l .. 16 l + 15 of the tile, their
+// prefix sums in registers, and per width reads the 16 earlier ones in four or five aligned
+// 16-byte loads. Samples are visited in order, so the first of the largest sums wins; the two
+// halves of a 32-sample block meet by one shuffle. About 80 instructions per width and trial,
+// where one 4-byte load and a tie rule per sample and width took 330 at a quarter of the issue
+// rate (113 us a tile of 64 trials x 512 samples x 9 widths, about 55 so).
+template <bool INTERIOR>
+__device__ __forceinline__ void fused_blocks(const FusedArgs& f, const uint32_t* E, int64_t rowk,
+                                             int64_t j0, int64_t nout, bool first, int lane) {
+  const int Bk = f.block, nw = f.nw, jl0 = 16 * lane;
+  uint32_t p[16];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint4 v = *reinterpret_cast<const uint4*>(E + 20 * lane + 4 * i);
+    p[4 * i] = v.x, p[4 * i + 1] = v.y, p[4 * i + 2] = v.z, p[4 * i + 3] = v.w;
+  }
+  const int64_t left = nout - j0 - jl0;  // window samples from this lane's first on
+  const int hi = (int)(left < 0 ? 0 : (left > 16 ? 16 : left));
+  const bool keep = hi > 0 && (Bk == 16 || (lane & 1) == 0);
+  const int64_t blk = (j0 + jl0) / Bk;
+#pragma unroll 1
+  for (int k = 0; k < nw; ++k) {
+    const int w = f.wd[k], m = (-w) & 3, x = -((w + m) >> 2);
+    const uint32_t* e = E + 20 * lane;
+    uint32_t d[16];
+    if (m == 0) row_diffs<0>(p, e, x, d);  // uniform
+    else if (m == 1) row_diffs<1>(p, e, x, d);
+    else if (m == 2) row_diffs<2>(p, e, x, d);
+    else row_diffs<3>(p, e, x, d);
+    if (!INTERIOR) {  // keys: 1 + the sum, 0 for a sample outside the window or the segment
+      const int64_t back = w - 1 - (j0 + jl0);
+      int lo = (int)(back < 0 ? 0 : (back > 16 ? 16 : back));
+      if (first) lo = max(lo, w - 1 - jl0);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) d[i] = i >= lo && i < hi ? d[i] + 1u : 0u;
+    }
+    // the largest and its first place: four quarters, then the quarters in order
+    uint32_t best[4];
+    int off[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      best[i] = d[4 * i];
+      off[i] = 4 * i;
+#pragma unroll
+      for (int q = 1; q < 4; ++q)
+        if (d[4 * i + q] > best[i]) best[i] = d[4 * i + q], off[i] = 4 * i + q;
+    }
+#pragma unroll
+    for (int i = 1; i < 4; i += 2)
+      if (best[i] > best[i - 1]) best[i - 1] = best[i], off[i - 1] = off[i];
+    if (best[2] > best[0]) best[0] = best[2], off[0] = off[2];
+    uint32_t key = best[0] + (INTERIOR ? 1u : 0u);
+    int at = off[0];
+    if (Bk == 32) {  // the odd lane holds the block's second half
+      const uint32_t ok = __shfl_xor_sync(0xffffffffu, key, 1);
+      const int oa = __shfl_xor_sync(0xffffffffu, at, 1);
+      if (ok > key) key = ok, at = oa + 16;
+    }
+    if (keep) {
+      const int64_t idx = (rowk + k) * f.nblk + blk;
+      f.key[idx] = key;
+      f.off[idx] = (uint8_t)(key ? at : 0);
+    }
+  }
+}
+
 template <int TT, int W, int kTPW, int KT>
 __device__ __forceinline__ void fused_search(const TiledArgs& a, const FusedArgs& f,
                                              const uint32_t (&acc)[kTPW][KT],
@@ -474,7 +563,9 @@ __device__ __forceinline__ void fused_search(const TiledArgs& a, const FusedArgs
   const int seg = by / f.seg_tiles;
   uint32_t* head = fused_edge(f, ntx, bx, seg);
   uint32_t* tail = head + kFusedTrials * (size_t)hist;
-  uint32_t* E = reinterpret_cast<uint32_t*>(smem + f.e_off) + (size_t)warp * (HP + TT) + HP;
+  static_assert(TT == 512, "sixteen samples a lane");
+  uint32_t* E = reinterpret_cast<uint32_t*>(smem + f.e_off) +
+                (size_t)warp * fused_row_words(HP) + HP / 4 * 5;
   const int64_t nout = a.nout;
   const uint64_t pol = l2_keep_policy();
 #pragma unroll
@@ -500,7 +591,7 @@ __device__ __forceinline__ void fused_search(const TiledArgs& a, const FusedArgs
         if (lane >= o) incl += x;
       }
       const uint32_t po = carry + incl;
-      *reinterpret_cast<uint2*>(E + 2 * (lane + 32 * k)) = make_uint2(po - od, po);
+      *reinterpret_cast<uint2*>(E + row_at(2 * (lane + 32 * k))) = make_uint2(po - od, po);
       carry += __shfl_sync(0xffffffffu, incl, 31);
     }
     // the previous tile's prefix sums in this tile's frame (none before a segment's first tile:
@@ -508,76 +599,48 @@ __device__ __forceinline__ void fused_search(const TiledArgs& a, const FusedArgs
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
       const int i = lane + 32 * r;
-      if (i < hist) E[i - hist] = hv[r];
+      if (i < hist) E[row_at(i - hist)] = hv[r];
     }
     __syncwarp();
     if (first && seg > 0) {
       uint32_t* hd = head + (size_t)t * hist;
-      for (int i = lane; i < hist; i += 32) hd[i] = E[i];
+      for (int i = lane; i < hist; i += 32) hd[i] = E[row_at(i)];
     }
     // this tile's last prefix sums in the next tile's frame (P[TT + m] - P[TT - 1])
-    for (int i = lane; i < hist; i += 32) st_keep(tl + i, E[TT - hist + i] - carry, pol);
+    for (int i = lane; i < hist; i += 32)
+      st_keep(tl + i, E[row_at(TT - hist + i)] - carry, pol);
     const int64_t rowk = (int64_t)(trial0 + t) * nw;
-    // one lane per item: a 32-sample block is two items of 16 samples (lanes b and b + 16), a
-    // smaller block one item; each lane visits its samples from (lane mod P) on, so the 32 lanes
-    // of a load read 32 different banks, and keeps per width the largest key and, on ties, the
-    // earliest sample
-    const int P = Bk == 32 ? 16 : Bk;
-    const int nitems = (TT / Bk) * (Bk == 32 ? 2 : 1);
     const bool interior = j0 >= wmax - 1 && !first && j0 + TT <= nout;
+    if (Bk >= 16) {
+      if (interior) fused_blocks<true>(f, E, rowk, j0, nout, first, lane);
+      else fused_blocks<false>(f, E, rowk, j0, nout, first, lane);
+      __syncwarp();  // the row is rewritten for the warp's next trial
+      continue;
+    }
+    // smaller blocks: a lane takes a whole one and visits its samples from (lane mod Bk) on,
+    // keeping per width the largest key and, on ties, the earliest sample
 #pragma unroll 1
-    for (int it = lane; it < nitems; it += 32) {
-      const int b = Bk == 32 ? (it & 15) : it;
-      const int h = Bk == 32 ? (it >> 4) : 0;
-      const int o0 = h * P;  // the item's first sample within its block
-      const int jl0 = b * Bk + o0;
-      uint32_t best[kMaxWidths];
-      int boff[kMaxWidths];
-#pragma unroll
-      for (int k = 0; k < kMaxWidths; ++k) best[k] = 0u, boff[k] = 32;
-#pragma unroll 1
-      for (int i = 0; i < P; ++i) {
-        const int pi = (i + lane) & (P - 1);
-        const int jl = jl0 + pi, o = o0 + pi;
-        const int64_t jg = j0 + jl;
-        const uint32_t p1 = E[jl] + 1u;
-#pragma unroll
-        for (int k = 0; k < kMaxWidths; ++k) {
-          if (k < nw) {
-            const int w = f.wd[k];
-            uint32_t key = p1 - E[jl - w];
-            if (!interior) {
-              const bool valid = jg < nout && jg >= w - 1 && (!first || jl >= w - 1);
-              key = valid ? key : 0u;
-            }
-            const bool take = key > best[k] || (key == best[k] && o < boff[k]);
-            best[k] = take ? key : best[k];
-            boff[k] = take ? o : boff[k];
-          }
-        }
-      }
-      if (Bk == 32) {  // every lane has an item: combine the two halves of each block
-#pragma unroll
-        for (int k = 0; k < kMaxWidths; ++k) {
-          if (k < nw) {
-            const uint32_t ob = __shfl_xor_sync(0xffffffffu, best[k], 16);
-            const int oo = __shfl_xor_sync(0xffffffffu, boff[k], 16);
-            const bool take = ob > best[k] || (ob == best[k] && oo < boff[k]);
-            best[k] = take ? ob : best[k];
-            boff[k] = take ? oo : boff[k];
-          }
-        }
-      }
+    for (int b = lane; b < TT / Bk; b += 32) {
       const int64_t jb = j0 + (int64_t)b * Bk;  // the block's first window sample
-      if (h == 0 && jb < nout) {
-        const int64_t blk = jb / Bk;
-#pragma unroll
-        for (int k = 0; k < kMaxWidths; ++k) {
-          if (k < nw) {
-            const int64_t idx = (rowk + k) * f.nblk + blk;
-            f.key[idx] = best[k];
-            f.off[idx] = (uint8_t)(best[k] ? boff[k] : 0);
-          }
+#pragma unroll 1
+      for (int k = 0; k < nw; ++k) {
+        const int w = f.wd[k];
+        uint32_t best = 0;
+        int boff = 32;
+        for (int i = 0; i < Bk; ++i) {
+          const int o = (i + lane) & (Bk - 1), jl = b * Bk + o;
+          const int64_t jg = j0 + jl;
+          const bool valid =
+              interior || (jg < nout && jg >= w - 1 && (!first || jl >= w - 1));
+          const uint32_t key = valid ? E[row_at(jl)] + 1u - E[row_at(jl - w)] : 0u;
+          const bool take = key > best || (key == best && o < boff);
+          best = take ? key : best;
+          boff = take ? o : boff;
+        }
+        if (jb < nout) {
+          const int64_t idx = (rowk + k) * f.nblk + jb / Bk;
+          f.key[idx] = best;
+          f.off[idx] = (uint8_t)(best ? boff : 0);
         }
       }
     }
@@ -1797,7 +1860,7 @@ cudaError_t make_ring_map(CUtensorMap* map, const void* ring, int is_u16, int64_
 bool fused_smem(int is_u16, int row_slot, int zcap, int pitch, int nstage, int hp,
                 int32_t* e_off, size_t* smem) {
   const SmemLayout L = smem_layout(is_u16 ? 2 : 1, row_slot, zcap, pitch, nstage);
-  const size_t rows = (size_t)kWarps * (hp + 512) * sizeof(uint32_t);
+  const size_t rows = (size_t)kWarps * fused_row_words(hp) * sizeof(uint32_t);
   size_t total = L.total, off = L.raw;
   if (L.tab - L.raw < rows) {  // the staging area is too small: the rows go after it
     off = L.total;

@@ -168,3 +168,36 @@ def test_wide_trial_tile(trials, sizes):
     finally:
         plan.close()
     check(w, x[:sum(sizes)], sizes, 2)
+
+
+@pytest.mark.parametrize("block", [2, 16, 32])
+@pytest.mark.parametrize("widths", [(1, 2, 3, 17, 100, 301, 512), (2, 6)])
+def test_fused_blocks_equal_plain(block, widths):
+    """The fused search's two block loops (16 and 32 samples; smaller) over widths of every
+    residue mod 4, segment starts and ragged windows: the plain path's candidates, SNRs included,
+    one for every block (threshold far below any SNR)."""
+    ranges = (configs.DMRange(0.0, 0.0625, 70, 1), configs.DMRange(4.375, 0.125, 20, 2))
+    w = configs.mid(nsamp=1 << 14, chunk_len=4096, n_streams=1, npulses=3, nchans=4096,
+                    ranges=ranges, index=76)
+    w.nchans, w.foff = 128, -300.0 / 1024
+    x = torch.from_numpy(w.generate(_arrivals(w))).cuda()
+    got = []
+    for fuse in (True, False):
+        plan = dd.Plan(w.freqs(), w.tsamp, w.ranges_array(), 6144, n_streams=1,
+                       max_width=max(widths), peak_block=block)
+        try:
+            if fuse:
+                assert plan.fuse_search(widths) == 2
+            out, T = [], 0
+            for n in (6144, 5000, 1030, 4210 - 1):
+                n -= n % 2
+                seq = plan.run(x[T:T + n], n)
+                T += n
+                plan.search(widths, -1e30)
+                out.append(plan.candidates(seq))
+        finally:
+            plan.close()
+        got.append(np.concatenate(out))
+    assert got[0].size == got[1].size > 1000
+    for f in ("range", "trial", "t_start", "width", "snr"):
+        np.testing.assert_array_equal(got[0][f], got[1][f], err_msg=f)
