@@ -10,6 +10,8 @@
 #include <math.h>
 
 #include <algorithm>
+#include <climits>
+#include <type_traits>
 
 #include "dd_internal.h"
 
@@ -504,6 +506,32 @@ __device__ __forceinline__ uint4 prefix4(const uint32_t* P, int idx, int w) {
   return make_uint4(a.w, b.x, b.y, b.z);
 }
 
+// A width's alignment, decided once per width (it is the same in every lane) instead of per load:
+// M = -w mod 4 entries into the aligned chunk; OWN: w < 4 with M > 0, where the second chunk is the
+// lane's own four prefix sums. f takes both as integral constants.
+template <typename F>
+__device__ __forceinline__ void by_alignment(int w, F&& f) {
+  const int m = (-w) & 3;
+  if (m == 0) f(std::integral_constant<int, 0>(), std::bool_constant<false>());
+  else if (w == 1) f(std::integral_constant<int, 3>(), std::bool_constant<true>());
+  else if (w == 2) f(std::integral_constant<int, 2>(), std::bool_constant<true>());
+  else if (m == 1) f(std::integral_constant<int, 1>(), std::bool_constant<false>());
+  else if (m == 2) f(std::integral_constant<int, 2>(), std::bool_constant<false>());
+  else f(std::integral_constant<int, 3>(), std::bool_constant<false>());
+}
+
+// Entries P[idx - w .. idx - w + 3] (q: P + idx, v: the lane's own entries P[idx .. idx + 3]).
+template <int M, bool OWN>
+__device__ __forceinline__ uint4 earlier4(const uint32_t* q, int w, const uint4& v) {
+  const uint4* c = reinterpret_cast<const uint4*>(q - w - M);
+  const uint4 a = c[0];
+  if (M == 0) return a;
+  const uint4 b = OWN ? v : c[1];
+  if (M == 1) return make_uint4(a.y, a.z, a.w, b.x);
+  if (M == 2) return make_uint4(a.z, a.w, b.x, b.y);
+  return make_uint4(a.w, b.x, b.y, b.z);
+}
+
 // A warp's view of one series. The search kernels give each warp a segment of consecutive
 // samples of one trial, taken in passes of kSpsPass samples: lane l owns the 4-sample chunks
 // 4l + 128 g (g = 0..3) of the pass. The warp's own shared-memory row P holds uint32 prefix sums
@@ -634,12 +662,15 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_sps(const SpsArgs a, const l
   // Per width k: SNR = (ca[k] * B - cb[k]) / den[k]. Window statistics: ca = n, cb = w * S1,
   // den = sqrt(w) * sqrt(n * S2 - S1^2). Clipped per-width statistics (a.wst): ca = N_k,
   // cb = T1_k, den = sqrt(N_k * T2_k - T1_k^2). A width with den 0 gives no candidates.
-  if (a.wst == nullptr) {
+  // One warp works them out (FP64 is slow here, and eight warps would share its pipe).
+  __shared__ int constant;  // a constant series has no candidates
+  if (wid > 0) {
+  } else if (a.wst == nullptr) {
     const Moments m = a.mom[i];
     const long long s1 = (long long)m.s1;
     const double sq = window_sqrt_var(m, n);
-    if (sq == 0.0) return;  // constant series: no candidates
-    if (tid < a.nw) {
+    if (tid == 0) constant = sq == 0.0;
+    if (tid < a.nw && sq != 0.0) {
       const int w = a.wd[tid];
       den[tid] = sqrt((double)w) * sq;
       ca[tid] = n;
@@ -647,6 +678,7 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_sps(const SpsArgs a, const l
       bthr[tid] = window_bound(w, s1, thr, den[tid], n);
     }
   } else if (tid < a.nw) {
+    if (tid == 0) constant = 0;
     const WidthStats st = a.wst[(int64_t)i * a.nw + tid];
     const unsigned long long un = (unsigned long long)st.n, ut1 = (unsigned long long)st.t1;
     const unsigned long long p_lo = un * st.t2lo;
@@ -665,6 +697,7 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_sps(const SpsArgs a, const l
                       : (tl <= 0.0 ? 0u : (tl >= 4294967295.0 ? 0xFFFFFFFFu : (uint32_t)floor(tl)));
   }
   __syncthreads();  // the only CTA barrier: the widths' statistics
+  if (constant) return;
   const long long s0 = ((long long)blockIdx.y * kSpsWarps + wid) * seg;
   if (s0 >= n) return;
   const long long s1 = s0 + seg < n ? s0 + seg : n;
@@ -693,19 +726,29 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_sps(const SpsArgs a, const l
     // ---- filter: every boxcar sum of this lane's samples against the bounds
     const bool interior = j0 >= wmax - 1 && j0 + kSpsPass <= n;  // every (sample, width) valid
     bool hot[4] = {false, false, false, false};
+    const uint32_t* Pq = P + 1 + H + 4 * lane;
     if (interior) {
+      // sums are below 2^31 (a wrapped one, from negative input, is passed over by the exact
+      // search): the largest sum less the bound, over the widths
+      int over[4] = {INT_MIN, INT_MIN, INT_MIN, INT_MIN};
 #pragma unroll 1
       for (int k = 0; k < nw; ++k) {
         const int w = a.wd[k];
-        const uint32_t t = bthr[k];
+        const int t = (int)min(bthr[k], 0x7FFFFFFFu);
+        by_alignment(w, [&](auto m, auto own) {
+          constexpr int M = decltype(m)::value;
+          constexpr bool OWN = decltype(own)::value;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          const uint4 st = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
-          const uint32_t mx = max(max(v[g].x - st.x, v[g].y - st.y),
-                                  max(v[g].z - st.z, v[g].w - st.w));
-          hot[g] |= mx >= t;
-        }
+          for (int g = 0; g < 4; ++g) {
+            const uint4 st = earlier4<M, OWN>(Pq + 128 * g, w, v[g]);
+            const int mx = max(max((int)(v[g].x - st.x), (int)(v[g].y - st.y)),
+                               max((int)(v[g].z - st.z), (int)(v[g].w - st.w)));
+            over[g] = max(over[g], max(mx, 0) - t);
+          }
+        });
       }
+#pragma unroll
+      for (int g = 0; g < 4; ++g) hot[g] = over[g] >= 0;
     } else {
 #pragma unroll 1
       for (int k = 0; k < nw; ++k) {
@@ -832,20 +875,24 @@ __global__ void __launch_bounds__(kSpsThreads) k_sps_fused(const SpsFusedArgs a)
   const int tid = threadIdx.x;
   const long long n = a.n;
   if (n <= 0) return;
-  const Moments m = a.mom[i];
-  const double sq = window_sqrt_var(m, n);
-  if (sq == 0.0) return;  // constant series: no candidates
+  __shared__ int constant;  // a constant series has no candidates
   const double thr = (double)a.threshold;
-  if (tid < a.nw) {
-    const int w = a.wd[tid];
-    den[tid] = sqrt((double)w) * sq;
-    ca[tid] = n;
-    cb[tid] = (long long)w * (long long)m.s1;
-    // a record can reach the threshold only if its sum passes k_sps's integer bound (key =
-    // sum + 1, so key > bound); the others are skipped before the FP64 SNR
-    kthr[tid] = window_bound(w, (long long)m.s1, thr, den[tid], n);
+  if (tid < 32) {  // one warp's FP64, as in k_sps
+    const Moments m = a.mom[i];
+    const double sq = window_sqrt_var(m, n);
+    if (tid == 0) constant = sq == 0.0;
+    if (tid < a.nw && sq != 0.0) {
+      const int w = a.wd[tid];
+      den[tid] = sqrt((double)w) * sq;
+      ca[tid] = n;
+      cb[tid] = (long long)w * (long long)m.s1;
+      // a record can reach the threshold only if its sum passes k_sps's integer bound (key =
+      // sum + 1, so key > bound); the others are skipped before the FP64 SNR
+      kthr[tid] = window_bound(w, (long long)m.s1, thr, den[tid], n);
+    }
   }
   __syncthreads();
+  if (constant) return;
   const int64_t row = (int64_t)i * a.nw;
   for (int64_t b = tid; b < a.nblk; b += kSpsThreads) {
     double bs = 0.0;
@@ -973,19 +1020,24 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_clip_stats(const ClipArgs a)
           uint32_t cn = cnts[32 * k];
           if (how == 2 && interior) {
             uint32_t sum = 0;
+            by_alignment(w, [&](auto m, auto own) {
+              constexpr int M = decltype(m)::value;
+              constexpr bool OWN = decltype(own)::value;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const uint4 s4 = prefix4(P, 1 + H + 4 * lane + 128 * g, w);
-              const uint32_t x[4] = {v[g].x - s4.x - lo, v[g].y - s4.y - lo, v[g].z - s4.z - lo,
-                                     v[g].w - s4.w - lo};
+              for (int g = 0; g < 4; ++g) {
+                const uint4 s4 = earlier4<M, OWN>(P + 1 + H + 4 * lane + 128 * g, w, v[g]);
+                const uint32_t x[4] = {v[g].x - s4.x - lo, v[g].y - s4.y - lo,
+                                       v[g].z - s4.z - lo, v[g].w - s4.w - lo};
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const uint32_t m = x[e] <= span ? x[e] : 0u;
-                if (x[e] <= span) ++cn;
-                sum += m;
-                c.c2 += (unsigned long long)m * m;
+                for (int e = 0; e < 4; ++e) {
+                  const bool in = x[e] <= span;
+                  const uint32_t xm = in ? x[e] : 0u;
+                  cn += in ? 1u : 0u;
+                  sum += xm;
+                  c.c2 += (unsigned long long)xm * xm;
+                }
               }
-            }
+            });
             c.c1 += sum;
           } else {
             uint32_t carry = 0;
