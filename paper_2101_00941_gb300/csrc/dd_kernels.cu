@@ -639,6 +639,8 @@ inline int64_t sps_segment(int n_trials, int64_t n, int hist) {
   while (seg > 2 * kSpsPass && seg / 2 >= 4 * hist &&
          n_trials * ((n + seg - 1) / seg) < 152 * 24)
     seg /= 2;
+  // a chip nearly idle: single passes, so that a bright pulse's groups spread over more warps
+  while (seg > kSpsPass && n_trials * ((n + seg - 1) / seg) < 152 * 4) seg /= 2;
   while ((n + seg * kSpsWarps - 1) / (seg * kSpsWarps) > 65535) seg *= 2;  // grid rows
   return seg;
 }
@@ -807,21 +809,31 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_sps(const SpsArgs a, const l
         }
         int kw = lane;
         if (have) bs = (double)(ca[lane] * (long long)mine - cb[lane]) / den[lane];
-        // the best width: largest SNR, then the earliest sample, then the smallest width
-        for (int o = 8; o > 0; o >>= 1) {
-          const double os = __shfl_xor_sync(0xffffffffu, bs, o);
-          const int oj = __shfl_xor_sync(0xffffffffu, moff, o);
-          const int ok = __shfl_xor_sync(0xffffffffu, kw, o);
-          const bool oh = __shfl_xor_sync(0xffffffffu, have ? 1 : 0, o) != 0;
-          if (oh && (!have || os > bs || (os == bs && (oj < moff || (oj == moff && ok < kw))))) {
-            have = true;
-            bs = os;
-            moff = oj;
-            kw = ok;
+        // The best width: largest SNR, then the earliest sample, then the smallest width. In
+        // FP32 first (a double's rounding to float is monotone, so the largest double is among
+        // the lanes holding the largest float); FP64 compares only where that leaves several.
+        const float fs = have ? (float)bs : -INFINITY;
+        float fm = fs;
+        for (int o = 8; o > 0; o >>= 1) fm = fmaxf(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+        const unsigned top = __ballot_sync(0xffffffffu, have && fs == fm) & 0xFFFFu;
+        if (__popc(top) > 1) {
+          for (int o = 8; o > 0; o >>= 1) {
+            const double os = __shfl_xor_sync(0xffffffffu, bs, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, moff, o);
+            const int ok = __shfl_xor_sync(0xffffffffu, kw, o);
+            const bool oh = __shfl_xor_sync(0xffffffffu, have ? 1 : 0, o) != 0;
+            if (oh && (!have || os > bs || (os == bs && (oj < moff || (oj == moff && ok < kw))))) {
+              have = true;
+              bs = os;
+              moff = oj;
+              kw = ok;
+            }
           }
+          leader = lane == 0;
+        } else {
+          leader = lane < 16 && ((top >> lane) & 1u) != 0;  // the winner writes
         }
-        leader = lane == 0;
-        bj = j + moff;
+        bj = j0 + c * 32 + moff;
         bwid = a.wd[kw & (kMaxWidths - 1)];
       } else {
         for (int k = 0; k < nw; ++k) {
