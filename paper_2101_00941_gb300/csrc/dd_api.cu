@@ -1103,14 +1103,11 @@ static int run_impl(dd_plan_t p, const uint8_t* chunk, int64_t nsamp, void* cuda
                             cudaMemcpyDeviceToDevice, st));
     DD_CK(cudaEventRecord(p->ev_hist, st));
   }
-  // hierarchical x2 decimation of the whole ring (history + new samples)
-  for (int l = 1; l <= p->levels; ++l) {
-    const void* in = (l == 1) ? (const void*)s.ring1 : (const void*)s.ringd[l - 1];
-    const int64_t in_stride = (l == 1) ? p->R1 : p->Rd[l - 1];
-    DD_CK(ddk::launch_decimate(in, l > 1, in_stride, s.ringd[l], p->Rd[l], p->Cp,
-                               (H + nsamp) >> l, st));
-    p->launches += 1;
-  }
+  // x2 decimation levels of the whole ring (history + new samples)
+  int nd = 0;
+  DD_CK(ddk::launch_decimate(s.ring1, p->R1, s.ringd + 1, p->Rd + 1, p->levels, p->Cp, H + nsamp,
+                             st, &nd));
+  p->launches += nd;
   // an external ordering point (serving: another beam's chunk must finish first); the copy,
   // corner turn and decimation above still overlap that chunk's work
   if (p->gate) {

@@ -295,8 +295,10 @@ cudaError_t launch_shift_table(const double* freqs, int32_t nchans, int32_t cpad
                                cudaStream_t st);
 cudaError_t launch_corner_turn(const uint8_t* in, int64_t n, int32_t nchans, uint8_t* ring,
                                int64_t ring_stride, int64_t col0, cudaStream_t st);
-cudaError_t launch_decimate(const void* in, int in_is_u16, int64_t in_stride, uint16_t* out,
-                            int64_t out_stride, int32_t cpad, int64_t n_out, cudaStream_t st);
+// Levels x2, x4, .. of the uint8 ring (n samples a row): out[l] has n >> (l + 1).
+cudaError_t launch_decimate(const uint8_t* in, int64_t in_stride, uint16_t* const* out,
+                            const int64_t* out_stride, int levels, int32_t cpad, int64_t n,
+                            cudaStream_t st, int* launches);
 cudaError_t launch_dedisp_naive(const DedispRange& r, int32_t cpad, cudaStream_t st);
 cudaError_t launch_dedisp_direct(const DedispRange& r, int32_t cpad, cudaStream_t st);
 cudaError_t launch_moments(const int32_t* y, int32_t ntr, int64_t n, int64_t stride, Moments* mom,

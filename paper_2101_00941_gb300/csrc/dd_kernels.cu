@@ -3,7 +3,7 @@
 //
 //   k_shift_table : FP64 delay table, one IEEE operation at a time (Sec. 3 DM plan)
 //   k_corner_turn : time-major uint8 spectra -> channel-major ring (Sec. 1 time chunks)
-//   k_decimate    : exact x2 time decimation, uint8/uint16 -> uint16
+//   k_decimate    : exact x2 time decimation levels, uint8/uint16 -> uint16
 //   k_dedisp_naive: one thread per output sample (reference-shaped; testing aid)
 //   k_moments     : exact S1 / 128-bit S2 of each series window (Sec. 2.2)
 //   k_sps         : boxcar SNR over prefix sums + block peak finding (Sec. 2.2)
@@ -162,26 +162,48 @@ cudaError_t launch_corner_turn(const uint8_t* in, int64_t n, int32_t nchans, uin
 
 // ------------------------------------------------------------------ decimation
 
-// out[c][m] = in[c][2m] + in[c][2m+1], four outputs per thread. Channels c = blockIdx.y,
-// blockIdx.y + gridDim.y, ... (a grid dimension holds at most 65535 of them).
-__global__ void k_decimate_u8(const uint8_t* __restrict__ in, int64_t in_stride,
-                              uint16_t* __restrict__ out, int64_t out_stride, int64_t n_out,
-                              int32_t cpad) {
+// Levels x2 .. x2^LEVELS of the uint8 ring in one pass: 16 samples per thread, 8, 4, 2 and 1 sums
+// of them stored. Bound by memory: the ring is read once and each level written once, 2.9 bytes
+// per sample with four levels against 4.6 when every level read the one before. Channels c =
+// blockIdx.y, blockIdx.y + gridDim.y, ... (a grid dimension holds at most 65535 of them). The
+// last thread of a row may read and write past the data, into the rows' slack.
+struct DecimateArgs {
+  const uint8_t* in;
+  int64_t in_stride;
+  uint16_t* out[4];
+  int64_t out_stride[4];
+  int64_t n;  // samples
+  int32_t cpad;
+};
+
+template <int LEVELS>
+__global__ void __launch_bounds__(256) k_decimate_u8(const DecimateArgs a) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (4 * k >= n_out) return;
-  for (int64_t c = blockIdx.y; c < cpad; c += gridDim.y) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(in + c * in_stride + 8 * k));
-    const uint32_t lo = (v.x & 0xFFu) + ((v.x >> 8) & 0xFFu);
-    const uint32_t hi = ((v.x >> 16) & 0xFFu) + (v.x >> 24);
-    const uint32_t lo2 = (v.y & 0xFFu) + ((v.y >> 8) & 0xFFu);
-    const uint32_t hi2 = ((v.y >> 16) & 0xFFu) + (v.y >> 24);
-    uint2 o;
-    o.x = lo | (hi << 16);
-    o.y = lo2 | (hi2 << 16);
-    *reinterpret_cast<uint2*>(out + c * out_stride + 4 * k) = o;
+  if (16 * k >= a.n) return;
+  for (int64_t c = blockIdx.y; c < a.cpad; c += gridDim.y) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.in + c * a.in_stride + 16 * k));
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t p[4];  // level 1: two 16-bit sums a word
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = (w[i] & 0x00FF00FFu) + ((w[i] >> 8) & 0x00FF00FFu);
+    *reinterpret_cast<uint4*>(a.out[0] + c * a.out_stride[0] + 8 * k) =
+        make_uint4(p[0], p[1], p[2], p[3]);
+    if (LEVELS < 2) continue;
+    uint32_t q[2];  // level 2: four sums (below 2^10) in two words
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      q[i] = ((p[2 * i] & 0xFFFFu) + (p[2 * i] >> 16)) |
+             ((p[2 * i + 1] & 0xFFFFu) + (p[2 * i + 1] >> 16)) << 16;
+    *reinterpret_cast<uint2*>(a.out[1] + c * a.out_stride[1] + 4 * k) = make_uint2(q[0], q[1]);
+    if (LEVELS < 3) continue;
+    const uint32_t r = ((q[0] & 0xFFFFu) + (q[0] >> 16)) | ((q[1] & 0xFFFFu) + (q[1] >> 16)) << 16;
+    *reinterpret_cast<uint32_t*>(a.out[2] + c * a.out_stride[2] + 2 * k) = r;
+    if (LEVELS < 4) continue;
+    a.out[3][c * a.out_stride[3] + k] = (uint16_t)((r & 0xFFFFu) + (r >> 16));
   }
 }
 
+// out[c][m] = in[c][2m] + in[c][2m+1] of a uint16 level (beyond x16), four outputs per thread.
 __global__ void k_decimate_u16(const uint16_t* __restrict__ in, int64_t in_stride,
                                uint16_t* __restrict__ out, int64_t out_stride, int64_t n_out,
                                int32_t cpad) {
@@ -198,16 +220,35 @@ __global__ void k_decimate_u16(const uint16_t* __restrict__ in, int64_t in_strid
   }
 }
 
-cudaError_t launch_decimate(const void* in, int in_is_u16, int64_t in_stride, uint16_t* out,
-                            int64_t out_stride, int32_t cpad, int64_t n_out, cudaStream_t st) {
-  if (n_out <= 0) return cudaSuccess;
-  dim3 grid((unsigned)(((n_out + 3) / 4 + 255) / 256), (unsigned)std::min(cpad, 65535));
-  if (in_is_u16)
-    k_decimate_u16<<<grid, 256, 0, st>>>(static_cast<const uint16_t*>(in), in_stride, out,
-                                         out_stride, n_out, cpad);
-  else
-    k_decimate_u8<<<grid, 256, 0, st>>>(static_cast<const uint8_t*>(in), in_stride, out,
-                                        out_stride, n_out, cpad);
+cudaError_t launch_decimate(const uint8_t* in, int64_t in_stride, uint16_t* const* out,
+                            const int64_t* out_stride, int levels, int32_t cpad, int64_t n,
+                            cudaStream_t st, int* launches) {
+  *launches = 0;
+  if (n <= 0 || levels < 1) return cudaSuccess;
+  DecimateArgs a;
+  a.in = in;
+  a.in_stride = in_stride;
+  const int first = std::min(levels, 4);
+  for (int l = 0; l < 4; ++l) {
+    a.out[l] = l < first ? out[l] : nullptr;
+    a.out_stride[l] = l < first ? out_stride[l] : 0;
+  }
+  a.n = n;
+  a.cpad = cpad;
+  const dim3 grid((unsigned)((n + 16 * 256 - 1) / (16 * 256)), (unsigned)std::min(cpad, 65535));
+  if (first == 1) k_decimate_u8<1><<<grid, 256, 0, st>>>(a);
+  else if (first == 2) k_decimate_u8<2><<<grid, 256, 0, st>>>(a);
+  else if (first == 3) k_decimate_u8<3><<<grid, 256, 0, st>>>(a);
+  else k_decimate_u8<4><<<grid, 256, 0, st>>>(a);
+  *launches = 1;
+  for (int l = 4; l < levels; ++l) {
+    const int64_t n_out = n >> (l + 1);
+    if (n_out <= 0) break;
+    const dim3 g((unsigned)(((n_out + 3) / 4 + 255) / 256), (unsigned)std::min(cpad, 65535));
+    k_decimate_u16<<<g, 256, 0, st>>>(out[l - 1], out_stride[l - 1], out[l], out_stride[l], n_out,
+                                      cpad);
+    *launches += 1;
+  }
   return cudaGetLastError();
 }
 
