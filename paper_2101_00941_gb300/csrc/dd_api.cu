@@ -734,21 +734,21 @@ int dd_plan(const double* freqs_mhz, int32_t nchans, double tsamp_s, const dd_ra
     p->rk.resize(nranges);
     if (!(o.flags & DD_FLAG_NAIVE)) {
       for (int r = 0; r < nranges; ++r) {
-        // the first shape that fits, in kShapes order; testing aids force the 256-output tile
-        // (DD_FLAG_TILE256) or the 32-trial tile (DD_FLAG_TRIALS32)
+        // The first shape that fits, in kShapes order; testing aids force the 256-output tile
+        // (DD_FLAG_TILE256) or the 32-trial tile (DD_FLAG_TRIALS32).
         // 128 trials x 256 outputs share each class's words among more trials than 64 x 512, but
         // round the trials up to 128 and see a wider spread of delays: by the estimated work of
-        // the launch (tiled_cost). Both measured on the 4096-channel plan, x1 / x2 / x4 / x8:
-        // 17.0 / 5.5 / 2.9 / 2.0 ms with 64 x 512 (about), 15.5 / 4.7 / 2.5 / 1.7 with 128 x 256;
-        // on the 1024-channel plan, whose spread per trial is as large and whose classes are more,
-        // 2.39 / 0.80 / 0.39 against 2.38 / 0.77 / 0.36
+        // the launch (tiled_cost). Measured, 64 x 512 against 128 x 256, ms per range: 4096-channel
+        // plan x1 .. x8 16.0 / 5.2 / 2.8 / 1.9 against 14.7 / 4.6 / 2.4 / 1.7; 8192-channel plan
+        // x2 .. x16 20.7 / 10.6 / 6.9 / 7.3 against 20.4 / 10.5 / 6.4 / 6.7 (x1, whose delays
+        // spread 291 samples over 64 trials: equal); 1024-channel plan x1 .. x4 2.27 / 0.77 / 0.38
+        // against 2.26 / 0.74 / 0.35. A launch that leaves SMs idle keeps the 512-output tile.
         const int64_t nout = o.chunk_len / ranges[r].decimation;
         const int32_t* rt = &full[(size_t)p->row0[r] * p->Cp];
         const double c64 = ddk::tiled_cost(rt, ranges[r].n_trials, p->Cp, ranges[r].decimation,
                                            512, 64, 512, nout, p->sms);
         const double c128 = ddk::tiled_cost(rt, ranges[r].n_trials, p->Cp, ranges[r].decimation,
                                             256, 128, 512, nout, p->sms);
-        // (a launch that leaves SMs idle keeps the 512-output tile)
         const bool fills = (int64_t)((ranges[r].n_trials + 63) / 64) * ((nout + 511) / 512) >= p->sms;
         const bool wide = fills && c128 >= 0 && (c64 < 0 || c128 < 0.97 * c64);
         for (int k = 0; k < kNumShapes && !p->rk[r].tiled; ++k) {

@@ -2,10 +2,12 @@
 // plain definition y[i][j] = sum_c x_d[c][j + s[i][c]], computed exactly in integers).
 //
 // One CTA owns a tile of D consecutive DM trials x TT output samples of one range and walks the
-// channels in stages of kNG groups of eight channels. Tile shapes (the plan picks the first that
-// fits, or times them all): 64 x 512 with 16 warps (128 registers per thread, 64 accumulators
-// per lane), the same tile with 32 warps (64 registers, 32 accumulators: twice the warps on the
-// same tables and shared memory), and 64 x 256 or 32 x 256 with 16 warps, two CTAs per SM.
+// channels in stages of kNG groups of eight channels. Tile shapes (the plan picks one by the
+// launch's estimated work, or times them all): 64 x 512 or 128 x 256 with 16 warps (128 registers
+// per thread, 64 accumulators per lane), 64 x 512 with 32 warps (64 registers, 32 accumulators:
+// twice the warps on the same tables and shared memory), and 64 x 256 or 32 x 256 with 16 warps,
+// two CTAs per SM. Bound by the shared-memory pipe (71% busy) and instruction issue (58%): 1216
+// trials x 65536 outputs x 4096 channels take 6.2 ms (uint8; 8.5 without the class chains).
 //
 //   * Delay classes. For an 8-channel group the tile's trials fall into a few classes by the
 //     relative delays (r0..r7) of the eight channels. A class shares one sequence of sums
