@@ -1208,12 +1208,16 @@ cudaError_t prepare_t(size_t smem) {
 
 namespace {
 
-// Instruction costs of a build task, for dealing tasks to warps: its set-up with the eight
-// channels of its first class, each link's store, each channel step (counted from build_stage).
+// Costs of a build task, for dealing tasks to warps: its set-up with the eight channels of its
+// first class, each link's store, each channel step. In instructions they would be about 100, 16,
+// 18 (uint8) and 80, 13, 14 (uint16); a task's set-up is a chain of dependent shared-memory reads
+// that a warp waits for, and counting it more than twice measured best (1216 trials x 65536 outputs x
+// 4096 channels, ms a run, uint8 / uint16: 6.37 / 4.01 with the instruction counts, 6.31 / 3.94
+// with 130 and 110, 6.29 / 3.92 with 170 and 140, 6.28 / 3.91 with these).
 struct BuildCost {
   int base, emit, step;
 };
-constexpr BuildCost kCostU8{100, 16, 18}, kCostU16{80, 13, 14};
+constexpr BuildCost kCostU8{230, 16, 18}, kCostU16{190, 13, 14};
 
 // Deal a stage's build work to W warps: per group and block of 31 units, the chain of links,
 // from and to classes that store units in the block, cut where the plan breaks the chain
