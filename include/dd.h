@@ -547,6 +547,24 @@ int dd_tiled_plan_check(const int32_t* shifts, int32_t n_trials, int32_t cpad,
                         int32_t* ok, int64_t* violations);
 
 /*
+ * dd_staged_plan_check -- host-only check of the staged direct kernel's plan for one range (no
+ * GPU, no CUDA call): walks the launch dd_run would make for one chunk, with the kernel's own copy
+ * arithmetic. Every copy lies inside its ring row and holds every sample its trials add; every
+ * trial's words lie inside the frame. (A plan asks the tiled kernel first; of the ranges it
+ * refuses, those this one refuses too run on the cached-read kernel. Both direct kernels are
+ * DD_KERNEL_DIRECT.)
+ *   shifts     : int32 [n_trials][cpad], as for dd_tiled_plan_check
+ *   overlap    : the plan's overlap O; chunk_len: the plan's option; before: samples given to
+ *                dd_run before the chunk; nsamp: the chunk's samples (all original samples)
+ *   ok         : receives 1 if the staged kernel can run the range, else 0
+ *   violations : receives the number of violated checks (0 expected; 0 when ok is 0)
+ * Errors: DD_ERR_ARG.
+ */
+int dd_staged_plan_check(const int32_t* shifts, int32_t n_trials, int32_t cpad,
+                         int32_t decimation, int64_t overlap, int64_t chunk_len, int64_t before,
+                         int64_t nsamp, int32_t* ok, int64_t* violations);
+
+/*
  * dd_selftest_wait -- failure-detection self-test of the device-side bounded wait. The tiled
  * dedispersion kernel waits on each stage's copy barrier for at most 2 s (or 2^26 polls); when
  * that runs out it sets an error bit that dd_candidates reports as DD_ERR_TIMEOUT, waits (again

@@ -38,7 +38,7 @@ DD_BATCH_AUTOTUNE = 2
 DD_BATCH_PERSISTENT = 4
 
 EXPORTS = ("dd_plan", "dd_plan_info", "dd_plan_kernel", "dd_selftest_wait",
-           "dd_tiled_plan_check", "dd_run", "dd_series", "sps_run", "dd_candidates", "dd_sync",
+           "dd_tiled_plan_check", "dd_staged_plan_check", "dd_run", "dd_series", "sps_run", "dd_candidates", "dd_sync",
            "dd_stats", "dd_sps_static", "dd_serve_create", "dd_serve_add_beam", "dd_serve_submit",
            "dd_serve_poll", "dd_serve_pending", "dd_serve_destroy", "dd_batch_create",
            "dd_batch_run", "dd_batch_wait", "dd_batch_info", "dd_batch_candidates",
@@ -125,6 +125,7 @@ def lib() -> ctypes.CDLL:
         L.dd_plan_kernel.argtypes = [vp, i32, P(i32), P(i32)]
         L.dd_selftest_wait.argtypes = [i32, P(i32), P(ctypes.c_double)]
         L.dd_tiled_plan_check.argtypes = [vp, i32, i32, i32, i32, i32, P(i32), P(i64)]
+        L.dd_staged_plan_check.argtypes = [vp, i32, i32, i32, i64, i64, i64, i64, P(i32), P(i64)]
         L.dd_run.argtypes = [vp, vp, i64, vp]
         L.dd_series.argtypes = [vp, i32, P(vp), P(i64), P(i64), P(i64)]
         L.sps_run.argtypes = [vp, vp, i32, f32]
@@ -236,6 +237,18 @@ def dd_tiled_plan_check(shifts, decimation: int, tile_samples: int = 512, tile_t
     _check(lib().dd_tiled_plan_check(a.ctypes.data, a.shape[0], a.shape[1], int(decimation),
                                      int(tile_samples), int(tile_trials), ctypes.byref(ok),
                                      ctypes.byref(bad)))
+    return ok.value, bad.value
+
+
+def dd_staged_plan_check(shifts, decimation: int, overlap: int, chunk_len: int, before: int,
+                         nsamp: int):
+    """Host-only check of the staged direct kernel's launch over one chunk of a range (see dd.h):
+    (ok, violations). `shifts` is int32 [n_trials][cpad] with cpad a multiple of 8."""
+    a = np.ascontiguousarray(shifts, dtype=np.int32)
+    ok, bad = ctypes.c_int32(), ctypes.c_int64()
+    _check(lib().dd_staged_plan_check(a.ctypes.data, a.shape[0], a.shape[1], int(decimation),
+                                      int(overlap), int(chunk_len), int(before), int(nsamp),
+                                      ctypes.byref(ok), ctypes.byref(bad)))
     return ok.value, bad.value
 
 

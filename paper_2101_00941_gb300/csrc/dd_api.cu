@@ -48,6 +48,15 @@ int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
 bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 
+// Elements of a ring row (level l: x2^l decimated) for `span` samples of history and chunk: rows
+// carry slack past the data so a ragged last time tile may stage (and ignore) a full tile, and,
+// where a range runs on the staged direct kernel (frame > 0: the plan's largest), a full staged row.
+int64_t ring_row(int64_t span, int l, int frame) {
+  const int64_t slack =
+      std::max<int64_t>(2048, frame > 0 ? round_up(ddk::staged_slack(frame), 256) : 0);
+  return (l == 0 ? round_up(span, 256) : round_up(span >> l, 128)) + slack;
+}
+
 int ilog2(int64_t v) {
   int l = 0;
   while ((int64_t(1) << l) < v) ++l;
@@ -782,9 +791,10 @@ int dd_plan(const double* freqs_mhz, int32_t nchans, double tsamp_s, const dd_ra
   // history kept on the device: O rounded up so every ring row starts 256-byte aligned
   p->H = round_up(p->O, 256);
   const int64_t span = p->H + p->L;
-  // rows carry slack past the data so a ragged last time tile may stage (and ignore) a full tile
-  p->R1 = round_up(span, 256) + 2048;
-  for (int l = 1; l <= p->levels; ++l) p->Rd[l] = round_up(span >> l, 128) + 2048;
+  int frame = 0;
+  for (const auto& k : p->rk) frame = std::max(frame, k.frame);
+  p->R1 = ring_row(span, 0, frame);
+  for (int l = 1; l <= p->levels; ++l) p->Rd[l] = ring_row(span, l, frame);
   p->series_off.resize(nranges);
   p->series_stride.resize(nranges);
   int64_t off = 0;
@@ -1423,6 +1433,28 @@ int dd_candidates(dd_plan_t p, int64_t seq, dd_cand_t* out, int64_t cap, int64_t
   if (count > cap || count > p->opts.max_cands)
     return fail(DD_ERR_CAP, "%lld candidates exceed the buffer (cap %lld, max_cands %lld)",
                 (long long)count, (long long)cap, (long long)p->opts.max_cands);
+  return DD_OK;
+}
+
+int dd_staged_plan_check(const int32_t* shifts, int32_t n_trials, int32_t cpad,
+                         int32_t decimation, int64_t overlap, int64_t chunk_len, int64_t before,
+                         int64_t nsamp, int32_t* ok, int64_t* violations) {
+  if (!shifts || !ok || !violations) return fail(DD_ERR_ARG, "NULL argument");
+  if (n_trials < 1 || cpad < 8 || cpad % 8 || !is_pow2(decimation) || decimation > 256 ||
+      overlap < 0 || before < 0 || nsamp < 1 || nsamp > chunk_len)
+    return fail(DD_ERR_ARG, "need n_trials >= 1, cpad a multiple of 8, decimation a power of two "
+                            "<= 256, 1 <= nsamp <= chunk_len, overlap and before >= 0");
+  // the window and ring of dd_run
+  const int64_t H = round_up(overlap, 256);
+  const int64_t lo = std::max<int64_t>(0, before - overlap);
+  const int64_t hi = std::max<int64_t>(0, before + nsamp - overlap);
+  int frame = 0;
+  *violations = 0;
+  *ok = ddk::staged_plan(shifts, n_trials, cpad, decimation, &frame);
+  if (*ok)
+    *violations = ddk::staged_plan_check(
+        shifts, n_trials, cpad, decimation, frame, (lo - (before - H)) / decimation,
+        (hi - lo) / decimation, ring_row(H + chunk_len, ilog2(decimation), frame));
   return DD_OK;
 }
 

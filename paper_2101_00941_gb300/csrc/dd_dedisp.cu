@@ -1011,6 +1011,15 @@ struct StagedLayout {
   int row;  // bytes of a staged row
 };
 
+// Where a staged row's copy starts in its ring row (bytes; at: ring column of the tile's first
+// sample at the tile's smallest delay). Every copy takes a whole staged row (StagedLayout::row),
+// as long as the widest trial tile of the range needs, from there: a tile of few trials that
+// starts at the largest delay, with few outputs left, copies up to frame + 32 samples past the
+// data, and the plan's ring rows are that long (staged_slack).
+__host__ __device__ inline int64_t staged_copy_start(int64_t at, int es) {
+  return at * es & ~(int64_t)15;
+}
+
 // frame: pair words per channel, a multiple of 8; the raw rows come first
 __host__ __device__ inline StagedLayout staged_layout(int es, int frame) {
   StagedLayout L;
@@ -1044,7 +1053,7 @@ __global__ void __launch_bounds__(512, 1) k_dedisp_staged(const StagedArgs a) {
   // copies: 64 threads per row
   const int crow = tid >> 6, cchunk = tid & 63;
   auto copy_rows = [&](int s, int32_t sfirst) {
-    const int64_t byte = (a.m0 + j0 + sfirst) * es & ~(int64_t)15;
+    const int64_t byte = staged_copy_start(a.m0 + j0 + sfirst, es);
     const unsigned char* src = static_cast<const unsigned char*>(a.xd) +
                                (int64_t)((sb + s) * kSC + crow) * a.xd_stride * es + byte;
     const uint32_t dst = sraw + (uint32_t)((s & 1) * kSC + crow) * (uint32_t)SL.row;
@@ -1964,6 +1973,37 @@ int staged_plan(const int32_t* tab, int ntr, int cpad, int decimation, int* fram
   if (staged_layout(es, (int)f).total > kSmemLimit) return 0;
   *frame = (int)f;
   return 1;
+}
+
+int64_t staged_slack(int frame) { return frame + 32; }
+
+// Host: walk the staged kernel's launch over a window of nout outputs from ring column m0 on, in
+// ring rows of row_len elements, with the kernel's own copy arithmetic. Returns the number of
+// violations of:
+//   - every 16-byte copy of every row lies inside the ring row;
+//   - the copied bytes hold every sample the tile's trials add;
+//   - every trial's pair words lie inside their plane of the frame.
+int64_t staged_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, int frame,
+                          int64_t m0, int64_t nout, int64_t row_len) {
+  const int es = decimation > 1 ? 2 : 1;
+  const StagedLayout L = staged_layout(es, frame);
+  const int64_t ring_row = row_len * es;
+  int64_t bad = ring_row % 16 != 0 || L.row % 16 != 0 || frame % 8 != 0;
+  for (int t0 = 0; t0 < ntr; t0 += kStTrials)
+    for (int64_t j0 = 0; j0 < nout; j0 += kStOut)
+      for (int c = 0; c < cpad; ++c) {
+        const int64_t byte = staged_copy_start(m0 + j0 + tab[(int64_t)t0 * cpad + c], es);
+        const int64_t end = byte + L.row;
+        bad += byte < 0 || byte % 16 != 0 || end > ring_row;
+        const int64_t left = std::min<int64_t>(kStOut, nout - j0);
+        for (int t = t0; t < std::min(ntr, t0 + kStTrials); ++t) {
+          const int64_t first = m0 + j0 + tab[(int64_t)t * cpad + c];
+          const int64_t o = first - byte / es;  // the trial's first word
+          bad += first * es < byte || (first + left) * es > end;
+          bad += o < 0 || o / 2 + kStOut / 2 > frame / 2;
+        }
+      }
+  return bad;
 }
 
 cudaError_t prepare_staged(int is_u16) {

@@ -238,6 +238,10 @@ cudaError_t launch_sps_fused(const SpsFusedArgs& a, cudaStream_t st);
 // Whether a range's delays fit the staged direct kernel (no delay falls with the trial, and the
 // rows of 64 trials fit shared memory); *frame: StagedArgs::frame.
 int staged_plan(const int32_t* shifts, int ntr, int cpad, int decimation, int* frame);
+// Samples past the data that a staged row's copy may take: the slack its ring rows need.
+int64_t staged_slack(int frame);
+int64_t staged_plan_check(const int32_t* shifts, int ntr, int cpad, int decimation, int frame,
+                          int64_t m0, int64_t nout, int64_t row_len);
 cudaError_t prepare_staged(int is_u16);
 // *launches: kernels launched (more than one where few tiles split the channels among CTAs).
 cudaError_t launch_staged(const StagedArgs& a, int is_u16, int sms, cudaStream_t st,

@@ -149,6 +149,38 @@ def test_staged_direct_kernel(nchans, trials, sizes):
     check(w, x[:sum(sizes)], sizes, 1)
 
 
+def _staged_takes(w, chunk_len):
+    """Whether the staged direct kernel takes each range of w (of those the tiled kernel refuses)."""
+    tabs = oracle.shift_tables(w.freqs(), w.tsamp, w.ranges_array())
+    O = oracle.overlap(tabs, w.ranges_array())
+    out = []
+    for t, r in zip(tabs, w.ranges):
+        t = np.pad(t, ((0, 0), (0, -t.shape[1] % 8)), mode="edge").astype(np.int32)
+        ok, bad = dd.dd_staged_plan_check(t, r.decimation, O, chunk_len, 0, chunk_len)
+        assert bad == 0
+        out.append(ok)
+    return out
+
+
+@pytest.mark.parametrize("ranges,sizes", [
+    (((0.0, 1.4, 65, 1),), [8448, 8448, 300]),
+    (((0.0, 2.4, 65, 2), (0.0, 1.2, 65, 1)), [8448, 8446, 258])])
+def test_staged_kernel_widest_rows(ranges, sizes):
+    """Trial tiles whose rows fill shared memory, and a last tile of one trial at the largest
+    delay: its rows end where the ring ends."""
+    w = _coarse(tuple(configs.DMRange(*r) for r in ranges), 64, 1 << 15, 77, bw=400.0)
+    w.fch1, w.widths = 1500.0, (2, 4, 64, 256)
+    x = w.generate(_arrivals(w))
+    assert _staged_takes(w, 8448) == [1] * len(ranges)
+    plan = dd.Plan(w.freqs(), w.tsamp, w.ranges_array(), 8448, n_streams=1, max_width=256)
+    try:
+        for r in range(len(ranges)):
+            assert plan.kernel(r)[0] == dd.DD_KERNEL_DIRECT
+    finally:
+        plan.close()
+    check(w, x[:sum(sizes)], sizes, 1)
+
+
 @pytest.mark.parametrize("trials,sizes", [(1024, [10240, 10240]), (1000, [10240, 10238, 9000])])
 def test_wide_trial_tile(trials, sizes):
     """Plans that take the 128-trial tile, for uint8 and uint16 data: full and ragged last tiles,

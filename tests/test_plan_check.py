@@ -117,3 +117,49 @@ def test_128_trial_tile_on_the_workloads():
     for w in (configs.mid(nsamp=1 << 17), configs.out_of_core(nsamp=1 << 20)):
         for tab, r in list(zip(_tables(w), w.ranges))[::3]:
             assert dd.dd_tiled_plan_check(tab, r.decimation, 256, 128) == (1, 0), r
+
+
+def _staged(nchans, bw, ranges, chunk, sizes):
+    """Violations of the staged direct kernel's launches over the chunks of a 1500 MHz, 64 us plan,
+    and which ranges it takes."""
+    w = configs.mid(nsamp=1 << 15, ranges=tuple(configs.DMRange(*r) for r in ranges))
+    w.nchans, w.fch1, w.foff = nchans, 1500.0, -bw / nchans
+    tabs = _tables(w)
+    O = oracle.overlap(tabs, w.ranges_array())
+    bad, oks, T = 0, [], 0
+    for n in sizes:
+        for t, r in zip(tabs, w.ranges):
+            ok, b = dd.dd_staged_plan_check(t, r.decimation, O, chunk, T, n)
+            oks.append(ok)
+            bad += b
+        T += n
+    return bad, oks
+
+
+# coarse channels with wide DM steps: a trial tile's delays spread over up to the widest frame of
+# the kernel's shared memory, and the last trial tile, of few trials, starts at the largest delay
+@pytest.mark.parametrize("nchans,bw,ranges,chunk,sizes", [
+    (256, 400.0, [(0.0, 1.4, 193, 1)], 8192, [8192, 8192]),
+    (256, 400.0, [(0.0, 1.3, 193, 1)], 8192, [8192, 8192]),
+    (64, 400.0, [(0.0, 1.4, 65, 1)], 65792, [65792, 65792, 300]),
+    (64, 400.0, [(0.0, 1.2, 65, 1)], 8448, [8448, 8448, 1]),
+    (64, 400.0, [(0.0, 2.4, 65, 2)], 8448, [8448, 8448, 2]),
+    (64, 400.0, [(0.0, 9.0, 129, 8), (0.0, 1.25, 449, 1)], 8448, [8448, 8192, 4104, 8448]),
+    (41, 400.0, [(30.0, 60.0, 66, 64)], 16384, [16384, 16384]),
+    (256, 400.0, [(0.0, 0.5, 800, 1), (400.0, 1.0, 400, 2)], 16384, [16384, 16000]),
+    (64, 100.0, [(0.0, 1.0, 401, 1)], 65536, [65536])])
+def test_staged_copies_stay_inside_the_ring(nchans, bw, ranges, chunk, sizes):
+    bad, oks = _staged(nchans, bw, ranges, chunk, sizes)
+    assert all(oks)
+    assert bad == 0
+
+
+def test_staged_plan_refusals():
+    assert _staged(64, 400.0, [(0.0, 1.8, 65, 1)], 8192, [8192]) == (0, [0])  # spread too wide
+    (tab,) = _tables(configs.tiny())
+    tab = tab.copy()
+    tab[10, 5] = tab[0, 5] - 1  # a delay below the tile's first
+    assert dd.dd_staged_plan_check(tab, 1, 2048, 8192, 0, 8192) == (0, 0)
+    for args in ((3, 0, 8192, 0, 8192), (1, -1, 8192, 0, 8192), (1, 0, 8192, 0, 8193)):
+        with pytest.raises(dd.DDError):
+            dd.dd_staged_plan_check(tab, *args)
