@@ -515,6 +515,7 @@ constexpr int kSpsThreads = 256;
 constexpr int kSpsWarps = kSpsThreads / 32;
 constexpr int kSpsPass = 512;                     // window samples per warp and pass
 constexpr int kSpsPad = 3;                        // aligns P[1 + hist + 4k] to 16 bytes
+constexpr int kMaxHist = 1024;                    // widths up to 1024, rounded up to 256
 
 // Exact argmax over the block of B lanes: the largest v among its valid lanes and its lowest lane
 // (`off`, within the block); false when the block has no valid lane.
@@ -1194,28 +1195,35 @@ __global__ void __launch_bounds__(kSpsThreads, 3) k_clip_stats(const ClipArgs a)
   if (tid < nw) a.out[(int64_t)i * nw + tid] = st[tid];
 }
 
+// Dynamic shared memory of k_clip_stats: a prefix-sum row and the lanes' sums per warp.
+static size_t clip_smem(int nw, int hist) {
+  return (sizeof(uint32_t) * (size_t)sps_row_words(hist) +
+          32 * (size_t)nw * (sizeof(ClipSum) + 2 * sizeof(uint32_t))) *
+         kSpsWarps;
+}
+
 cudaError_t launch_clip_stats(const ClipArgs& a, cudaStream_t st) {
   if (a.n <= 0 || a.n_trials <= 0 || a.nw <= 0) return cudaSuccess;
-  if (a.hist < 0 || a.hist % 256 || a.hist > 1024 || a.iters < 0 || !(a.kappa > 0))
+  if (a.nw > kMaxWidths || a.hist < 0 || a.hist % 256 || a.hist > kMaxHist || a.iters < 0 ||
+      !(a.kappa > 0))
     return cudaErrorInvalidValue;
-  const size_t smem = (sizeof(uint32_t) * (size_t)sps_row_words(a.hist) +
-                       32 * (size_t)a.nw * (sizeof(ClipSum) + 2 * sizeof(uint32_t))) *
-                      kSpsWarps;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_clip_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  // The limit is state of the function on the device, shared by every plan and host thread: always
+  // the largest a launch can need, so that no thread lowers it between another's set and launch.
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_clip_stats, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)clip_smem(kMaxWidths, kMaxHist));
+  if (e != cudaSuccess) return e;
+  const size_t smem = clip_smem(a.nw, a.hist);
   k_clip_stats<<<a.n_trials, kSpsThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sps(const SpsArgs& a, cudaStream_t st) {
   if (a.n <= 0 || a.n_trials <= 0 || a.nw <= 0) return cudaSuccess;
-  if (a.hist < 0 || a.hist % 256 || a.hist > 1024 || a.block < 1 || a.block > 32)
+  if (a.hist < 0 || a.hist % 256 || a.hist > kMaxHist || a.block < 1 || a.block > 32)
     return cudaErrorInvalidValue;
   const size_t smem = sizeof(uint32_t) * (size_t)sps_row_words(a.hist) * kSpsWarps;
-  if (smem > 48 * 1024) {
+  if (smem > 48 * 1024) {  // the largest history only: the limit set is always the same
     const cudaError_t e =
         cudaFuncSetAttribute(k_sps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

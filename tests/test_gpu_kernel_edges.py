@@ -2,6 +2,8 @@
 clipped statistics at the edges of a warp's passes and segments, the corner turn of spectra that
 start at any byte, the staged direct kernel with and without a split of the channels, and the
 128-trial tile. Series, moments and statistics are whole numbers and are compared exactly."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -233,3 +235,51 @@ def test_fused_blocks_equal_plain(block, widths):
     assert got[0].size == got[1].size > 1000
     for f in ("range", "trial", "t_start", "width", "snr"):
         np.testing.assert_array_equal(got[0][f], got[1][f], err_msg=f)
+
+
+def _both(*calls):
+    """Run the calls on host threads at once; the first exception of any is raised here."""
+    errors = []
+
+    def guarded(f):
+        try:
+            f()
+        except Exception as e:  # noqa: BLE001 - handed to the test's thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=guarded, args=(f,)) for f in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def test_clipped_searches_on_two_threads():
+    """Two plans on two host threads, whose clipped statistics need 147 KB and 67 KB of shared
+    memory: neither thread's launches fail for the other's, and every pass gives the same
+    candidates."""
+    x = torch.randint(96, 160, (256, 8), dtype=torch.uint8, device="cuda",
+                      generator=torch.Generator("cuda").manual_seed(78))
+    x[100:104] = 255
+    torch.cuda.synchronize()
+    f = 1500.0 - np.arange(8.0)
+
+    def loop(widths):
+        plan = dd.Plan(f, 64e-6, [(0.0, 1.0, 1, 1)] * 8, 256, n_streams=1, max_width=1024)
+        try:  # eight launches a pass
+            first = None
+            for _ in range(800):
+                seq = plan.run(x, 256)
+                plan.search(widths, 4.0, estimator=dd.DD_EST_CLIPPED)
+                got = plan.candidates(seq)
+                got["t_start"] -= 256 * seq
+                first = got if first is None else first
+                np.testing.assert_array_equal(got, first)
+            assert first.size > 0
+        finally:
+            plan.close()
+
+    _both(lambda: loop((1, 2, 4, 7, 12, 24, 48, 96, 100, 128, 200, 256, 500, 512, 1000, 1024)),
+          lambda: loop((1, 2, 4, 8, 16, 32, 64)))
