@@ -1810,11 +1810,14 @@ int64_t tiled_plan_check(const int32_t* tab, int ntr, int cpad, int decimation, 
 cudaError_t launch_tiled_persistent(const PersistArgs& p, int is_u16, int tt, int nstage, int D,
                                     int nt, size_t smem, int ctas, cudaStream_t st) {
   if (p.nseg <= 0 || ctas <= 0) return cudaSuccess;
+  if (smem > kSmemLimit) return cudaErrorInvalidValue;
+  // The limit set is the largest any plan may need, not this launch's: it is state of the function
+  // on the device, and another host thread's batch must not find it lowered.
 #define DD_PERSIST(T, U16, TT, NS, DT, NTH)                                     \
   if (is_u16 == U16 && tt == TT && nstage == NS && D == DT && nt == NTH) {       \
     cudaError_t e = cudaFuncSetAttribute(k_dedisp_persistent<T, TT, NS, DT, NTH>, \
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                         (int)smem);                            \
+                                         (int)kSmemLimit);                      \
     if (e != cudaSuccess) return e;                                             \
     k_dedisp_persistent<T, TT, NS, DT, NTH><<<ctas, NTH, smem, st>>>(p);        \
     return cudaGetLastError();                                                  \

@@ -283,3 +283,24 @@ def test_clipped_searches_on_two_threads():
 
     _both(lambda: loop((1, 2, 4, 7, 12, 24, 48, 96, 100, 128, 200, 256, 500, 512, 1000, 1024)),
           lambda: loop((1, 2, 4, 8, 16, 32, 64)))
+
+
+def test_persistent_batches_on_two_threads():
+    """Two persistent batches on two host threads whose tiles need different amounts of shared
+    memory: neither thread's launches fail for the other's."""
+    f = 1550.0 - np.arange(256) * 300.0 / 4096
+    x = torch.randint(96, 160, (1 << 15, 256), dtype=torch.uint8, device="cuda",
+                      generator=torch.Generator("cuda").manual_seed(79))
+    torch.cuda.synchronize()
+
+    def loop(step):
+        b = dd.Batch([(f, 64e-6, x)], [(0.0, step, 64, 1)], 2048, (1, 2, 4), 9.0, persistent=True)
+        try:
+            assert b.info(0)[2] == 512  # the tiled kernel, one instance for both
+            for _ in range(2000):  # sixteen rounds, a launch each
+                b.run()
+                b.wait()
+        finally:
+            b.close()
+
+    _both(lambda: loop(0.02), lambda: loop(0.6))
