@@ -89,6 +89,19 @@ def check(w, x, chunk_sizes, n_streams, kind="device", trials=None, flags=0, blo
     return nmatch
 
 
+def staged_takes(w, chunk_len):
+    """Whether the staged direct kernel takes each range of w (of those the tiled kernel refuses)."""
+    tabs = oracle.shift_tables(w.freqs(), w.tsamp, w.ranges_array())
+    O = oracle.overlap(tabs, w.ranges_array())
+    out = []
+    for t, r in zip(tabs, w.ranges):
+        t = np.pad(t, ((0, 0), (0, -t.shape[1] % 8)), mode="edge").astype(np.int32)
+        ok, bad = dd.dd_staged_plan_check(t, r.decimation, O, chunk_len, 0, chunk_len)
+        assert bad == 0
+        out.append(ok)
+    return out
+
+
 def oracle_candidates_match(w, x, chunk_sizes, got_per_chunk, block=32):
     """Run the oracle over the chunks and compare each chunk's candidates (sorted by the library:
     range, trial, t_start, width) with it, per block (tests/_parity.py). Returns the number of

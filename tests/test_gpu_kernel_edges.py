@@ -13,7 +13,7 @@ from _parity import clipped_trial_snr, compare_candidates
 
 torch = pytest.importorskip("torch")
 import paper_2101_00941_gb300 as dd  # noqa: E402
-from _gpu_check import _arrivals, check  # noqa: E402
+from _gpu_check import _arrivals, check, staged_takes  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -151,19 +151,6 @@ def test_staged_direct_kernel(nchans, trials, sizes):
     check(w, x[:sum(sizes)], sizes, 1)
 
 
-def _staged_takes(w, chunk_len):
-    """Whether the staged direct kernel takes each range of w (of those the tiled kernel refuses)."""
-    tabs = oracle.shift_tables(w.freqs(), w.tsamp, w.ranges_array())
-    O = oracle.overlap(tabs, w.ranges_array())
-    out = []
-    for t, r in zip(tabs, w.ranges):
-        t = np.pad(t, ((0, 0), (0, -t.shape[1] % 8)), mode="edge").astype(np.int32)
-        ok, bad = dd.dd_staged_plan_check(t, r.decimation, O, chunk_len, 0, chunk_len)
-        assert bad == 0
-        out.append(ok)
-    return out
-
-
 @pytest.mark.parametrize("ranges,sizes", [
     (((0.0, 1.4, 65, 1),), [8448, 8448, 300]),
     (((0.0, 2.4, 65, 2), (0.0, 1.2, 65, 1)), [8448, 8446, 258])])
@@ -173,7 +160,7 @@ def test_staged_kernel_widest_rows(ranges, sizes):
     w = _coarse(tuple(configs.DMRange(*r) for r in ranges), 64, 1 << 15, 77, bw=400.0)
     w.fch1, w.widths = 1500.0, (2, 4, 64, 256)
     x = w.generate(_arrivals(w))
-    assert _staged_takes(w, 8448) == [1] * len(ranges)
+    assert staged_takes(w, 8448) == [1] * len(ranges)
     plan = dd.Plan(w.freqs(), w.tsamp, w.ranges_array(), 8448, n_streams=1, max_width=256)
     try:
         for r in range(len(ranges)):

@@ -22,7 +22,7 @@ from synth import configs
 
 torch = pytest.importorskip("torch")
 import paper_2101_00941_gb300 as dd  # noqa: E402
-from _gpu_check import check, run_gpu  # noqa: E402
+from _gpu_check import check, run_gpu, staged_takes  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -115,6 +115,27 @@ def test_direct_kernel_swar_flush(fill):
     sizes = [8192] * 3
     assert O < 8192
     check(w, x[:sum(sizes)], sizes, 2)
+
+
+@pytest.mark.parametrize("nchans,foff,ranges,sizes", [
+    (600, -1.0, ((0.0, 3.0, 20, 1), (0.0, 6.0, 40, 2)), [16384, 14654, 4258]),
+    (41, -30.0, ((0.0, 7.0, 21, 32), (0.0, 0.2, 33, 1)), [81920, 80192, 4256])])
+@pytest.mark.parametrize("fill", ["saturated", "uniform"])
+def test_cached_read_kernel_flush_and_uint16(nchans, foff, ranges, sizes, fill):
+    """Delays that spread too far over a trial tile for the staged kernel's shared memory, so that
+    the ranges run on the cached-read direct kernel: 256 x 255 = 65,280 in a 16-bit SWAR lane
+    before each 256-channel flush (x1: two flushes and a ragged third), its three-word loads of
+    uint16 data (x2 at every second alignment, x32 up to 255 x 32), an odd trial at the end of its
+    pairs."""
+    w = _workload(nchans, 1530.0, foff, 64e-6, tuple(configs.DMRange(*r) for r in ranges),
+                  (1, 2, 32, 64), sum(sizes))
+    chunk = sizes[0]
+    kinds, O = _kernels(w, chunk_len=chunk)
+    assert [k for k, _ in kinds] == [dd.DD_KERNEL_DIRECT] * 2
+    assert staged_takes(w, chunk) == [0, 0]
+    assert O < chunk
+    x = _saturated(w.nsamp, nchans) if fill == "saturated" else _uniform(w.nsamp, nchans, 6)
+    check(w, x, sizes, 2)
 
 
 # ---------------------------------------------------------------- search: sums just under 2^31
