@@ -50,14 +50,16 @@ extern "C" {
 #define DD_FLAG_NAIVE 2u    /* use the one-thread-per-output dedispersion kernel (testing aid) */
 #define DD_FLAG_DEVICE_INPUT 4u /* chunks are always in device memory: no staging buffer is
                                    allocated and host chunks are refused (DD_ERR_ARG) */
-#define DD_FLAG_TILE256 8u  /* plan the tiled kernel with 256-sample time tiles only (testing
-                               aid; 512-sample tiles are tried first otherwise) */
-#define DD_FLAG_TRIALS32 16u /* plan the tiled kernel with 32-trial tiles only (testing aid;
-                                64-trial tiles are tried first otherwise) */
+/* Without a flag, dd_plan takes per range the tiled kernel's 64-trial x 512-sample or 128 x 256
+ * tile by the launch's estimated work, and smaller tiles where neither fits. */
+#define DD_FLAG_TILE256 8u  /* plan the tiled kernel with 64- or 32-trial x 256-sample tiles only
+                               (testing aid) */
+#define DD_FLAG_TRIALS32 16u /* plan the tiled kernel with 32-trial tiles only (testing aid) */
 #define DD_FLAG_AUTOTUNE 32u /* dd_plan times every tile shape that fits each range (trials x
-                                outputs x threads: 64 x 512 x 512, 64 x 512 x 1024, 64 x 256 x
-                                512, 32 x 256 x 512) on the plan's own buffers and keeps the
-                                fastest (adds a few launches per range to planning) */
+                                outputs x threads: 64 x 512 x 512, 128 x 256 x 512, 64 x 512 x
+                                1024, 64 x 256 x 512, 32 x 256 x 512) on the plan's own buffers
+                                and keeps the fastest (adds a few launches per range to
+                                planning) */
 #define DD_FLAG_WARPS32 64u /* plan the tiled kernel with 1024-thread CTAs only (testing aid) */
 
 typedef struct dd_plan_s* dd_plan_t;
@@ -142,7 +144,7 @@ int dd_plan_kernel(dd_plan_t plan, int32_t range, int32_t* kind, int32_t* tile_s
  * dd_plan_model -- the work of one dedispersion launch of range `range` over a window of `nout`
  * outputs, counted on the host (no GPU work); it is what roofline fractions divide by.
  *   kind, tile_samples : as dd_plan_kernel
- *   tile_trials        : trials per tile of the tiled kernel (64 or 32), else 0
+ *   tile_trials        : trials per tile of the tiled kernel (128, 64 or 32), else 0
  *   cta_threads        : threads per CTA of the tiled kernel (512 or 1024), else 0
  *   ctas_per_sm        : CTAs of the tiled kernel's tile shape per SM (1 or 2), else 0
  *   outputs            : DM-trial*samples, n_trials * nout
@@ -300,6 +302,8 @@ int sps_run_ex(dd_plan_t plan, const int32_t* widths, int32_t nwidths, float thr
  *   out    : caller-owned host array of cap entries, sorted by (range, trial, t_start, width)
  *   ncands : receives the number of candidates found
  *   timeout_ms : bound on the wait (<= 0: 600000)
+ * The wait polls: without sleeping for its first millisecond (the calling thread keeps a core busy,
+ * yielding between polls), then with 20 us sleeps.
  * Errors: DD_ERR_STATE (unknown, recycled or unsearched chunk), DD_ERR_TIMEOUT (the wait ran
  * out, or a dedispersion kernel of this chunk ran out of its bounded device-side wait, so the
  * chunk's results are not valid; later chunks are not affected), DD_ERR_CAP (more than cap or

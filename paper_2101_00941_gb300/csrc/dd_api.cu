@@ -65,7 +65,8 @@ int ilog2(int64_t v) {
 
 // Bounded wait on an event (no spin on the GPU side; host polls with a deadline). The first
 // kSpinUs are polled without sleeping: a 20 us sleep returns after 70 to 80 us with the default
-// timer slack, as long as a small chunk's own work; after that the thread sleeps between polls.
+// timer slack, as long as a small chunk's own work; after that the thread sleeps between polls. A
+// thread that collects keeps a core busy for that first millisecond (it yields between polls).
 constexpr int64_t kSpinUs = 1000;
 
 int wait_event(cudaEvent_t ev, int64_t timeout_ms) {
@@ -1062,9 +1063,9 @@ int dd_fuse_search(dd_plan_t p, const int32_t* widths, int32_t nwidths, uint32_t
   return DD_OK;
 }
 
-// dd_run's work; with `defer`, the tiled launches of the 64 x 512 x 512 shape are not made but
-// handed back (argument block and instance) for a persistent launch the caller makes later on
-// the same stream.
+// dd_run's work; with `defer`, the tiled launches of the 64 x 512 and 128 x 256 tiles with 512
+// threads are not made but handed back (argument block and instance) for a persistent launch the
+// caller makes later on the same stream.
 static int run_impl(dd_plan_t p, const uint8_t* chunk, int64_t nsamp, void* cuda_stream,
                     std::vector<ddk::DeferredTile>* defer) {
   if (!p) return fail(DD_ERR_ARG, "plan is NULL");

@@ -7,7 +7,8 @@
 // per thread, 64 accumulators per lane), 64 x 512 with 32 warps (64 registers, 32 accumulators:
 // twice the warps on the same tables and shared memory), and 64 x 256 or 32 x 256 with 16 warps,
 // two CTAs per SM. Bound by the shared-memory pipe (71% busy) and instruction issue (58%): 1216
-// trials x 65536 outputs x 4096 channels take 6.2 ms (uint8; 8.5 without the class chains).
+// trials x 65536 outputs x 4096 channels take 6.3 ms (uint8; 8.5 before the class chains, the
+// packed sums, the 128-trial tile and leaner stages, 6.8 with the first two of them alone).
 //
 //   * Delay classes. For an 8-channel group the tile's trials fall into a few classes by the
 //     relative delays (r0..r7) of the eight channels. A class shares one sequence of sums
@@ -875,8 +876,8 @@ __device__ __forceinline__ bool tile_body(const TiledArgs& a, int bx, int by,
     // (2) pair words of stage s + 1, and
     // (3) accumulation of stage s: lane l of the warp reads, for each of its trials, pair word
     //     l + 32k of the trial's plane in both groups (outputs 2(l + 32k) and 2(l + 32k) + 1).
-    // Half of each scheduler's warps take (3) first: the build is bound by instruction issue, the
-    // accumulation by the shared-memory pipe.
+    // Every warp builds first: with every second warp accumulating first, so that the two phases'
+    // pipes overlap, the launch above took 7.40 ms against 6.38.
     if (ok && s + 1 < nstages) build_stage<T>(tnext, rnext, znext, pos, warp, lane);
     {
       const uint32_t zs = zcur + 4u * lane, tc = tcur + zrow;

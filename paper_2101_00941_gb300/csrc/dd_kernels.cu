@@ -666,7 +666,7 @@ struct SpsRow {
     for (int q = 0; q < H; q += 128) {
       const uint4 t = *reinterpret_cast<const uint4*>(P + 1 + kSpsPass + q + 4 * lane);
       *reinterpret_cast<uint4*>(P + 1 + q + 4 * lane) = t;
-      __syncwarp();  // at H > 512 a later read lies where an earlier write went
+      __syncwarp();  // at H > 512 a later write lands where an earlier read came from
     }
     __syncwarp();
   }
@@ -677,13 +677,14 @@ __host__ __device__ constexpr int sps_row_words(int hist) { return kSpsPad + 1 +
 // Samples of a warp's segment: 8 passes (their history re-read is 6% at H = 256), 16 with wide
 // boxcars (H >= 512), fewer while the launch has less than 24 warps per SM and a segment stays
 // at least four times its history.
+constexpr int kSegSms = 152;  // a GB300's SMs; only the split depends on it, no result
 inline int64_t sps_segment(int n_trials, int64_t n, int hist) {
   int64_t seg = kSpsPass * (hist >= 512 ? 16 : 8);
   while (seg > 2 * kSpsPass && seg / 2 >= 4 * hist &&
-         n_trials * ((n + seg - 1) / seg) < 152 * 24)
+         n_trials * ((n + seg - 1) / seg) < kSegSms * 24)
     seg /= 2;
   // a chip nearly idle: single passes, so that a bright pulse's groups spread over more warps
-  while (seg > kSpsPass && n_trials * ((n + seg - 1) / seg) < 152 * 4) seg /= 2;
+  while (seg > kSpsPass && n_trials * ((n + seg - 1) / seg) < kSegSms * 4) seg /= 2;
   while ((n + seg * kSpsWarps - 1) / (seg * kSpsWarps) > 65535) seg *= 2;  // grid rows
   return seg;
 }
